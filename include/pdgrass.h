@@ -61,6 +61,8 @@ extern "C" {
 
 typedef struct pdg_options {
   int32_t score_mode;       /* PDG_SCORE_STRETCH or PDG_SCORE_RESISTANCE */
+  /* The greedy runs as one join over cells of the tree for all subtasks together; the tiers that the next
+     options shape decide only candidate sets whose cells are too full for it. */
   int32_t warp_tier_max;    /* subtasks with 2..warp_tier_max candidates get one warp each (<= 32) */
   int64_t k_override;       /* >= 0: use this budget instead of floor(alpha*|V|) */
   double candidate_factor;  /* first candidate prefix holds about factor*k edges (>= 1) */
@@ -196,12 +198,14 @@ int pdg_handle_info(pdg_handle h, int64_t* n, int64_t* m, int64_t* n_offtree, in
 /*
  * pdg_last_stats -- counters of the last recovery: candidates examined (the
  * prefix of the global order that was scored into subtasks), subtasks,
- * largest subtask, candidates in the warp tier / cooperative tier, rounds of
- * the cooperative tier, prefix retries, attempts, kernels launched by the
- * recovery, cooperative-tier candidates that showed an earlier registrant of
- * one of their pairs ("constrained"), ancestor pairs registered by the
- * cooperative tier, and the site of a failed internal index check (0 if none;
- * such a recovery returns PDG_E_CUDA).  stats must hold 12 int64.
+ * largest subtask, candidates alone in their subtask (tiers: in the warp or
+ * block tier too) / in subtasks of several (tiers: in the cooperative tier),
+ * rounds (the join: 1; tiers: rounds of the cooperative tier), prefix retries,
+ * attempts, kernels launched by the recovery, candidates that an earlier one
+ * may mark ("constrained"; the join: does mark), cell entries (tiers: ancestor
+ * pairs registered by the cooperative tier), and the site of a failed internal
+ * index check (0 if none; such a recovery returns PDG_E_CUDA).  stats must
+ * hold 12 int64.
  */
 int pdg_last_stats(pdg_handle h, int64_t* stats);
 

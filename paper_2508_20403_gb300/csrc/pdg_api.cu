@@ -123,8 +123,17 @@ __global__ void k_reset_recover(DevScalars* dsc) {
   dsc->score_ticket = 0;
 }
 
-__global__ void k_reset_attempt(DevScalars* dsc) {
+// The attempt's scalars, the join's cell table emptied (the slots; the members
+// behind them need no clearing), and its candidates per LCA set to zero.
+__global__ void k_reset_attempt(DevScalars* dsc, uint4* __restrict__ tab, int64_t slots, uint4* __restrict__ lca_count,
+                                int64_t counts) {
   dep_sync();
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < slots; i += (int64_t)gridDim.x * blockDim.x)
+    tab[i] = make_uint4(~0u, ~0u, 0u, 0u);  // key, count
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < counts; i += (int64_t)gridDim.x * blockDim.x)
+    lca_count[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (blockIdx.x != 0 || threadIdx.x != 0) return;
+  dsc->join_conf = 0;
   dsc->err &= ERR_RANGE | ERR_TIMEOUT | ERR_BOUNDS;  // errors of steps A1-A3 end the recovery
   dsc->epoch++;
   dsc->bounds_site = 0;
@@ -188,37 +197,77 @@ int ensure_scan_status(Handle& h, int64_t n_max) {
   return PDG_OK;
 }
 
+static int ensure_tiers(Handle& h, int c);
+
 int ensure_candidates(Handle& h, int64_t R, int c) {
   const int64_t Rmax = std::max<int64_t>(h.E_off, 1);
   R = std::min<int64_t>(std::max<int64_t>(R, 1), Rmax);
   int st;
   if (R > h.Rcap) {
-    void* old[] = {h.cand_idx, h.rk[0], h.rk[1], h.rv[0], h.rv[1], h.rank_cand, h.lsort_rank, h.scan_tmp,
-                   h.radix_status, h.rec_u, h.rec_v, h.rec_anc, h.rec_du, h.rec_dv, h.rec_rank,
-                   h.rec_lca, h.rec_b, h.state, h.acc_flag, h.seg_begin, h.warp_seg, h.block_seg, h.big_pos, h.big_seg, h.big_chunk,
-                   h.pos_x, h.seg_regs, h.seg_pref,
-                   h.pmask, h.reg_slot, h.pslot, h.und_list};
+    void* old[] = {h.cand_idx, h.rk[0], h.rk[1], h.rv[0], h.rv[1], h.rank_cand, h.scan_tmp,
+                   h.radix_status, h.acc_flag, h.cand_rec, h.join_rec, h.join_probe, h.join_conf, h.join_list};
     for (void* p : old) device_release(h, p);
     const int64_t tiles = (R + kTile - 1) / kTile;
+    const int64_t join_list = std::min<int64_t>(kJoinListPer * R, INT32_MAX);  // runs start at 32-bit offsets
     if ((st = alloc_n(h, &h.cand_idx, R)) || (st = alloc_n(h, &h.rk[0], R)) || (st = alloc_n(h, &h.rk[1], R)) ||
         (st = alloc_n(h, &h.rv[0], R)) || (st = alloc_n(h, &h.rv[1], R)) || (st = alloc_n(h, &h.rank_cand, R)) ||
-        (st = alloc_n(h, &h.lsort_rank, R)) || (st = alloc_n(h, &h.scan_tmp, R + 1)) ||
+        (st = alloc_n(h, &h.scan_tmp, R + 1)) ||
         (st = alloc_n(h, &h.radix_status, (int64_t)kRadixPassesMax * 256 * tiles)) ||
-        (st = alloc_n(h, &h.rec_u, R)) ||
-        (st = alloc_n(h, &h.rec_v, R)) || (st = alloc_n(h, &h.rec_anc, 2 * PDG_MAX_C * R)) ||
-        (st = alloc_n(h, &h.rec_du, R)) || (st = alloc_n(h, &h.rec_dv, R)) || (st = alloc_n(h, &h.rec_rank, R)) ||
-        (st = alloc_n(h, &h.rec_lca, R)) || (st = alloc_n(h, &h.rec_b, R)) || (st = alloc_n(h, &h.state, R)) ||
-        (st = alloc_n(h, &h.acc_flag, R)) || (st = alloc_n(h, &h.seg_begin, R + 1)) ||
-        (st = alloc_n(h, &h.warp_seg, R)) || (st = alloc_n(h, &h.block_seg, R)) || (st = alloc_n(h, &h.big_pos, R)) || (st = alloc_n(h, &h.big_seg, R)) || (st = alloc_n(h, &h.big_chunk, R)) ||
-        (st = alloc_n(h, &h.pos_x, R)) || (st = alloc_n(h, &h.seg_regs, R)) || (st = alloc_n(h, &h.seg_pref, R + 1)) ||
-        (st = alloc_n(h, &h.pmask, R)) || (st = alloc_n(h, &h.reg_slot, 16 * R)) || (st = alloc_n(h, &h.und_list, R)) ||
-        (st = alloc_n(h, &h.pslot, 32 * R))) {
+        (st = alloc_n(h, &h.acc_flag, R)) || (st = device_alloc(h, &h.cand_rec, (size_t)32 * R)) ||
+        (st = device_alloc(h, &h.join_rec, (size_t)32 * R)) ||
+        (st = device_alloc(h, &h.join_probe, (size_t)32 * R)) || (st = alloc_n(h, &h.join_conf, 8 * R)) ||
+        (st = alloc_n(h, &h.join_list, join_list))) {
       h.Rcap = 0;
       return st;
     }
     h.Rcap = R;
+    h.join_slots = 0;
+    h.join_list_cap = join_list;
+    if ((st = grow_join(h))) return st;
   }
   if ((st = ensure_scan_status(h, h.Rcap + 1))) return st;
+  return h.tiered ? ensure_tiers(h, c) : PDG_OK;
+}
+
+// the join's cell table: join_factor slots per candidate of the capacity
+int grow_join(Handle& h) {
+  device_release(h, h.join_tab);
+  h.join_tab = nullptr;
+  h.join_slots = 0;
+  device_release(h, h.join_ranks);
+  h.join_ranks = nullptr;
+  const int64_t slots = std::min<int64_t>(h.join_factor * h.Rcap + 1024, (1ll << 32) - 16) / 16 * 16;
+  int st;
+  if ((st = device_alloc(h, &h.join_tab, (size_t)slots * kJoinSlotBytes)) ||
+      (st = alloc_n(h, &h.join_ranks, slots * kJoinInline)))
+    return st;
+  h.join_slots = slots;
+  return PDG_OK;
+}
+
+// the tiers' buffers for Rcap candidates, and their pair table
+static int ensure_tiers(Handle& h, int c) {
+  const int64_t R = h.Rcap;
+  int st;
+  if (R > h.tier_cap) {
+    void* old[] = {h.lsort_rank, h.rec_u, h.rec_v, h.rec_anc, h.rec_du, h.rec_dv, h.rec_rank, h.rec_lca, h.rec_b, h.state,
+                   h.seg_begin, h.warp_seg, h.block_seg, h.big_pos, h.big_seg, h.big_chunk, h.pos_x, h.seg_regs,
+                   h.seg_pref, h.pmask, h.reg_slot, h.pslot, h.und_list};
+    for (void* p : old) device_release(h, p);
+    if ((st = alloc_n(h, &h.lsort_rank, R)) || (st = alloc_n(h, &h.rec_u, R)) ||
+        (st = alloc_n(h, &h.rec_v, R)) || (st = alloc_n(h, &h.rec_anc, 2 * PDG_MAX_C * R)) ||
+        (st = alloc_n(h, &h.rec_du, R)) || (st = alloc_n(h, &h.rec_dv, R)) || (st = alloc_n(h, &h.rec_rank, R)) ||
+        (st = alloc_n(h, &h.rec_lca, R)) || (st = alloc_n(h, &h.rec_b, R)) || (st = alloc_n(h, &h.state, R)) ||
+        (st = alloc_n(h, &h.seg_begin, R + 1)) ||
+        (st = alloc_n(h, &h.warp_seg, R)) || (st = alloc_n(h, &h.block_seg, R)) || (st = alloc_n(h, &h.big_pos, R)) || (st = alloc_n(h, &h.big_seg, R)) || (st = alloc_n(h, &h.big_chunk, R)) ||
+        (st = alloc_n(h, &h.pos_x, R)) || (st = alloc_n(h, &h.seg_regs, R)) || (st = alloc_n(h, &h.seg_pref, R + 1)) ||
+        (st = alloc_n(h, &h.pmask, R)) || (st = alloc_n(h, &h.reg_slot, 16 * R)) || (st = alloc_n(h, &h.und_list, R)) ||
+        (st = alloc_n(h, &h.pslot, 32 * R))) {
+      h.tier_cap = 0;
+      return st;
+    }
+    h.tier_cap = R;
+  }
   // pair table: twice the registrations plus 16 slots per cooperative subtask (at most R / 33 subtasks)
   return grow_tables(h, std::max<int64_t>(1024, 2 * (int64_t)(c + 1) * (c + 1) * h.Rcap + h.Rcap), 0);
 }
@@ -470,6 +519,8 @@ int sparsify_batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_
       (st = alloc_n(h, &h.hist, (int64_t)num_graphs * kSelBins)) || (st = alloc_n(h, &h.sel, num_graphs)) ||
       (st = alloc_n(h, &h.d_cand_ptr, num_graphs + 1)) || (st = alloc_n(h, &h.d_graph_tmp, num_graphs + 1)) ||
       (st = alloc_n(h, &h.gstat, num_graphs)) || (st = alloc_n(h, &h.gcount, num_graphs)) ||
+      (st = alloc_n(h, &h.lca_count, n)) ||
+      (st = device_alloc(h, &h.join_part, (size_t)h.num_sms * 8 * (sizeof(int4) + sizeof(int32_t)))) ||
       (st = alloc_n(h, &h.d_k, num_graphs)) || (st = alloc_n(h, &h.d_out_ptr, num_graphs + 1)) ||
       (st = alloc_n(h, &h.radix_dtot, 256)) || (st = alloc_n(h, &h.radix_hist, kRadixHistWords)) ||
       (st = alloc_n(h, &h.radix_counters, 2 * kRadixPassesMax)) ||
@@ -758,6 +809,8 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
     dev_ids = h.out_ids;
     dev_scores = out_scores ? h.out_scores : nullptr;
   }
+  // the tiers only where a recovery of the same kind needed them
+  if (!(h.c_mem == c && h.mode_mem == h.opt.score_mode)) h.tiered = false;
   h.launches = 0;
   DepScope dep_scope(h);  // kernels of the recovery may launch as programmatic dependents
   const bool prof = h.opt.profile != 0;
@@ -793,7 +846,10 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
       mark(3);
     }
     ++h.launches;
-    launch_k(h, k_reset_attempt, 1, 1, 0, h.dsc);
+    const int64_t clear = h.tiered ? 0 : h.join_slots;
+    const int64_t counts = h.tiered ? 0 : (h.n + 3) / 4;
+    launch_k(h, k_reset_attempt, grid_for(h, clear + counts), kBlock, 0, h.dsc, static_cast<uint4*>(h.join_tab), clear,
+             reinterpret_cast<uint4*>(h.lca_count), counts);
     PDG_CUDA(cudaMemcpyAsync(h.sel, s.sel, sizeof(GraphSel) * G, cudaMemcpyHostToDevice, h.stream));
     stream_op(h);
     mark(4);
@@ -801,7 +857,7 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
     mark(5);
     if ((e = step_sort(h))) return e;
     mark(6);
-    if ((e = step_accept(h, c))) return e;
+    if ((e = h.tiered ? step_accept(h, c) : step_join(h, c))) return e;
     mark(7);
     if ((e = step_budget(h, dev_ids, dev_scores))) return e;
     mark(8);
@@ -837,8 +893,8 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
     any_select_cur = any_select;
     if ((st = ensure_candidates(h, std::max<int64_t>(h.Rcap, need + need / 4 + 4096), c))) return st;
     // the launch sequence a CUDA graph bakes in
-    const GraphKey key{c, h.opt.score_mode, any_select ? 1 : 0, coop_rounds(h, c), h.Rcap, h.table_cap, h.xcap,
-                       (void*)dev_ids, (void*)dev_scores, out_total};
+    const GraphKey key{c, h.opt.score_mode, any_select ? 1 : 0, h.tiered ? coop_rounds(h, c) : 0, h.Rcap, h.table_cap, h.xcap,
+                       h.join_slots, h.tiered, (void*)dev_ids, (void*)dev_scores, out_total};
     bool replayed = false;
     if (first && h.opt.use_graph && h.gexec && key == h.gkey) {
       // replay on the private stream, ordered after the caller's stream
@@ -864,11 +920,23 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
     const int err = h.hsc->err;
     if (getenv("PDG_DEBUG_ATTEMPTS"))
       fprintf(stderr, "pdgrass: attempt %d err %d n_cand %lld n_big %lld n_big_seg %lld big_regs %lld table_cap %lld "
-                      "xcap %lld Rcap %lld\n", attempts, err, (long long)h.hsc->n_cand, (long long)h.hsc->n_big,
+                      "xcap %lld Rcap %lld tiered %d conf spill %llu slots %lld\n", attempts, err, (long long)h.hsc->n_cand, (long long)h.hsc->n_big,
               (long long)h.hsc->n_big_seg, (long long)h.hsc->big_regs, (long long)h.table_cap, (long long)h.xcap,
-              (long long)h.Rcap);
+              (long long)h.Rcap, (int)h.tiered, h.hsc->join_conf, (long long)h.join_slots);
     if (err & ERR_RANGE) return PDG_E_RANGE;
     if (err & ERR_TIMEOUT) return PDG_E_TIMEOUT;
+    if ((err & ERR_DENSE) && !h.tiered) {  // the cells are too full for the join: the tiers decide these candidates
+      h.tiered = true;
+      if ((st = ensure_candidates(h, h.Rcap, c))) return st;
+      first = false;
+      continue;
+    }
+    if ((err & ERR_TABLE) && !h.tiered) {  // the cells outgrew the table
+      h.join_factor *= 2;
+      if ((st = grow_join(h))) return st;
+      first = false;
+      continue;
+    }
     if (err & ERR_TABLE) {
       // pair table too small for the registrations, or too few exact blocks
       const int64_t slots = std::max<int64_t>(h.table_cap, 2 * h.hsc->big_regs + 16 * h.hsc->n_big_seg + 1024);
@@ -905,7 +973,7 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
       }
       h.c_mem = c;
       h.mode_mem = h.opt.score_mode;
-      h.rounds_mem = h.hsc->rounds_used + (h.hsc->finish_left > 0 ? 1 : 0);
+      h.rounds_mem = h.tiered ? h.hsc->rounds_used + (h.hsc->finish_left > 0 ? 1 : 0) : -1;
       if (first && !replayed && h.opt.use_graph && attempts == 1) {
         // this call needed one attempt: capture it for replay by later calls
         const cudaStream_t user = h.stream;
@@ -922,7 +990,7 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
             h.gexec = nullptr;
             if (cudaGraphInstantiate(&h.gexec, graph, 0) == cudaSuccess) {
               h.gkey = key;
-              h.gkey.rounds = coop_rounds(h, c);  // the capture already used the remembered round count
+              h.gkey.rounds = h.tiered ? coop_rounds(h, c) : 0;  // the capture already used the remembered round count
               h.glaunches = h.launches;
             } else {
               h.gexec = nullptr;
@@ -1045,7 +1113,7 @@ int pdg_edge_endpoints(pdg_handle hp, const int32_t* ids, int64_t count, int32_t
     d_v = tmp + 2 * count;
   }
   ++h.launches;
-  k_reset_attempt<<<1, 1, 0, h.stream>>>(h.dsc);
+  k_reset_attempt<<<1, 1, 0, h.stream>>>(h.dsc, nullptr, 0, nullptr, 0);
   ++h.launches;
   k_endpoints<<<grid_for(h, count), kBlock, 0, h.stream>>>(h.el_u, h.el_v, h.m, h.vtx_of_pre, d_ids, count, d_u,
                                                             d_v, h.dsc);

@@ -31,6 +31,17 @@ constexpr uint64_t kEmptyKey = ~0ull;
 constexpr int kRmqMaxLevels = 6;  // levels of the range-minimum structure (n < 2^30: 30 / 5)
 constexpr int kRmqStMax = 6144;   // level-2 entries up to which levels 2+ are one sparse table (n <= 6.29M)
 
+// The join of steps A5 + A6 walks the members of coarse cells; a cell of
+// kJoinCellMax members, or a block that met more earlier members in the cells
+// it entered than kJoinPairsBase + kJoinPairsPer per registration, sends the
+// attempt to the tiers.
+constexpr int kJoinInline = 8;          // member ranks per slot (one sector)
+constexpr int kJoinSlotBytes = 16;      // a slot of the cell table without its members
+constexpr uint32_t kJoinCellMax = 2048;
+constexpr unsigned long long kJoinPairsBase = 1ull << 16;
+constexpr unsigned long long kJoinPairsPer = 64;
+constexpr int64_t kJoinListPer = 8;  // (marker, candidate) pairs kept per candidate of the capacity
+
 // error bits raised by validation kernels (mapped to a status on the host)
 enum : int {
   ERR_NOT_CSR = 1,
@@ -43,6 +54,7 @@ enum : int {
   ERR_CAPACITY = 128,
   ERR_TABLE = 256,
   ERR_BOUNDS = 512,  // a saved index was out of range (checked and skipped; bounds_site says where)
+  ERR_DENSE = 1024,  // the join's cells are too full: the attempt is repeated with the tiers
 };
 
 // candidate state in the cooperative tier
@@ -56,7 +68,7 @@ enum : int32_t { G_OK = 0, G_UNDER = 1, G_RETRY = 2 };
 // retries with larger tables where that helps).  Kernels that index with
 // data produced earlier in the attempt return at once when one is set, so an
 // attempt cut short never reads half-built structures.
-constexpr int kAbortErr = ERR_TABLE | ERR_TIMEOUT | ERR_BOUNDS;
+constexpr int kAbortErr = ERR_TABLE | ERR_TIMEOUT | ERR_BOUNDS | ERR_DENSE;
 
 struct DevScalars {
   int32_t err;          // ERR_* bits
@@ -88,6 +100,7 @@ struct DevScalars {
   int32_t bounds_site;  // first failed bounds check (see ERR_BOUNDS)
   int32_t bounds_where;  // its round (99: serial finisher)
   int64_t bounds_pos, bounds_val;  // its position and offending value
+  unsigned long long join_conf;   // join: (marker, candidate) pairs found
   int64_t finish_left;  // cooperative tier: candidates the rounds left to the serial finisher
 };
 
@@ -133,13 +146,14 @@ struct GraphSel {
 // reads at replay time (budgets, prefix sizes, output offsets).
 struct GraphKey {
   int c = -1, score_mode = -1, any_select = -1, rounds = -1;
-  int64_t Rcap = -1, table_cap = -1, xcap = -1;
+  int64_t Rcap = -1, table_cap = -1, xcap = -1, join_slots = -1;
+  bool tiered = false;
   void* out_ids = nullptr;
   void* out_scores = nullptr;
   int64_t out_total = -1;
   bool operator==(const GraphKey& o) const {
     return c == o.c && score_mode == o.score_mode && any_select == o.any_select && rounds == o.rounds && Rcap == o.Rcap &&
-           table_cap == o.table_cap && xcap == o.xcap && out_ids == o.out_ids && out_scores == o.out_scores &&
+           table_cap == o.table_cap && xcap == o.xcap && join_slots == o.join_slots && tiered == o.tiered && out_ids == o.out_ids && out_scores == o.out_scores &&
            out_total == o.out_total;
   }
 };
@@ -170,6 +184,7 @@ struct Handle {
   int32_t* tour = nullptr;
   int64_t A = 0;
   int32_t* vtx_of_pre = nullptr;
+  void* up = nullptr;  // int4 per label: parent, grandparent, great-grandparent (-1: none), depth
   int64_t* d_vtx_ptr = nullptr;
   int64_t* d_edge_ptr = nullptr;
   int64_t* d_off_ptr = nullptr;
@@ -222,8 +237,27 @@ struct Handle {
   int64_t* d_cand_ptr = nullptr;  // G+1
   int64_t* d_graph_tmp = nullptr;  // G+1 scratch
 
+  // steps A5 + A6: false: the join; true: the tiers (this attempt's candidates fill the join's cells too much;
+  // remembered for later recoveries with (c_mem, mode_mem))
+  bool tiered = false;
   // candidate buffers (grow-only, capacity Rcap)
   int64_t Rcap = 0;
+  // the join: records and probes by rank, cell table, candidates per LCA
+  void* cand_rec = nullptr;  // candidates in id order, 32 bytes: u, v, LCA, canonical id, score bits
+  void* join_rec = nullptr;
+  void* join_probe = nullptr;
+  void* join_tab = nullptr;
+  uint32_t* join_conf = nullptr;
+  uint32_t* join_list = nullptr;
+  int64_t join_list_cap = 0;
+  uint32_t* join_ranks = nullptr;
+  int64_t join_slots = 0;         // a multiple of 16
+  int64_t join_factor = 3;        // slots per candidate
+  int32_t* lca_count = nullptr;   // [n]
+  void* join_part = nullptr;      // per block: the join's shares of the statistics
+  int join_blocks = 0, join_pair_blocks = 0;
+  // the tiers' buffers below are allocated when a recovery first needs them
+  int64_t tier_cap = 0;
   int32_t* cand_idx = nullptr;     // off-tree index of each candidate (id order within graph)
   uint64_t* rk[2] = {nullptr, nullptr};  // radix keys ping-pong
   int32_t* rv[2] = {nullptr, nullptr};   // radix values ping-pong
@@ -526,10 +560,12 @@ constexpr int64_t kPcgMaxEdges = 8192;  // recovered edges of the PCG quality me
 // z0: nullable, the preconditioner applied to the centred right-hand side, n values)
 int pcg_quality(Handle& h, const int32_t* ids, int64_t k, const double* b, double tol, int32_t max_iter,
                 int32_t* iters, double* relres, double* hist = nullptr, double* z0 = nullptr);
-int step_sort(Handle& h);                       // A4b: (graph, score desc, id asc) then (lca, rank)
-int step_accept(Handle& h, int c);              // A5 + A6
+int step_sort(Handle& h);                       // A4b: (graph, score desc, id asc); for the tiers then (lca, rank)
+int step_join(Handle& h, int c);                // A5 + A6 as a join over tree cells
+int step_accept(Handle& h, int c);              // A5 + A6 by tiers
 int step_budget(Handle& h, int32_t* out_ids, double* out_scores);  // A7
 int ensure_candidates(Handle& h, int64_t R, int c);
+int grow_join(Handle& h);
 int grow_tables(Handle& h, int64_t slots, int64_t xblocks);
 int device_alloc(Handle& h, void** p, size_t bytes);
 

@@ -120,18 +120,6 @@ __global__ void k_lay_pre(const int32_t* __restrict__ tour, const int64_t* __res
   }
 }
 
-// the largest hop depth: after the down arc at tour position p the depth is
-// (down arcs up to p) - (up arcs before p) = 2 dpre[p] + 1 - p (every graph's
-// tour starts after as many down arcs as its offset counts)
-__global__ void k_lay_depth(const int32_t* __restrict__ tour, const int64_t* __restrict__ dpre, int64_t A,
-                            DevScalars* dsc) {
-  long long mx = 0;
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < A; p += (int64_t)gridDim.x * blockDim.x)
-    if (tour[p] >= 0) mx = max(mx, (long long)(2 * dpre[p] + 1 - p));
-  for (int o = 16; o; o >>= 1) mx = max(mx, __shfl_down_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax((long long*)&dsc->max_depth, mx);
-}
-
 __global__ void k_lay_roots(const int32_t* __restrict__ parent, const int64_t* __restrict__ vtx_ptr, int32_t G,
                             int64_t n, int32_t* __restrict__ pre_of) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
@@ -162,8 +150,13 @@ __global__ void k_lay_vertices(const int32_t* __restrict__ pre_of, const int32_t
   }
 }
 
-__global__ void k_lay_tour(int32_t* __restrict__ tour, const int32_t* __restrict__ pre_of, int64_t A, int64_t n,
-                           int32_t* __restrict__ bad) {
+// The tour in labels, and the hop depths: after the down arc at tour position p
+// the depth is (down arcs up to p) - (up arcs before p) = 2 dpre[p] + 1 - p
+// (every graph's tour starts after as many down arcs as its offset counts).
+__global__ void k_lay_tour(int32_t* __restrict__ tour, const int32_t* __restrict__ pre_of,
+                           const int64_t* __restrict__ dpre, int64_t A, int64_t n, int4* __restrict__ up,
+                           DevScalars* dsc, int32_t* __restrict__ bad) {
+  int mx = 0;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < A; p += (int64_t)gridDim.x * blockDim.x) {
     const int32_t y = tour[p];
     const int32_t v = y >= 0 ? y : ~y;
@@ -172,7 +165,24 @@ __global__ void k_lay_tour(int32_t* __restrict__ tour, const int32_t* __restrict
       tour[p] = 0;
       continue;
     }
-    tour[p] = y >= 0 ? pre_of[v] : ~pre_of[v];
+    const int32_t x = pre_of[v];
+    tour[p] = y >= 0 ? x : ~x;
+    if (y < 0 || x < 0 || x >= n) continue;  // (a label out of range is reported by k_lay_vertices)
+    const int depth = (int)(2 * dpre[p] + 1 - p);
+    up[x].w = depth;
+    mx = max(mx, depth);
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax((long long*)&dsc->max_depth, (long long)mx);
+}
+
+// three ancestors of every label beside its depth: the climbs of the join take three steps per load
+__global__ void k_lay_up(const int32_t* __restrict__ parent_pre, int64_t n, int4* __restrict__ up) {
+  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t p1 = parent_pre[x];
+    const int32_t p2 = p1 >= 0 ? parent_pre[p1] : -1;
+    const int32_t p3 = p2 >= 0 ? parent_pre[p2] : -1;
+    up[x] = make_int4(p1, p2, p3, p1 >= 0 ? up[x].w : 0);
   }
 }
 
@@ -214,6 +224,7 @@ int build_tree_layout(Handle& h) {
   // resident layout
   if ((st = device_alloc(h, (void**)&h.tour, sizeof(int32_t) * (size_t)std::max<int64_t>(A, 1))) ||
       (st = device_alloc(h, (void**)&h.vtx_of_pre, sizeof(int32_t) * (size_t)n)) ||
+      (st = device_alloc(h, &h.up, sizeof(int4) * (size_t)n)) ||
       (st = device_alloc(h, (void**)&h.P, sizeof(u128) * (size_t)n)))
     return st;
   // range-minimum levels: level j + 1 holds the minima of the 32-entry groups of level j, up to one group;
@@ -286,15 +297,14 @@ int build_tree_layout(Handle& h) {
     k_lay_arcs<<<gn, kBlock, 0, s>>>(tadj, tptr, h.parent, ranked[c], h.d_vtx_ptr, G, n, h.tour, dflag, bad);
     if ((st = ensure_scan_status(h, A)) || (st = scan_excl_i32(h, dflag, dpre, A, nullptr, A))) return fail(st);
     k_lay_pre<<<ga, kBlock, 0, s>>>(h.tour, dpre, A, h.d_vtx_ptr, G, pre_of);
-    LAY_CK(cudaMemsetAsync(&h.dsc->max_depth, 0, sizeof(int64_t), s));
-    k_lay_depth<<<ga, kBlock, 0, s>>>(h.tour, dpre, A, h.dsc);
   }
   k_lay_roots<<<gn, kBlock, 0, s>>>(h.parent, h.d_vtx_ptr, G, n, pre_of);
   k_lay_vertices<<<gn, kBlock, 0, s>>>(pre_of, h.parent, n, h.vtx_of_pre, parent_pre, h.P, h.rmq_val[0], bad);
-  if (A > 0) k_lay_tour<<<ga, kBlock, 0, s>>>(h.tour, pre_of, A, n, bad);
+  LAY_CK(cudaMemsetAsync(&h.dsc->max_depth, 0, sizeof(int64_t), s));
+  if (A > 0)
+    k_lay_tour<<<ga, kBlock, 0, s>>>(h.tour, pre_of, dpre, A, n, static_cast<int4*>(h.up), h.dsc, bad);
   {
     int32_t hbad = 0;
-    if (A == 0) LAY_CK(cudaMemsetAsync(&h.dsc->max_depth, 0, sizeof(int64_t), s));
     LAY_CK(cudaMemcpyAsync(&hbad, bad, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     LAY_CK(cudaMemcpyAsync(h.hsc, h.dsc, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
     LAY_CK(cudaStreamSynchronize(s));
@@ -306,6 +316,7 @@ int build_tree_layout(Handle& h) {
     if (h.hsc->e_max != INT_MIN && h.hsc->e_max - h.hsc->e_min + 53 + dep_bits > 96) return fail(PDG_E_RANGE);
   }
   if (m > 0) k_lay_edges<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, pre_of, m);
+  k_lay_up<<<gn, kBlock, 0, s>>>(parent_pre, n, static_cast<int4*>(h.up));
   LAY_CK(cudaMemcpyAsync(h.parent, parent_pre, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
   LAY_CK(cudaGetLastError());
 #undef LAY_CK

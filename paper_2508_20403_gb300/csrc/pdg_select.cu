@@ -170,6 +170,14 @@ __global__ void __launch_bounds__(kBlock) k_sel_pick(uint32_t* __restrict__ hist
 // blocks add up the counts of the blocks before them and place each tile's
 // selected edges by a block scan.  Both passes stream the keys with vector
 // loads.
+struct CandSrc {
+  const int32_t* u;
+  const int32_t* v;
+  const int32_t* lca;
+  const int32_t* id;
+  int4* rec;  // [2 R]: u, v, LCA, canonical id; score bits
+};
+
 template <bool WRITE>
 __global__ void __launch_bounds__(kBlock) k_sel_compact(const uint64_t* __restrict__ key, int64_t E,
                                                         const int64_t* __restrict__ off_ptr, int32_t G,
@@ -177,9 +185,11 @@ __global__ void __launch_bounds__(kBlock) k_sel_compact(const uint64_t* __restri
                                                         int64_t* __restrict__ bcount, int64_t cap,
                                                         int32_t* __restrict__ cand_idx,
                                                         uint64_t* __restrict__ rkey, int32_t* __restrict__ rval,
-                                                        const int64_t* __restrict__ cand_ptr, DevScalars* dsc) {
+                                                        const int64_t* __restrict__ cand_ptr, CandSrc src,
+                                                        DevScalars* dsc) {
   dep_sync();
   __shared__ int64_t sm[kBlock / 32 + 1];
+  __shared__ uint16_t s_pick[WRITE ? kTile : 1];
   const int64_t chunk = sel_chunk(E, gridDim.x);
   const int64_t b0 = (int64_t)blockIdx.x * chunk;
   const int64_t b1 = min(E, b0 + chunk);
@@ -240,20 +250,27 @@ __global__ void __launch_bounds__(kBlock) k_sel_compact(const uint64_t* __restri
       tot += cnt;
       continue;
     }
+    // the tile's selected edges are listed in shared memory, then taken by neighbouring threads: every access
+    // below but the gathers of the edge's own words is coalesced, and those are in id order
     int64_t tile_tot;
-    int64_t pos = run + block_excl_scan(cnt, sm, &tile_tot);
+    int at = (int)block_excl_scan(cnt, sm, &tile_tot);
 #pragma unroll
-    for (int i = 0; i < kItems; i++) {
-      if (pick & (1u << i)) {
-        if (pos < cap) {
-          cand_idx[pos] = (int32_t)(base + i);
-          rkey[pos] = ~k[i];  // ascending ~score = descending score
-          rval[pos] = (int32_t)pos;
-        }
-        pos++;
-      }
+    for (int i = 0; i < kItems; i++)
+      if (pick & (1u << i)) s_pick[at++] = (uint16_t)(threadIdx.x * kItems + i);
+    __syncthreads();
+    for (int j = threadIdx.x; j < (int)tile_tot; j += kBlock) {
+      const int64_t i = t0 + s_pick[j], pos = run + j;
+      if (pos >= cap) break;
+      const uint64_t kk = __ldg(key + i);
+      cand_idx[pos] = (int32_t)i;
+      rkey[pos] = ~kk;  // ascending ~score = descending score
+      rval[pos] = (int32_t)pos;
+      // what the later steps read of a candidate, in one sector
+      src.rec[2 * pos] = make_int4(__ldg(src.u + i), __ldg(src.v + i), __ldg(src.lca + i), __ldg(src.id + i));
+      reinterpret_cast<uint64_t*>(src.rec)[4 * pos + 2] = kk;
     }
     run += tile_tot;
+    __syncthreads();
   }
   if (!WRITE) {
     tot = block_sum(tot, sm);
@@ -283,10 +300,11 @@ int step_select(Handle& h) {
   int64_t* bcount = h.blk_a;
   ++h.launches;
   launch_k(h, k_sel_compact<false>, nb, kBlock, 0, h.key, E, h.d_off_ptr, h.G, h.sel, bcount, 0, nullptr, nullptr,
-           nullptr, h.d_cand_ptr, h.dsc);
+           nullptr, h.d_cand_ptr, CandSrc{}, h.dsc);
   ++h.launches;
   launch_k(h, k_sel_compact<true>, nb, kBlock, 0, h.key, E, h.d_off_ptr, h.G, h.sel, bcount, h.Rcap, h.cand_idx,
-           h.rk[0], h.rv[0], h.d_cand_ptr, h.dsc);
+           h.rk[0], h.rv[0], h.d_cand_ptr,
+           CandSrc{h.off_u, h.off_v, h.lca, h.off_id, static_cast<int4*>(h.cand_rec)}, h.dsc);
   PDG_CUDA(cudaGetLastError());
   return PDG_OK;
 }

@@ -399,6 +399,7 @@ struct CoopSortArgs {
   const int64_t* cand_ptr;
   int32_t G;
   int nd_graph, nd_lca;
+  int group;  // 1: also group the ranks by LCA (the tiers read subtasks; the join needs the order alone)
   uint32_t* counts;  // [tiles][256]
   uint32_t* totals;  // [kCoKeySets][kMaxDigits][256], zero at launch
   uint32_t* bar;     // barrier arrivals, zero at launch
@@ -422,6 +423,7 @@ struct CoopSmem {
 // no returned atomic on the path.  The wait is bounded (spin_limit).
 __device__ __forceinline__ void coop_barrier(const CoopSortArgs& a, uint32_t& target) {
   __syncthreads();
+  if (gridDim.x == 1) return;  // a single tile: its own block is the whole grid
   target += gridDim.x;
   if (threadIdx.x == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar) : "memory");
@@ -629,7 +631,14 @@ __global__ void __launch_bounds__(kCoThreads) k_sort_coop(CoopSortArgs a) {
     __syncthreads();
     coop_keyset(a, sm, 1, a.nd_graph, cur, target, N, tiles);
   }
-  // 3. rank_cand[r] = candidate at rank r; keys := LCA, values := rank; group by LCA
+  // 3. rank_cand[r] = candidate at rank r; for the tiers keys := LCA, values := rank, grouped by LCA
+  if (!a.group) {
+    if (blockIdx.x < tiles)
+      for (int64_t i = t0 + threadIdx.x; i < N && i < t0 + kCoTile; i += kCoThreads)
+        a.rank_cand[i] = __ldcg(a.v[cur] + i);
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.dsc->radix_sel = cur;
+    return;
+  }
   if (blockIdx.x < tiles)
     for (int64_t i = t0 + threadIdx.x; i < N && i < t0 + kCoTile; i += kCoThreads) {
       const int32_t c = __ldcg(a.v[cur] + i);
@@ -694,6 +703,7 @@ static int step_sort_coop(Handle& h, int grid_max) {
   a.nd_graph = 0;
   while ((1ll << (8 * a.nd_graph)) < h.G) a.nd_graph++;
   a.nd_lca = 0;
+  a.group = h.tiered ? 1 : 0;
   while ((1ll << (8 * a.nd_lca)) < h.n) a.nd_lca++;
   a.counts = h.radix_status;
   a.totals = totals;
@@ -719,8 +729,7 @@ int step_sort(Handle& h) {
   // one cooperative launch when every tile of the candidate capacity has its own resident block
   const int cgrid = h.opt.sort_one_launch ? coop_sort_grid() : 0;
   if (cgrid > 0 && (h.Rcap + kCoTile - 1) / kCoTile <= cgrid &&
-      kRadixHistOnesweep + (int64_t)kCoKeySets * kMaxDigits * kRdxBins <= kRadixHistWords &&
-      (int64_t)cgrid * kRdxBins <= (int64_t)kRadixPassesMax * 256 * ((h.Rcap + kTile - 1) / kTile))
+      kRadixHistOnesweep + (int64_t)kCoKeySets * kMaxDigits * kRdxBins <= kRadixHistWords)
     return step_sort_coop(h, cgrid);
   const int grid = h.num_sms * 4;
   const int64_t tiles_max = sort_tiles(h);
@@ -741,6 +750,12 @@ int step_sort(Handle& h) {
     while ((1ll << (8 * nd)) < h.G) nd++;
     if ((st = onesweep(h, 0, nd, pass))) return st;
     pass += nd;
+  }
+  if (!h.tiered) {  // the join needs the order alone
+    ++h.launches;
+    launch_k(h, k_copy_vals, grid, kBlock, 0, h.rv[0], h.rv[1], h.rank_cand, h.dsc);
+    PDG_CUDA(cudaGetLastError());
+    return PDG_OK;
   }
   // 2. group ranks by LCA
   ++h.launches;
