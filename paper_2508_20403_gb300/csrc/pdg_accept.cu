@@ -117,7 +117,7 @@ __device__ __forceinline__ bool strictly_similar(const int32_t (&Up)[kA], const 
 __global__ void __launch_bounds__(kBlock) k_build_records(
     const int32_t* __restrict__ lsort_rank, const int32_t* __restrict__ rank_cand, const int32_t* __restrict__ cand_idx,
     const int32_t* __restrict__ ou, const int32_t* __restrict__ ov, const int32_t* __restrict__ lca,
-    const u128* __restrict__ P, const int32_t* __restrict__ parent,
+    const int4* __restrict__ up, const int32_t* __restrict__ parent,
     int c, const DevScalars* __restrict__ dsc, int64_t cap, int32_t* __restrict__ rec_u, int32_t* __restrict__ rec_v,
     int32_t* __restrict__ rec_anc, int32_t* __restrict__ rec_du, int32_t* __restrict__ rec_dv,
     uint8_t* __restrict__ rec_b, int32_t* __restrict__ rec_rank, int32_t* __restrict__ rec_lca) {
@@ -129,8 +129,7 @@ __global__ void __launch_bounds__(kBlock) k_build_records(
     const int32_t i = cand_idx[rank_cand[r]];
     const int32_t u = ou[i], v = ov[i];  // u < v
     const int32_t l = lca[i];
-    const int32_t dl = (int32_t)(uint32_t)P[l];
-    const int32_t du = (int32_t)(uint32_t)P[u] - dl, dv = (int32_t)(uint32_t)P[v] - dl;
+    const int32_t dl = up[l].w, du = up[u].w - dl, dv = up[v].w - dl;
     rec_u[s] = u;
     rec_v[s] = v;
     int32_t au = u, av = v;
@@ -1086,7 +1085,7 @@ int step_accept(Handle& h, int c) {
   int st;
   ++h.launches;
   launch_k(h, k_build_records, grid, kBlock, 0, h.lsort_rank, h.rank_cand, h.cand_idx, h.off_u, h.off_v, h.lca,
-           h.P, h.parent, c, h.dsc, cap, h.rec_u, h.rec_v, h.rec_anc,
+           static_cast<const int4*>(h.up), h.parent, c, h.dsc, cap, h.rec_u, h.rec_v, h.rec_anc,
            h.rec_du, h.rec_dv, h.rec_b, h.rec_rank, h.rec_lca);
   // subtask boundaries, tier lists, per-position tiers
   const int64_t lb_tiles = (cap + kLbTile - 1) / kLbTile;

@@ -120,7 +120,6 @@ __global__ void k_reset_recover(DevScalars* dsc) {
   dsc->err = 0;
   dsc->e_min = INT_MAX;
   dsc->e_max = INT_MIN;
-  dsc->score_ticket = 0;
 }
 
 // The attempt's scalars, the join's cell table emptied (the slots; the members

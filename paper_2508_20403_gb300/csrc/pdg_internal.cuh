@@ -28,8 +28,6 @@ constexpr int kBlockTierDefault = 0;  // off: on the mesh and R-MAT workloads th
 constexpr int kRadixHistOnesweep = 16 * 256 + 2 * kRadixPassesMax;  // per-pass sort: histograms, skip flags, buffers
 constexpr int kRadixHistWords = kRadixHistOnesweep + 3 * 8 * 256;     // + the one-launch sort's key-set histograms
 constexpr uint64_t kEmptyKey = ~0ull;
-constexpr int kRmqMaxLevels = 6;  // levels of the range-minimum structure (n < 2^30: 30 / 5)
-constexpr int kRmqStMax = 6144;   // level-2 entries up to which levels 2+ are one sparse table (n <= 6.29M)
 
 // The join of steps A5 + A6 walks the members of coarse cells; a cell of
 // kJoinCellMax members, or a block that met more earlier members in the cells
@@ -95,7 +93,6 @@ struct DevScalars {
   int64_t n_cand_wanted;  // candidates the selection produced (may exceed capacity)
   int64_t n_constrained;  // cooperative tier: candidates with a possible earlier marker
   int64_t n_big_chunk;    // cooperative tier: chunks of at most kBigChunk positions
-  unsigned long long score_ticket;  // step A3: next tile of off-tree edges to score
   uint32_t epoch;       // attempts so far (tags the cooperative tier's undecided entries)
   int32_t bounds_site;  // first failed bounds check (see ERR_BOUNDS)
   int32_t bounds_where;  // its round (99: serial finisher)
@@ -200,20 +197,14 @@ struct Handle {
   int64_t* blk_b = nullptr;
   int nblk = 0;
 
-  // tree: P(x) = D(x) * 2^32 + depth(x); D = exact root distance in units of 2^-S
-  u128* P = nullptr;
-  // range-minimum structure over val0[x] = depth(x) * 2^32 + parent(x):
-  // level j + 1 holds the minima of the 32-entry groups of level j
-  int rmq_levels = 0;
-  int64_t rmq_size[kRmqMaxLevels] = {0};
-  uint64_t* rmq_val[kRmqMaxLevels] = {nullptr};
-  uint32_t* rmq_mask[kRmqMaxLevels] = {nullptr};
-  uint64_t* rmq_pmin[kRmqMaxLevels] = {nullptr};  // per entry: minimum from its group's start (null: top level)
-  uint64_t* rmq_smin[kRmqMaxLevels] = {nullptr};  // per entry: minimum to its group's end
-  uint64_t* rmq_st = nullptr;  // sparse table over level 2 (row t: minima of 2^t entries; row 0 is level 2)
-  int rmq_st_rows = 0;
+  // per label one 32-byte record: P(x) = D(x) * 2^32 + depth(x) (u128; D = exact root distance in units of
+  // 2^-S), then of the parent array, inside the label's 32-label group: minimum up to it, minimum after it,
+  // suffix-minimum mask, its own parent
+  void* rec = nullptr;
+  // sparse table over the group minima of the parent array (row t: minima of 2^t consecutive groups)
+  int32_t* rmq_table = nullptr;
+  int rmq_rows = 0;
   u128* ts_sum = nullptr;        // tree scan: tile sums
-  uint32_t* ts_done = nullptr;   // range-minimum build: blocks finished
 
   // scores
   uint64_t* key = nullptr;  // FP64 score bits (positive -> order preserving)
@@ -345,6 +336,14 @@ __device__ __forceinline__ int64_t row_of(const int64_t* __restrict__ row_ptr, i
     if (__ldg(row_ptr + mid) <= p) lo = mid; else hi = mid;
   }
   return lo;
+}
+
+// one aligned 32-byte sector in one load (two 16-byte loads of it are two requests, and the second misses L1
+// while the first is in flight)
+__device__ __forceinline__ void load_sector(const void* p, uint4& x, uint4& y) {
+  asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w), "=r"(y.x), "=r"(y.y), "=r"(y.z), "=r"(y.w)
+      : "l"(p));
 }
 
 // index of the first entry >= x in a sorted int32 range, or end

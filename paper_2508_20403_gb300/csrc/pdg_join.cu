@@ -103,14 +103,6 @@ __device__ __forceinline__ uint32_t home_bucket(const JoinArgs& a, uint64_t key)
   return (uint32_t)__umul64hi(mix64(key), a.buckets);
 }
 
-// one aligned 32-byte sector in one load (two 16-byte loads of it are two requests, and the second misses L1
-// while the first is in flight)
-__device__ __forceinline__ void load_sector(const void* p, uint4& x, uint4& y) {
-  asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w), "=r"(y.x), "=r"(y.y), "=r"(y.z), "=r"(y.w)
-      : "l"(p));
-}
-
 __device__ __forceinline__ uint64_t slot_key(const uint4& x) { return (uint64_t)x.y << 32 | x.x; }
 
 // the slot of `key` in a finished table (its words to `found`), or kNoSlot

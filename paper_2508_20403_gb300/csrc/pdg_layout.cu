@@ -6,8 +6,8 @@
 //   * Vertices are relabelled in DFS preorder of T (per graph of a batch,
 //     inside the graph's own vertex range, the root first).  Every subtree is
 //     then a contiguous label range, so
-//       - LCA(u, v), u < v, is the parent of any vertex of minimum depth among
-//         the labels (u, v] (a range-minimum query, step A3), and
+//       - LCA(u, v), u < v, is the smallest parent among the labels (u, v] (a
+//         range-minimum query, step A3), and
 //       - the children of an LCA order the same way as the endpoints below
 //         them, which orients the records of step A5 without a search.
 //     The canonical edge list keeps its order (canonical ids are unchanged);
@@ -133,7 +133,7 @@ __global__ void k_lay_roots(const int32_t* __restrict__ parent, const int64_t* _
 // (root distance 0, depth 0)
 __global__ void k_lay_vertices(const int32_t* __restrict__ pre_of, const int32_t* __restrict__ parent, int64_t n,
                                int32_t* __restrict__ vtx_of_pre, int32_t* __restrict__ parent_pre,
-                               u128* __restrict__ P, uint64_t* __restrict__ val0, int32_t* __restrict__ bad) {
+                               u128* __restrict__ rec, int32_t* __restrict__ bad) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
     const int32_t x = pre_of[v];
     const int32_t p = parent[v];
@@ -143,10 +143,7 @@ __global__ void k_lay_vertices(const int32_t* __restrict__ pre_of, const int32_t
     }
     vtx_of_pre[x] = (int32_t)v;
     parent_pre[x] = p < 0 ? -1 : pre_of[p];
-    if (p < 0) {
-      P[x] = 0;
-      val0[x] = 0;  // never inside a query range (every range starts after a vertex of the root's graph)
-    }
+    if (p < 0) rec[2 * (int64_t)x] = 0;
   }
 }
 
@@ -225,36 +222,13 @@ int build_tree_layout(Handle& h) {
   if ((st = device_alloc(h, (void**)&h.tour, sizeof(int32_t) * (size_t)std::max<int64_t>(A, 1))) ||
       (st = device_alloc(h, (void**)&h.vtx_of_pre, sizeof(int32_t) * (size_t)n)) ||
       (st = device_alloc(h, &h.up, sizeof(int4) * (size_t)n)) ||
-      (st = device_alloc(h, (void**)&h.P, sizeof(u128) * (size_t)n)))
+      (st = device_alloc(h, &h.rec, 2 * sizeof(u128) * (size_t)n)))
     return st;
-  // range-minimum levels: level j + 1 holds the minima of the 32-entry groups of level j, up to one group;
-  // when level 2 is small enough, it and everything above it is one sparse table instead
-  h.rmq_levels = 0;
-  h.rmq_st = nullptr;
-  h.rmq_st_rows = 0;
-  for (int64_t sz = n;; sz = (sz + 31) / 32) {
-    if (h.rmq_levels >= kRmqMaxLevels) return PDG_E_INVALID_ARG;
-    if (h.rmq_levels == 2 && sz <= kRmqStMax) {
-      int rows = 1;
-      while ((1ll << rows) <= sz) rows++;  // rows t = 0 .. floor(log2 sz)
-      if ((st = device_alloc(h, (void**)&h.rmq_st, sizeof(uint64_t) * (size_t)sz * rows))) return st;
-      h.rmq_st_rows = rows;
-      h.rmq_size[2] = sz;
-      h.rmq_val[2] = h.rmq_st;  // row 0: the level-2 entries themselves
-      h.rmq_levels = 3;
-      break;
-    }
-    h.rmq_size[h.rmq_levels] = sz;
-    if ((st = device_alloc(h, (void**)&h.rmq_val[h.rmq_levels], sizeof(uint64_t) * (size_t)sz)) ||
-        (st = device_alloc(h, (void**)&h.rmq_mask[h.rmq_levels], sizeof(uint32_t) * (size_t)sz)))
-      return st;
-    if (sz > 32 &&  // below the top level, queries read partial groups from these
-        ((st = device_alloc(h, (void**)&h.rmq_pmin[h.rmq_levels], sizeof(uint64_t) * (size_t)sz)) ||
-         (st = device_alloc(h, (void**)&h.rmq_smin[h.rmq_levels], sizeof(uint64_t) * (size_t)sz))))
-      return st;
-    h.rmq_levels++;
-    if (sz <= 32) break;
-  }
+  // the range-minimum table: a row per power of two up to the number of 32-label groups
+  const int64_t n1 = (n + 31) / 32;
+  h.rmq_rows = 1;
+  while ((1ll << h.rmq_rows) <= n1) h.rmq_rows++;
+  if ((st = device_alloc(h, (void**)&h.rmq_table, sizeof(int32_t) * (size_t)n1 * h.rmq_rows))) return st;
   uint8_t* tflag = nullptr;
   int32_t *tdeg = nullptr, *cur = nullptr, *tadj = nullptr, *rev = nullptr, *arc_uv = nullptr, *dflag = nullptr;
   int32_t *succ = nullptr, *rd = nullptr, *pre_of = nullptr, *parent_pre = nullptr;
@@ -299,7 +273,8 @@ int build_tree_layout(Handle& h) {
     k_lay_pre<<<ga, kBlock, 0, s>>>(h.tour, dpre, A, h.d_vtx_ptr, G, pre_of);
   }
   k_lay_roots<<<gn, kBlock, 0, s>>>(h.parent, h.d_vtx_ptr, G, n, pre_of);
-  k_lay_vertices<<<gn, kBlock, 0, s>>>(pre_of, h.parent, n, h.vtx_of_pre, parent_pre, h.P, h.rmq_val[0], bad);
+  k_lay_vertices<<<gn, kBlock, 0, s>>>(pre_of, h.parent, n, h.vtx_of_pre, parent_pre,
+                                       static_cast<u128*>(h.rec), bad);
   LAY_CK(cudaMemsetAsync(&h.dsc->max_depth, 0, sizeof(int64_t), s));
   if (A > 0)
     k_lay_tour<<<ga, kBlock, 0, s>>>(h.tour, pre_of, dpre, A, n, static_cast<int4*>(h.up), h.dsc, bad);

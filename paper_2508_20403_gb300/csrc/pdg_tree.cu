@@ -12,16 +12,24 @@
 // k_tree_sum + k_tree_scan: one prefix sum over the Euler tour.  A down arc
 // into v adds word(v) = fixed(r(v)) * 2^32 + 1, an up arc out of v subtracts
 // it, so the running sum at v's down arc is P(v).  Integer addition is
-// associative: the tiled scan gives the same bits as a sequential walk.  The
-// same pass writes, per vertex (preorder label x), the range-minimum key
-// val0[x] = depth(x) * 2^32 + parent(x).
+// associative: the tiled scan gives the same bits as a sequential walk.
 //
-// k_rmq_build: the range-minimum structure over val0.  Level j + 1 holds the
-// minima of the 32-entry groups of level j, up to a single group.  Inside a
-// group, mask[k] has bit i set when entry i (i <= k) has a smaller depth than
-// every later entry up to k (a suffix minimum); the minimum depth over [i, k]
-// in one group is then found at the lowest set bit of mask[k] at or above i.
-// A query (step A3) combines at most two partial groups per level.
+// k_rmq_groups + k_rmq_rows: the structure that answers LCA queries.  With
+// preorder labels u < v, LCA(u, v) is the SMALLEST parent label among the
+// labels (u, v]: all of them lie in the subtree of l = LCA(u, v), whose root
+// has its smallest label, and none is l itself, so no parent is below l; and
+// the child of l on v's side lies there, so l is among the parents.  So the
+// query is a plain range minimum over the 4-byte parent array: inside 32-label
+// groups the running minima from both ends (and, for a range inside one group,
+// the suffix-minimum mask: bit i of mask[k] set when the parent of entry
+// i <= k is below those of all later entries up to k, so the minimum of
+// [i, k] stands at the lowest set bit at or above i); over whole groups a
+// sparse table, row t the minima of 2^t consecutive groups.
+//
+// What step A3 gathers of a label is one 32-byte record: P, the two running
+// minima, the mask, the parent.  That kernel is bound by the number of
+// distinct sectors its lanes touch per edge (one tag lookup each in L1), so
+// two records, two table entries and P(l) take the place of nine words.
 #include <algorithm>
 #include <climits>
 
@@ -85,11 +93,9 @@ struct TreeScanArgs {
   const int32_t* tour;
   int64_t A;
   const double* rtree;
-  const int32_t* parent;
   int dep_bits;
   DevScalars* dsc;
-  u128* P;
-  uint64_t* val0;
+  u128* rec;   // a label's record: P, then the range-minimum words
   u128* tsum;  // [tiles] tile sums
 };
 
@@ -183,204 +189,122 @@ __global__ void __launch_bounds__(kTsThreads, 4) k_tree_scan(TreeScanArgs a) {
   for (int i = 0; i < kTsItems; i++) {
     if (arc[i] == INT_MIN) continue;
     p += arc_word(arc[i], r[i], e_min, range_ok);
-    if (arc[i] >= 0) {  // the down arc into x: P(x) and the range-minimum key
-      const int32_t x = arc[i];
-      a.P[x] = p;
-      a.val0[x] = ((uint64_t)(uint32_t)p << 32) | (uint32_t)__ldg(a.parent + x);
-    }
+    if (arc[i] >= 0) a.rec[2 * (int64_t)arc[i]] = p;  // the down arc into x: P(x)
   }
 }
 
-// The range-minimum structure in one launch.  Each block takes 8192 entries
-// of level 0 (256 groups) and then the 256 group minima it produced (8 groups
-// of level 1); the last block to finish builds the remaining, small levels.
-// A group's masks are the stacks of suffix minima, as a bit set, that a walk
-// over its 32 entries would hold: entry k pops the stacked entries whose
-// depth is not below its own, then pushes itself, and the stack after entry
-// k is mask[k] (built without the walk, see rmq_chunk).
+// One block takes 256 groups of 32 labels: a warp loads 32 of them (coalesced),
+// its lanes build one group's masks each from registers (mask[k] =
+// (mask[k-1] & {j < k : parent j < parent k}) | bit k, 31 comparisons, no
+// data-dependent step), then the warp walks the groups with a lane per label
+// for the running minima, so that the records leave as whole runs.  The first
+// rows of the sparse table, up to windows of 256 groups, come from the block's
+// minima and those of the 256 groups after them, which it recomputes (one
+// warp-wide minimum per group) rather than wait for another block.  Padding
+// past the last label is larger than any parent.
 constexpr int kRmqThreads = 256;
-constexpr int kRmqChunk = kRmqThreads * 32;  // entries per block and pass
-
-struct RmqArgs {
-  uint64_t* val[kRmqMaxLevels];
-  uint32_t* mask[kRmqMaxLevels];
-  uint64_t* pmin[kRmqMaxLevels];
-  uint64_t* smin[kRmqMaxLevels];
-  int64_t size[kRmqMaxLevels];
-  int levels;
-  uint32_t* done;  // blocks finished (the last one resets it)
-  uint64_t* st;    // level 2 and up as one sparse table (null: as levels)
-  int st_rows;
-};
-
-// entries [base, base + len) of one level (len <= kRmqChunk, base a multiple
-// of 32): their masks, the minima from the group start up to each entry
-// (pmin) and from each entry to the group end (smin), and the minimum of
-// every group to val_next[entry / 32] when val_next is given.
-// The chunk is staged in shared memory by coalesced loads; then one thread
-// takes one group into registers and builds it without a data-dependent
-// step: the stack after entry k keeps the earlier stack entries shallower
-// than entry k, so mask[k] = (mask[k-1] & {j < k : depth j < depth k}) | bit k,
-// where the set is 31 comparisons of registers; pmin and smin are running
-// minima of the 64-bit keys (a minimum-depth entry of the range; ties carry
-// the same parent inside any query range).  Padding past the level's end is
-// deeper than any entry.
-// (FROM_PREV: the level was written by an earlier kernel, so its reads may use
-// the read-only cache; levels written by this kernel are read from L2)
-__device__ __forceinline__ uint64_t rmq_load(const uint64_t* p, bool from_prev) {
-  return from_prev ? __ldg(p) : __ldcg(p);
-}
+constexpr int kRmqGroups = 256;  // groups per block
+constexpr int kRmqRow0 = 8;      // rows 0 .. kRmqRow0 are built with the groups
 
 struct RmqSmem {
-  uint64_t v[kRmqChunk / 32][33];  // values, a padded row per group (then the minima being written out)
-  uint32_t m[kRmqChunk / 32][33];  // masks
+  int32_t p[kRmqGroups][33];   // parents, a padded row per group
+  uint32_t m[kRmqGroups][33];  // masks
+  int32_t row[2][2 * kRmqGroups];
 };
 
-__device__ void rmq_chunk(const uint64_t* __restrict__ val, int64_t size, int64_t base, int len,
-                          uint32_t* __restrict__ mask, uint64_t* __restrict__ pmin, uint64_t* __restrict__ smin,
-                          uint64_t* __restrict__ val_next, RmqSmem& sm, bool from_prev) {
-  constexpr int kPer = kRmqChunk / kRmqThreads;
-  const int t = threadIdx.x;
-  const int ngroups = (len + 31) / 32;
-  {
-    uint64_t x[kPer];  // a thread's loads are independent and in flight together
-#pragma unroll
-    for (int i = 0; i < kPer; i++) {
-      const int li = i * kRmqThreads + t;
-      const int64_t idx = base + li;
-      x[i] = (li < ngroups * 32 && li < len && idx < size) ? rmq_load(val + idx, from_prev) : ~0ull;
-    }
-#pragma unroll
-    for (int i = 0; i < kPer; i++) {
-      const int li = i * kRmqThreads + t;
-      if (li < ngroups * 32) sm.v[li >> 5][li & 31] = x[i];
-    }
-  }
-  __syncthreads();
-  uint64_t v[32];
-  const bool own = t < ngroups;
-  if (own) {
-#pragma unroll
-    for (int k = 0; k < 32; k++) v[k] = sm.v[t][k];
-    uint32_t mk = 0;
-#pragma unroll
-    for (int k = 0; k < 32; k++) {
-      const uint32_t dk = (uint32_t)(v[k] >> 32);
-      uint32_t shallower = 0;
-#pragma unroll
-      for (int j = 0; j < k; j++) shallower |= ((uint32_t)(v[j] >> 32) < dk ? 1u : 0u) << j;
-      mk = (mk & shallower) | (1u << k);
-      sm.m[t][k] = mk;
-    }
-    uint64_t pm = ~0ull;
-#pragma unroll
-    for (int k = 0; k < 32; k++) {
-      pm = min(pm, v[k]);
-      sm.v[t][k] = pm;  // only this thread reads its row
-    }
-    if (val_next && base + 32 * t < size) val_next[(base >> 5) + t] = pm;
-    uint64_t sf = ~0ull;
-#pragma unroll
-    for (int k = 31; k >= 0; k--) {
-      sf = min(sf, v[k]);
-      v[k] = sf;
-    }
-  }
-  __syncthreads();
-  for (int i = t; i < len; i += kRmqThreads) {
-    const int64_t idx = base + i;
-    if (idx >= size) break;  // idx grows with i
-    mask[idx] = sm.m[i >> 5][i & 31];
-    if (pmin) pmin[idx] = sm.v[i >> 5][i & 31];
-  }
-  if (pmin) {  // uniform
-    __syncthreads();
-    if (own) {
-#pragma unroll
-      for (int k = 0; k < 32; k++) sm.v[t][k] = v[k];
-    }
-    __syncthreads();
-    for (int i = t; i < len; i += kRmqThreads) {
-      const int64_t idx = base + i;
-      if (idx >= size) break;
-      smin[idx] = sm.v[i >> 5][i & 31];
-    }
-  }
-  __syncthreads();
-}
-
-// Level 2 and up as a sparse table: row t holds the minimum of the 2^t entries from each position, so any range
-// [lo, hi] of level 2 is the smaller of two entries of row floor(log2(hi - lo + 1)).  Row 0 is level 2 itself
-// (written by the blocks as their level-1 group minima); each further row comes from the one before, kept in
-// shared memory (two rows of at most kRmqStMax entries), and is stored as it is made.
-__device__ void rmq_sparse_table(const RmqArgs& a, uint64_t* buf) {
-  const int64_t n2 = a.size[2];
-  uint64_t* cur = buf;
-  uint64_t* nxt = buf + kRmqStMax;
-  for (int64_t i = threadIdx.x; i < n2; i += kRmqThreads) cur[i] = __ldcg(a.st + i);
-  __syncthreads();
-  for (int r = 1; r < a.st_rows; r++) {
-    const int64_t h = 1ll << (r - 1);
-    uint64_t* row = a.st + (int64_t)r * n2;
-    for (int64_t i = threadIdx.x; i + 2 * h <= n2; i += kRmqThreads) {
-      const uint64_t x = min(cur[i], cur[i + h]);
-      nxt[i] = x;
-      row[i] = x;
-    }
-    __syncthreads();
-    uint64_t* t = cur;
-    cur = nxt;
-    nxt = t;
-  }
-}
-
-__global__ void __launch_bounds__(kRmqThreads, 2) k_rmq_build(RmqArgs a) {
+__global__ void __launch_bounds__(kRmqThreads) k_rmq_groups(const int32_t* __restrict__ parent, int64_t n, int64_t n1,
+                                                            int4* __restrict__ rec, int32_t* __restrict__ table,
+                                                            int rows) {
   dep_sync();
   extern __shared__ __align__(16) unsigned char rmq_smem[];
   RmqSmem& sm = *reinterpret_cast<RmqSmem*>(rmq_smem);
-  __shared__ int s_last;
-  const int64_t b0 = (int64_t)blockIdx.x * kRmqChunk;
-  // the chunks this block builds, in order (one call site keeps the register budget of one chunk):
-  // its 8192 entries of level 0, their 256 minima on level 1, and for the last block every chunk of level 2 up
-  int j = 0;
-  int64_t base = b0;
-  int len = kRmqChunk;
-  bool tail = false;
-  for (;;) {
-    rmq_chunk(a.val[j], a.size[j], base, len, a.mask[j], a.pmin[j], a.smin[j],
-              j + 1 < a.levels ? a.val[j + 1] : nullptr, sm, j == 0);
-    if (!tail) {
-      if (j == 0 && a.levels > 1) {
-        j = 1;
-        base = b0 / 32;
-        len = kRmqThreads;
-        continue;
-      }
-      if (a.levels <= 2) return;  // uniform
-      if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = (atomicAdd(a.done, 1u) == gridDim.x - 1) ? 1 : 0;
-      }
-      __syncthreads();
-      if (!s_last) return;
-      __threadfence();
-      if (a.st) {  // uniform: the sparse table over level 2, two rows at a time in shared memory
-        rmq_sparse_table(a, reinterpret_cast<uint64_t*>(&sm));
-        break;
-      }
-      tail = true;
-      j = 2;
-      base = 0;
-    } else {
-      base += kRmqChunk;
-      if (base >= a.size[j]) {
-        if (++j >= a.levels) break;
-        base = 0;
-      }
-    }
-    len = (int)min((int64_t)kRmqChunk, a.size[j] - base);
+  const int lane = threadIdx.x & 31, w0 = threadIdx.x & ~31;  // the warp's first group
+  const int64_t g0 = (int64_t)blockIdx.x * kRmqGroups;
+  int32_t halo[32];  // the block after this one: this warp's share of its groups
+#pragma unroll
+  for (int j = 0; j < 32; j++) {
+    const int64_t x = (g0 + w0 + j) * 32 + lane;
+    sm.p[w0 + j][lane] = x < n ? __ldg(parent + x) : INT_MAX;
   }
-  if (threadIdx.x == 0) *a.done = 0;
+  if (rows > 1) {
+#pragma unroll
+    for (int j = 0; j < 32; j++) {
+      const int64_t x = (g0 + kRmqGroups + w0 + j) * 32 + lane;
+      halo[j] = x < n ? __ldg(parent + x) : INT_MAX;
+    }
+#pragma unroll
+    for (int j = 0; j < 32; j++) {
+      const int32_t m = __reduce_min_sync(0xffffffffu, halo[j]);
+      if (lane == j) sm.row[0][kRmqGroups + w0 + j] = m;
+    }
+  }
+  __syncwarp();
+  {
+    int32_t v[32];
+#pragma unroll
+    for (int k = 0; k < 32; k++) v[k] = sm.p[w0 + lane][k];
+    uint32_t mk = 0;
+#pragma unroll
+    for (int k = 0; k < 32; k++) {
+      uint32_t below = 0;
+#pragma unroll
+      for (int j = 0; j < k; j++) below |= (v[j] < v[k] ? 1u : 0u) << j;
+      mk = (mk & below) | (1u << k);
+      sm.m[w0 + lane][k] = mk;
+    }
+  }
+  __syncwarp();
+#pragma unroll 4
+  for (int j = 0; j < 32; j++) {
+    const int64_t x = (g0 + w0 + j) * 32 + lane;
+    const int32_t p = sm.p[w0 + j][lane];
+    int32_t pre = p, suf = p;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t a = __shfl_up_sync(0xffffffffu, pre, o), b = __shfl_down_sync(0xffffffffu, suf, o);
+      if (lane >= o) pre = min(pre, a);
+      if (lane + o < 32) suf = min(suf, b);
+    }
+    const int32_t after = __shfl_down_sync(0xffffffffu, suf, 1);  // the entries after this one
+    if (x < n) rec[2 * x + 1] = make_int4(pre, lane < 31 ? after : INT_MAX, (int)sm.m[w0 + j][lane], p);
+    if (lane == 31) sm.row[0][w0 + j] = pre;
+  }
+  __syncthreads();
+  int cur = 0;
+  for (int t = 0; t < rows && t <= kRmqRow0; t++) {
+    if (t > 0) {
+      const int o = 1 << (t - 1);
+      for (int i = threadIdx.x; i < 2 * kRmqGroups; i += kRmqThreads)
+        sm.row[cur ^ 1][i] = min(sm.row[cur][i], i + o < 2 * kRmqGroups ? sm.row[cur][i + o] : INT_MAX);
+      cur ^= 1;
+      __syncthreads();
+    }
+    const int64_t g = g0 + threadIdx.x;
+    if (g < n1) table[(int64_t)t * n1 + g] = sm.row[cur][threadIdx.x];
+  }
+}
+
+// Rows t0 + 1 .. t0 + kRmqStep of the sparse table from row t0: row t0 + s at i
+// is the minimum of row t0 at i, i + 2^t0, .. (2^s of them), so each further
+// row adds coalesced loads of row t0 to the minimum of the row before.
+constexpr int kRmqStep = 5;
+
+__global__ void __launch_bounds__(kBlock) k_rmq_rows(int32_t* __restrict__ table, int64_t n1, int t0, int rows) {
+  dep_sync();
+  const int32_t* base = table + (int64_t)t0 * n1;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n1; i += (int64_t)gridDim.x * blockDim.x) {
+    int32_t m = base[i];
+#pragma unroll
+    for (int s = 1; s <= kRmqStep; s++) {
+      if (t0 + s >= rows) break;
+#pragma unroll
+      for (int j = 1 << (s - 1); j < 1 << s; j++) {
+        const int64_t k = i + ((int64_t)j << t0);
+        if (k < n1) m = min(m, base[k]);
+      }
+      table[(int64_t)(t0 + s) * n1 + i] = m;
+    }
+  }
 }
 
 }  // namespace
@@ -389,7 +313,7 @@ __global__ void __launch_bounds__(kRmqThreads, 2) k_rmq_build(RmqArgs a) {
 // stream capture; thread-safe initialisation)
 static cudaError_t rmq_smem_attr() {
   static const cudaError_t e =
-      cudaFuncSetAttribute(k_rmq_build, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RmqSmem));
+      cudaFuncSetAttribute(k_rmq_groups, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RmqSmem));
   return e;
 }
 
@@ -398,43 +322,31 @@ int step_tree(Handle& h) {
   while ((1ll << dep_bits) <= h.max_depth) dep_bits++;
   if (h.A > 0) {
     const int64_t tiles = (h.A + kTsTile - 1) / kTsTile;
-    TreeScanArgs a{h.tour, h.A, h.rtree, h.parent, dep_bits, h.dsc, h.P, h.rmq_val[0], h.ts_sum};
+    TreeScanArgs a{h.tour, h.A, h.rtree, dep_bits, h.dsc, static_cast<u128*>(h.rec), h.ts_sum};
     ++h.launches;
     launch_k(h, k_tree_sum, (int)tiles, kTsThreads, 0, a);
     ++h.launches;
     launch_k(h, k_tree_scan, (int)tiles, kTsThreads, 0, a);
     PDG_CUDA(cudaGetLastError());
   }
-  // the range-minimum structure over val0
-  RmqArgs r{};
-  for (int j = 0; j < h.rmq_levels; j++) {
-    r.val[j] = h.rmq_val[j];
-    r.mask[j] = h.rmq_mask[j];
-    r.pmin[j] = h.rmq_pmin[j];
-    r.smin[j] = h.rmq_smin[j];
-    r.size[j] = h.rmq_size[j];
-  }
-  r.levels = h.rmq_levels;
-  r.st = h.rmq_st;
-  r.st_rows = h.rmq_st_rows;
-  r.done = h.ts_done;
   PDG_CUDA(rmq_smem_attr());
+  const int64_t n1 = (h.n + 31) / 32;
   ++h.launches;
-  launch_k(h, k_rmq_build, (int)((h.rmq_size[0] + kRmqChunk - 1) / kRmqChunk), kRmqThreads, sizeof(RmqSmem), r);
+  launch_k(h, k_rmq_groups, (int)((n1 + kRmqGroups - 1) / kRmqGroups), kRmqThreads, sizeof(RmqSmem), h.parent, h.n, n1,
+           static_cast<int4*>(h.rec), h.rmq_table, h.rmq_rows);
+  for (int t0 = kRmqRow0; t0 + 1 < h.rmq_rows; t0 += kRmqStep) {
+    ++h.launches;
+    launch_k(h, k_rmq_rows, grid_for(h, n1), kBlock, 0, h.rmq_table, n1, t0, h.rmq_rows);
+  }
   PDG_CUDA(cudaGetLastError());
   return PDG_OK;
 }
 
-// the tree-scan work space for a tour of A arcs (tile sums) and the range-minimum build's block counter
+// the tree scan's work space for a tour of A arcs (tile sums)
 int tree_scan_workspace(Handle& h) {
   PDG_CUDA(rmq_smem_attr());
   const int64_t tiles = std::max<int64_t>((h.A + kTsTile - 1) / kTsTile, 1);
-  int st;
-  if ((st = device_alloc(h, (void**)&h.ts_sum, sizeof(u128) * (size_t)tiles)) ||
-      (st = device_alloc(h, (void**)&h.ts_done, sizeof(uint32_t))))
-    return st;
-  PDG_CUDA(cudaMemsetAsync(h.ts_done, 0, sizeof(uint32_t), h.stream));
-  return PDG_OK;
+  return device_alloc(h, (void**)&h.ts_sum, sizeof(u128) * (size_t)tiles);
 }
 
 }  // namespace pdg
