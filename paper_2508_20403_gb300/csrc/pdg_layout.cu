@@ -59,10 +59,15 @@ __global__ void k_lay_cut(const int32_t* __restrict__ parent, const int64_t* __r
 // (down), ~x otherwise (up, leaving x); dflag marks the down arcs.
 // List ranking by pointer jumping on one packed word per arc, (successor << 32) | arcs to the end: one
 // gather per arc and round instead of two.
-__global__ void k_lay_pack(const int32_t* __restrict__ succ, const int32_t* __restrict__ rd, int64_t A,
-                           uint64_t* __restrict__ out) {
+// Parent links that hold a 2-cycle have fewer distinct edges than a tree: the
+// arrays' last arcs then do not exist, nothing may follow them, and the tree is bad.
+__global__ void k_lay_pack(const int32_t* __restrict__ succ, const int32_t* __restrict__ rd,
+                           const int64_t* __restrict__ tptr, int64_t n, int64_t A, uint64_t* __restrict__ out,
+                           int32_t* __restrict__ bad) {
+  const int64_t arcs = tptr[n];
+  if (arcs != A && blockIdx.x == 0 && threadIdx.x == 0) *bad = 1;
   for (int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; a < A; a += (int64_t)gridDim.x * blockDim.x)
-    out[a] = ((uint64_t)(uint32_t)succ[a] << 32) | (uint32_t)rd[a];
+    out[a] = a < arcs ? ((uint64_t)(uint32_t)succ[a] << 32) | (uint32_t)rd[a] : 0xffffffff00000000ull;
 }
 
 __global__ void k_lay_rank(const uint64_t* __restrict__ in, uint64_t* __restrict__ out, int64_t A) {
@@ -246,7 +251,10 @@ int build_tree_layout(Handle& h) {
   } while (0)
   LAY_CK(cudaMemsetAsync(bad, 0, sizeof(int32_t), s));
   LAY_CK(cudaMemsetAsync(pre_of, 0xff, sizeof(int32_t) * n, s));  // -1: not reached
-  if (A > 0) LAY_CK(cudaMemsetAsync(h.tour, 0xff, sizeof(int32_t) * A, s));
+  if (A > 0) {  // positions that the arcs of a bad tree leave open
+    LAY_CK(cudaMemsetAsync(h.tour, 0xff, sizeof(int32_t) * A, s));
+    LAY_CK(cudaMemsetAsync(dflag, 0, sizeof(int32_t) * A, s));
+  }
   LAY_CK(cudaMemsetAsync(tdeg, 0, sizeof(int32_t) * n, s));
   LAY_CK(cudaMemsetAsync(cur, 0, sizeof(int32_t) * n, s));
   if (m > 0) {
@@ -260,7 +268,7 @@ int build_tree_layout(Handle& h) {
     k_tour_fix_rev<<<gn, kBlock, 0, s>>>(tptr, tadj, n, rev);
     k_st_succ<<<ga, kBlock, 0, s>>>(tadj, rev, tptr, tdeg, n, succ, rd);
     k_lay_cut<<<gn, kBlock, 0, s>>>(h.parent, tptr, tdeg, rev, n, succ, rd);
-    k_lay_pack<<<ga, kBlock, 0, s>>>(succ, rd, A, ranked[0]);
+    k_lay_pack<<<ga, kBlock, 0, s>>>(succ, rd, tptr, n, A, ranked[0], bad);
     int bits = 1;
     while ((1ll << bits) <= A) bits++;
     int c = 0;
