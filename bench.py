@@ -220,26 +220,26 @@ def step_bytes(n, nnz, E, G, R, k):
     once, gathers at element size), per recovery."""
     A = 2 * (n - G)  # Euler-tour arcs
     return {
-        # stream the canonical edge list (u, v: 4 B, w: 8 B), gather parent, write r(v) and the off-tree SoA
-        "classify": 16 * (nnz // 2) + 4 * n + 8 * n + 20 * E,
-        # two passes over the tour (arc 4 B + r gather 8 B); write P (16 B) and the range-minimum key (8 B),
-        # read parent (4 B); the range-minimum build reads the keys (8 B) and writes the masks (4 B)
-        "tree": 2 * 12 * A + 28 * n + 12 * n,
-        # read (u, v, w) 16 B, gather P(u), P(v), P(LCA) 48 B, write key + lca 12 B
-        "score": 76 * E,
-        # two histogram passes + one compaction pass over the keys, write candidates (idx, key, val)
-        "select": 24 * E + 16 * R,
-        # 8 score digits + 3 LCA digits, each: read key+val 12 B, write 12 B
-        "sort": 11 * 24 * R,
-        # records (~44 B written + read), tier lists
-        "accept": 100 * R,
+        # the tree's weights in label order in, r(v) out
+        "classify": 16 * n,
+        # two passes over the tour (arc 4 B + r gather 8 B); write P (16 B); the range-minimum build reads the
+        # parents (4 B) and writes the other half of the records (16 B)
+        "tree": 2 * 12 * A + 36 * n,
+        # read (u, v, w) 16 B and write key + lca 12 B per edge; gather P(u), P(v), P(LCA) 48 B per off-tree edge
+        "score": 28 * (nnz // 2) + 48 * E,
+        # one pass over the keys, write candidates (record, key, val, id)
+        "select": 8 * (nnz // 2) + 48 * R,
+        # 8 score digits, each: read key+val 12 B, write 12 B
+        "sort": 8 * 24 * R,
+        # the join: records and probes (64 B written + read), a cell (32 B) entered and five read
+        "accept": 320 * R,
         "budget": 8 * R + 12 * k,
     }
 
 
 # the longest single launch of a recovery: step A3 is one kernel, k_score
 DOMINANT_KERNEL = "k_score"
-SCORE_BYTES_PER_EDGE = 76  # read u, v (8 B), w (8 B); gather P(u), P(v), P(lca) (48 B); write key, lca (12 B)
+SCORE_BYTES_PER_EDGE = 76  # off-tree edge: read u, v (8 B), w (8 B); gather P(u), P(v), P(lca) (48 B); write key, lca (12 B)
 
 
 def path_bytes(n, m, E, k):

@@ -1084,7 +1084,7 @@ int step_accept(Handle& h, int c) {
   const int64_t cap = h.Rcap;
   int st;
   ++h.launches;
-  launch_k(h, k_build_records, grid, kBlock, 0, h.lsort_rank, h.rank_cand, h.cand_idx, h.off_u, h.off_v, h.lca,
+  launch_k(h, k_build_records, grid, kBlock, 0, h.lsort_rank, h.rank_cand, h.cand_idx, h.el_u, h.el_v, h.lca,
            static_cast<const int4*>(h.up), h.parent, c, h.dsc, cap, h.rec_u, h.rec_v, h.rec_anc,
            h.rec_du, h.rec_dv, h.rec_b, h.rec_rank, h.rec_lca);
   // subtask boundaries, tier lists, per-position tiers

@@ -138,6 +138,7 @@ __global__ void k_reset_attempt(DevScalars* dsc, uint4* __restrict__ tab, int64_
   dsc->bounds_site = 0;
   dsc->rounds_used = 0;
   dsc->n_cand = 0;
+  dsc->n_list = 0;
   dsc->n_seg = 0;
   dsc->n_warp_seg = 0;
   dsc->n_block_seg = 0;
@@ -225,7 +226,22 @@ int ensure_candidates(Handle& h, int64_t R, int c) {
     if ((st = grow_join(h))) return st;
   }
   if ((st = ensure_scan_status(h, h.Rcap + 1))) return st;
+  // the selection's list: a power of two of the scores, usually a few times the candidates
+  if (h.list_cap < std::min<int64_t>(Rmax, 4 * h.Rcap) && (st = grow_list(h, 4 * h.Rcap))) return st;
   return h.tiered ? ensure_tiers(h, c) : PDG_OK;
+}
+
+int grow_list(Handle& h, int64_t entries) {
+  entries = std::min<int64_t>(entries, std::max<int64_t>(h.E_off, 1));
+  device_release(h, h.list_id);
+  device_release(h, h.list_key);
+  h.list_id = nullptr;
+  h.list_key = nullptr;
+  h.list_cap = 0;
+  int st;
+  if ((st = alloc_n(h, &h.list_id, entries)) || (st = alloc_n(h, &h.list_key, entries))) return st;
+  h.list_cap = entries;
+  return PDG_OK;
 }
 
 // the join's cell table: join_factor slots per candidate of the capacity
@@ -473,7 +489,6 @@ int sparsify_batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_
       cudaMemcpyAsync(h.d_vtx_ptr, vtx_ptr, sizeof(int64_t) * (num_graphs + 1), cudaMemcpyHostToDevice, h.stream) !=
           cudaSuccess)
     return fail(PDG_E_CUDA);
-  h.nblk = (int)std::max<int64_t>(1, std::min<int64_t>(2048, (h.m + kTile - 1) / kTile));
   if ((st = validate_graph(h, false))) return fail(st);  // acyclicity, depth and range: build_tree_layout
   // per-graph edge counts from the row offsets at the graph boundaries
   std::vector<int64_t> rp_at(num_graphs + 1);
@@ -510,23 +525,21 @@ int sparsify_batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_
   }
   h.E_off = h.off_ptr_h[num_graphs];
   // workspace
-  const int64_t E = std::max<int64_t>(h.E_off, 1);
   if ((st = alloc_n(h, &h.d_edge_ptr, num_graphs + 1)) || (st = alloc_n(h, &h.d_off_ptr, num_graphs + 1)) ||
-      (st = alloc_n(h, &h.off_u, E)) || (st = alloc_n(h, &h.off_v, E)) || (st = alloc_n(h, &h.off_id, E)) ||
-      (st = alloc_n(h, &h.off_w, E)) || (st = alloc_n(h, &h.rtree, n)) ||
-      (st = alloc_n(h, &h.key, E)) || (st = alloc_n(h, &h.lca, E)) ||
+      (st = alloc_n(h, &h.rtree, n)) || (st = alloc_n(h, &h.key, h.m)) || (st = alloc_n(h, &h.lca, h.m)) ||
       (st = alloc_n(h, &h.hist, (int64_t)num_graphs * kSelBins)) || (st = alloc_n(h, &h.sel, num_graphs)) ||
-      (st = alloc_n(h, &h.d_cand_ptr, num_graphs + 1)) || (st = alloc_n(h, &h.d_graph_tmp, num_graphs + 1)) ||
+      (st = alloc_n(h, &h.d_cand_ptr, num_graphs + 1)) ||
+      (st = device_alloc(h, &h.list_tile, sizeof(int2) * (size_t)select_tiles(h.m))) || (st = alloc_n(h, &h.d_graph_tmp, num_graphs + 1)) ||
       (st = alloc_n(h, &h.gstat, num_graphs)) || (st = alloc_n(h, &h.gcount, num_graphs)) ||
       (st = alloc_n(h, &h.lca_count, n)) ||
       (st = device_alloc(h, &h.join_part, (size_t)h.num_sms * 8 * (sizeof(int4) + sizeof(int32_t)))) ||
       (st = alloc_n(h, &h.d_k, num_graphs)) || (st = alloc_n(h, &h.d_out_ptr, num_graphs + 1)) ||
       (st = alloc_n(h, &h.radix_dtot, 256)) || (st = alloc_n(h, &h.radix_hist, kRadixHistWords)) ||
       (st = alloc_n(h, &h.radix_counters, 2 * kRadixPassesMax)) ||
-      (st = ensure_scan_status(h, std::max<int64_t>(std::max<int64_t>(n, num_graphs), E) + 1)))
+      (st = ensure_scan_status(h, std::max<int64_t>(n, num_graphs) + 1)))
     return fail(st);
-  // the tree's layout: preorder labels, Euler tour, the relabelled edge list and parents
-  if ((st = build_tree_layout(h)) || (st = tree_scan_workspace(h)) || (st = classify_layout(h))) return fail(st);
+  // the tree's layout: preorder labels, Euler tour, the relabelled edge list, parents and tree weights
+  if ((st = build_tree_layout(h)) || (st = tree_scan_workspace(h))) return fail(st);
   HostStage& s = hp->stage;
   s.G = num_graphs;
   s.sel = static_cast<GraphSel*>(pinned_alloc(sizeof(GraphSel) * num_graphs));
@@ -837,7 +850,7 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
       mark(0);
       ++h.launches;
       launch_k(h, k_reset_recover, 1, 1, 0, h.dsc);
-      if ((e = step_classify(h))) return e;
+      if ((e = step_resist(h))) return e;
       mark(1);
       if ((e = step_tree(h))) return e;
       mark(2);
@@ -893,7 +906,7 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
     if ((st = ensure_candidates(h, std::max<int64_t>(h.Rcap, need + need / 4 + 4096), c))) return st;
     // the launch sequence a CUDA graph bakes in
     const GraphKey key{c, h.opt.score_mode, any_select ? 1 : 0, h.tiered ? coop_rounds(h, c) : 0, h.Rcap, h.table_cap, h.xcap,
-                       h.join_slots, h.tiered, (void*)dev_ids, (void*)dev_scores, out_total};
+                       h.join_slots, h.list_cap, h.tiered, (void*)dev_ids, (void*)dev_scores, out_total};
     bool replayed = false;
     if (first && h.opt.use_graph && h.gexec && key == h.gkey) {
       // replay on the private stream, ordered after the caller's stream
@@ -953,6 +966,11 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
       return PDG_E_CUDA;
     }
     if (err & ERR_CAPACITY) {
+      if (h.hsc->n_list > h.list_cap) {  // the boundary bucket outgrew the list
+        if ((st = grow_list(h, h.hsc->n_list + h.hsc->n_list / 8))) return st;
+        first = false;
+        continue;
+      }
       const int64_t wanted = h.hsc->n_cand_wanted;
       if (wanted <= h.Rcap) return PDG_E_CUDA;  // inconsistent selection
       if ((st = ensure_candidates(h, wanted + wanted / 8 + 4096, c))) return st;

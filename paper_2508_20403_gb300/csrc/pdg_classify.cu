@@ -1,22 +1,21 @@
 // Step A1: split the edges of G into tree and off-tree edges (Sec. 2.2: every
-// edge of G is either a tree edge or an off-tree edge) and compact the
-// off-tree edges, in canonical id order, into structure-of-arrays form.
+// edge of G is either a tree edge or an off-tree edge).
 //
 // Canonical id of {u, v}, u < v: rank of the CSR entry (u, v) among all
 // entries with row < col in row-major order.  The handle keeps the graph as
 // its canonical edge list (id order; built once from the CSR by
 // build_edge_list at init, endpoints then relabelled in the tree's preorder
-// as (a, b), a < b), so every recovery classifies by streaming that list: a
-// parent's label is below its child's, so edge (a, b) is a tree edge iff
-// parent[b] == a.  The write pass also records, for every non-root vertex x,
-// r(x) = fl(1/w(x, parent x)) (the resistive weight W_re = 1/w of Eq. RT),
-// computed on the integer pipes (pdg_fp.cuh), and the exponent range of these
-// r that fixes the fixed-point scale of step A2.
+// as (a, b), a < b): a parent's label is below its child's, so edge (a, b) is a
+// tree edge iff parent[b] == a.  Recoveries make that test where the edge is
+// scored: the record gathered for b holds its parent, so telling the edges
+// apart costs nothing there, and no off-tree list is written and read again
+// (compacting one took 0.068 of 0.45 ms on mesh 128^3, 0.63 of 2.05 ms on
+// R-MAT scale 22).  What is left of the step is k_resist.
 //
-// Layout: each block owns a contiguous chunk of edges (CSR entries for the
-// edge-list build), taken in tiles of kTile; each thread reads kItems
-// consecutive items with vector loads.  Two passes: a count pass, then a
-// write pass that places each tile's output as one contiguous run.
+// Edge-list layout: each block owns a contiguous chunk of CSR entries, taken in
+// tiles of kTile; each thread reads kItems consecutive entries with vector
+// loads.  Two passes: a count pass, then a write pass that places each tile's
+// output as one contiguous run.
 #include <climits>
 
 #include "pdg_fp.cuh"
@@ -184,134 +183,63 @@ __global__ void __launch_bounds__(kBlock) k_edge_list(const int64_t* __restrict_
   }
 }
 
-// Recovery-time classification of the canonical edge list.  Count pass:
-// off-tree edges per block.  Write pass: r(x) for the tree edges (queued per
-// warp so the reciprocals run densely, every lane on a tree edge) and the
-// off-tree SoA, staged per tile and written as one coalesced run.
-template <bool WRITE>
-__global__ void __launch_bounds__(kBlock) k_classify(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
-                                                     const double* __restrict__ ew,
-                                                     const int32_t* __restrict__ parent, int64_t m,
-                                                     int64_t* __restrict__ cnt_off,
-                                                     const int64_t* __restrict__ off_off,
-                                                     double* __restrict__ rtree, int32_t* __restrict__ ou,
-                                                     int32_t* __restrict__ ov, int32_t* __restrict__ oid,
-                                                     double* __restrict__ ow, DevScalars* __restrict__ dsc) {
+// Recovery, tree edges: r(x) = fl(1/w(x, parent x)) of every label from the
+// tree's weights in label order, and the exponent range of these r (it fixes
+// the fixed-point scale of step A2).  One stream in, one out; the off-tree
+// edges are told apart where they are scored.
+__global__ void __launch_bounds__(kBlock) k_resist(const double* __restrict__ wup, int64_t n, double* __restrict__ rtree,
+                                                   DevScalars* __restrict__ dsc) {
   dep_sync();
-  __shared__ int64_t sm[kBlock / 32 + 1];
-  // write pass: per-warp queue of (child, weight) for the reciprocals, then
-  // the tile's off-tree records (a tile holds at most kTile entries of each)
-  __shared__ double st_w[WRITE ? kTile : 1];
-  __shared__ int32_t st_u[WRITE ? kTile : 1], st_v[WRITE ? kTile : 1], st_id[WRITE ? kTile : 1];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t chunk = cls_chunk(m, gridDim.x);
-  const int64_t b0 = (int64_t)blockIdx.x * chunk;
-  const int64_t b1 = min(m, b0 + chunk);
-  int64_t run_off = WRITE ? off_off[blockIdx.x] : 0;
-  int64_t tot_off = 0;
-  int e_lo = INT_MAX, e_hi = INT_MIN;  // exponent range of the r(x) this thread writes
-  for (int64_t t0 = b0; t0 < b1; t0 += kTile) {
-    const int64_t base = t0 + (int64_t)threadIdx.x * kItems;
-    int32_t a[kItems], b[kItems], child[kItems];
-    double x[kItems];
-    uint32_t is_off = 0, is_tree = 0;
-    if (base < b1) {
-      load_cols(eu, base, b1, a);
-      load_cols(ev, base, b1, b);
-      if (WRITE) load_weights(ew, base, b1, x);
-      int32_t pb[kItems];
+  __shared__ int s_lo, s_hi;
+  if (threadIdx.x == 0) {
+    s_lo = INT_MAX;
+    s_hi = INT_MIN;
+  }
+  __syncthreads();
+  int e_lo = INT_MAX, e_hi = INT_MIN;
+  // four labels per thread: their loads, then their reciprocals, overlap
+  for (int64_t x = ((int64_t)blockIdx.x * kBlock + threadIdx.x) * 4; x < n; x += (int64_t)gridDim.x * kBlock * 4) {
+    double w[4], r[4];
+    if (x + 4 <= n) {
+      const double2 a = __ldg(reinterpret_cast<const double2*>(wup + x)), b = __ldg(reinterpret_cast<const double2*>(wup + x) + 1);
+      w[0] = a.x;
+      w[1] = a.y;
+      w[2] = b.x;
+      w[3] = b.y;
+    } else {
 #pragma unroll
-      for (int i = 0; i < kItems; i++) pb[i] = (base + i < b1) ? __ldg(parent + b[i]) : -1;
-#pragma unroll
-      for (int i = 0; i < kItems; i++) {
-        if (base + i >= b1) continue;
-        if (pb[i] == a[i]) {
-          is_tree |= 1u << i;
-          child[i] = b[i];
-        } else {
-          is_off |= 1u << i;
-        }
-      }
+      for (int i = 0; i < 4; i++) w[i] = x + i < n ? __ldg(wup + x + i) : 0.0;
     }
-    const int64_t n_off = __popc(is_off);
-    if (!WRITE) {
-      tot_off += n_off;
-      continue;
-    }
-    {
-      const int ntree = __popc(is_tree);
-      const int incl = warp_incl_scan(ntree);
-      int slot = wid * (kTile / (kBlock / 32)) + incl - ntree;
 #pragma unroll
-      for (int i = 0; i < kItems; i++) {
-        if (is_tree & (1u << i)) {
-          st_u[slot] = child[i];
-          st_w[slot] = x[i];
-          slot++;
-        }
-      }
-      __syncwarp();
-      const int tot = __shfl_sync(0xffffffffu, incl, 31);
-      for (int j = lane; j < tot; j += 32) {
-        const int q = wid * (kTile / (kBlock / 32)) + j;
-        const double wq = st_w[q];
-        bool ok;
-        const uint64_t rb = rcp_rn_bits((uint64_t)__double_as_longlong(wq), &ok);
-        const double r = ok ? __longlong_as_double((long long)rb) : __drcp_rn(wq);
-        rtree[st_u[q]] = r;
-        const int e = (int)(((uint64_t)__double_as_longlong(r) >> 52) & 0x7ff) - 1023;
+    for (int i = 0; i < 4; i++) {
+      bool ok;
+      const uint64_t rb = rcp_rn_bits((uint64_t)__double_as_longlong(w[i]), &ok);
+      r[i] = w[i] == 0.0 ? 0.0 : ok ? __longlong_as_double((long long)rb) : __drcp_rn(w[i]);  // 0: a root
+      if (w[i] != 0.0) {
+        const int e = (int)(((uint64_t)__double_as_longlong(r[i]) >> 52) & 0x7ff) - 1023;
         e_lo = min(e_lo, e);
         e_hi = max(e_hi, e);
       }
     }
-    int64_t tile_tot;
-    int lpos = (int)block_excl_scan(n_off, sm, &tile_tot);  // also orders the queue reads
-    // stage the tile's off-tree records in shared memory ...
+    if (x + 4 <= n) {
+      reinterpret_cast<double2*>(rtree + x)[0] = make_double2(r[0], r[1]);
+      reinterpret_cast<double2*>(rtree + x)[1] = make_double2(r[2], r[3]);
+    } else {
 #pragma unroll
-    for (int i = 0; i < kItems; i++) {
-      if (is_off & (1u << i)) {
-        st_u[lpos] = a[i];
-        st_v[lpos] = b[i];
-        st_id[lpos] = (int32_t)(base + i);
-        st_w[lpos] = x[i];
-        lpos++;
-      }
+      for (int i = 0; i < 4; i++)
+        if (x + i < n) rtree[x + i] = r[i];
     }
-    __syncthreads();
-    // ... and write them out as one contiguous, coalesced run
-    const int cnt = (int)tile_tot;
-    for (int j = threadIdx.x; j < cnt; j += kBlock) {
-      ou[run_off + j] = st_u[j];
-      ov[run_off + j] = st_v[j];
-      oid[run_off + j] = st_id[j];
-      ow[run_off + j] = st_w[j];
-    }
-    run_off += tile_tot;
-    __syncthreads();
   }
-  if (!WRITE) {
-    tot_off = block_sum(tot_off, sm);
-    if (threadIdx.x == 0) cnt_off[blockIdx.x] = tot_off;
-  } else {
-    // the exponent range of r over the tree (it fixes the fixed-point scale of
-    // step A2): one atomic pair per block
-    e_lo = __reduce_min_sync(0xffffffffu, e_lo);
-    e_hi = __reduce_max_sync(0xffffffffu, e_hi);
-    __shared__ int s_lo, s_hi;
-    if (threadIdx.x == 0) {
-      s_lo = INT_MAX;
-      s_hi = INT_MIN;
-    }
-    __syncthreads();
-    if (lane == 0) {
-      atomicMin(&s_lo, e_lo);
-      atomicMax(&s_hi, e_hi);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      if (s_lo != INT_MAX) atomicMin(&dsc->e_min, s_lo);
-      if (s_hi != INT_MIN) atomicMax(&dsc->e_max, s_hi);
-    }
+  e_lo = __reduce_min_sync(0xffffffffu, e_lo);
+  e_hi = __reduce_max_sync(0xffffffffu, e_hi);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&s_lo, e_lo);
+    atomicMax(&s_hi, e_hi);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (s_lo != INT_MAX) atomicMin(&dsc->e_min, s_lo);
+    if (s_hi != INT_MIN) atomicMax(&dsc->e_max, s_hi);
   }
 }
 
@@ -334,29 +262,10 @@ int build_edge_list(Handle& h) {
   return PDG_OK;
 }
 
-// Init: the number of off-tree edges in each block's chunk of the edge list is
-// a fact of the fixed tree, so the write offsets of the recovery's compaction
-// are counted once here (a count pass and a scan) and kept.
-int classify_layout(Handle& h) {
-  if (h.m == 0) return PDG_OK;
-  const int nb = h.nblk;
-  int st;
-  if ((st = device_alloc(h, (void**)&h.cls_off, sizeof(int64_t) * (size_t)(nb + 1)))) return st;
-  int64_t* cnt_off = h.blk_a;
+int step_resist(Handle& h) {
   ++h.launches;
-  launch_k(h, k_classify<false>, nb, kBlock, 0, h.el_u, h.el_v, h.el_w, h.parent, h.m, cnt_off, nullptr, nullptr,
-           nullptr, nullptr, nullptr, nullptr, h.dsc);
-  PDG_CUDA(cudaGetLastError());
-  return scan_excl_i64(h, cnt_off, h.cls_off, nb, nullptr, nb);
-}
-
-// Recovery: one pass classifies every edge, writes r(x) of the tree edges
-// and the off-tree records at the offsets counted at init.
-int step_classify(Handle& h) {
-  if (h.m == 0) return PDG_OK;
-  ++h.launches;
-  launch_k(h, k_classify<true>, h.nblk, kBlock, 0, h.el_u, h.el_v, h.el_w, h.parent, h.m, nullptr, h.cls_off,
-           h.rtree, h.off_u, h.off_v, h.off_id, h.off_w, h.dsc);
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)h.num_sms * 8, (h.n + 4 * kBlock - 1) / (4 * kBlock)));
+  launch_k(h, k_resist, grid, kBlock, 0, h.wup, h.n, h.rtree, h.dsc);
   PDG_CUDA(cudaGetLastError());
   return PDG_OK;
 }

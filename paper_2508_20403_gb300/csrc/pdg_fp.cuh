@@ -13,22 +13,21 @@
 // doubles); inputs outside the normal range of the fast path fall back to the
 // hardware operation.
 //
-//   reciprocal: Newton's iteration x <- x + x (1 - m x) for 1/m on the 53-bit
-//     significand m, started from the single-precision reciprocal of its top
-//     24 bits and run twice in 128-bit fixed point (each step squares the
-//     relative error: 2^-22 -> 2^-44 -> below one unit), then the exact
-//     quotient floor(2^105 / m) by comparing products, and the rounding bit
-//     from the remainder (no ties: 2^106 / m is never an odd integer for a
-//     significand that is not a power of two).
+//   reciprocal: one step of Newton's iteration x <- x + x (1 - m x) for 1/m on
+//     the 53-bit significand m, from the single-precision reciprocal of its top
+//     bits (2^-22 -> 2^-44 relative), then the exact quotient floor(2^105 / m)
+//     from the remainder, and the rounding bit from what remains (no ties:
+//     2^106 / m is never an odd integer for a significand that is not a power
+//     of two).  Five 64-bit products; the earlier form, two steps in 128-bit
+//     fixed point, took 26 us of a recovery on 2.1 M tree edges.
 //   fixed point to FP64: the leading bit of the integer fixes the exponent;
 //     the 53 bits below it, rounded by the remainder, the significand.
 #pragma once
 
 #include <stdint.h>
+#include <string.h>
 
 namespace pdg {
-
-typedef unsigned __int128 u128;
 
 #ifdef __CUDACC__
 #define PDG_HD __host__ __device__ __forceinline__
@@ -46,48 +45,53 @@ PDG_HD int clz64(uint64_t x) {
 #endif
 }
 
-PDG_HD float rcp_f32(float f) {
+// bits of 1/f to 2^-23 relative, for the bits of a float f in [1, 2)
+PDG_HD uint32_t rcp_f32_bits(uint32_t f) {
 #ifdef __CUDA_ARCH__
-  return __frcp_rn(f);
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint_as_float(f)));
+  return __float_as_uint(y);
 #else
-  return 1.0f / f;
+  float x;
+  memcpy(&x, &f, 4);
+  x = 1.0f / x;
+  memcpy(&f, &x, 4);
+  return f;
 #endif
 }
 
 // round(2^105 / m) for a significand 2^52 < m < 2^53; *ok is false if the
 // bounded correction did not settle (it always does; the caller then falls
-// back to a hardware division)
+// back to a hardware division).  Residuals are taken modulo 2^64: each is known
+// to be far smaller, so the low words of the products are enough.
 PDG_HD uint64_t rcp_significand(uint64_t m, bool* ok) {
-  const u128 two105 = (u128)1 << 105;
-  // 2^29 / m to about 2^-22 relative, as 2^105 / m in fixed point
-  const float y = rcp_f32((float)(uint32_t)(m >> 29));
-  uint64_t x = (uint64_t)(y * 0x1p76f);  // y * 2^76, truncated
-#pragma unroll
-  for (int it = 0; it < 2; it++) {
-    const u128 mx = (u128)m * x;
-    const bool above = mx > two105;
-    const u128 e = above ? mx - two105 : two105 - mx;  // |2^105 - m x| < 2^86
-    const u128 t = (u128)(uint64_t)(e >> 33) * x;        // e x / 2^33
-    const uint64_t c = (uint64_t)(t >> 72);              // e x / 2^105
-    x = above ? x - c : x + c;
-  }
-  u128 mx = (u128)m * x;
+  // X = 2^84 / m as a 32-bit integer, to 2^-22 relative: the bits of a single-precision reciprocal of m's top 24
+  // bits, built and taken apart without conversions (they run on a slow unit)
+  const uint32_t y = rcp_f32_bits(0x3f800000u | ((uint32_t)(m >> 29) & 0x7fffffu));  // of [1, 2): in (1/2, 1]
+  const uint32_t x = y >= 0x3f800000u ? 0xffffffffu : (y << 8) | 0x80000000u;
+  // 2^105 / m = 2^21 (X + r / m) with r = 2^84 - m X, |r| <= 2^62, and r / m ~ r X / 2^84
+  const int64_t r = (int64_t)(0 - m * (uint64_t)x);
+  uint64_t q = ((uint64_t)x << 21) + (uint64_t)(((r >> 31) * (int64_t)(uint64_t)x) >> 32);
+  // q is within a few hundred units now: the remainder fits 64 bits, and gives the rest
+  int64_t rem = (int64_t)(0 - m * q);
+  const int64_t d = ((rem >> 32) * (int64_t)(uint64_t)x) >> 52;
+  q += (uint64_t)d;
+  rem -= d * (int64_t)m;
   bool settled = false;
-  for (int k = 0; k < 8; k++) {  // x = floor(2^105 / m): m x <= 2^105 < m (x + 1)
-    if (mx > two105) {
-      x--;
-      mx -= m;
-    } else if (two105 - mx >= m) {
-      x++;
-      mx += m;
+  for (int k = 0; k < 4; k++) {  // q = floor(2^105 / m): 0 <= rem < m
+    if (rem < 0) {
+      q--;
+      rem += (int64_t)m;
+    } else if (rem >= (int64_t)m) {
+      q++;
+      rem -= (int64_t)m;
     } else {
       settled = true;
       break;
     }
   }
   *ok = settled;
-  const uint64_t rem = (uint64_t)(two105 - mx);
-  return (rem > m - rem) ? x + 1 : x;  // 2 rem > m: round up
+  return ((uint64_t)rem > m - (uint64_t)rem) ? q + 1 : q;  // 2 rem > m: round up
 }
 
 // IEEE bits of fl(1/w) for positive normal w whose reciprocal is normal;

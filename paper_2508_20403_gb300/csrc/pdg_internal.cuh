@@ -17,6 +17,7 @@ typedef unsigned __int128 u128;
 constexpr int kBlock = 256;         // threads per block for streaming kernels
 constexpr int kItems = 8;           // items per thread in blocked tiles
 constexpr int kTile = kBlock * kItems;
+constexpr int kSelRunsMax = 9000;   // blocks of the candidate selection (their counts lie in blk_a)
 constexpr int kSelBins = 4096;      // 12-bit digits of the candidate selection
 constexpr int kRadixPassesMax = 16; // 8 score digits + <= 4 graph digits + <= 4 LCA digits
 // Block tier: one block per subtask of warp_tier_max+1 .. block_tier_max
@@ -91,6 +92,7 @@ struct DevScalars {
   int64_t radix_len;    // radix sort: histogram length (256 * tiles)
   int64_t n_warp_cand;  // candidates in the warp tier
   int64_t n_cand_wanted;  // candidates the selection produced (may exceed capacity)
+  int64_t n_list;         // selection: edges of the boundary bucket and above (may exceed the list's capacity)
   int64_t n_constrained;  // cooperative tier: candidates with a possible earlier marker
   int64_t n_big_chunk;    // cooperative tier: chunks of at most kBigChunk positions
   uint32_t epoch;       // attempts so far (tags the cooperative tier's undecided entries)
@@ -143,14 +145,14 @@ struct GraphSel {
 // reads at replay time (budgets, prefix sizes, output offsets).
 struct GraphKey {
   int c = -1, score_mode = -1, any_select = -1, rounds = -1;
-  int64_t Rcap = -1, table_cap = -1, xcap = -1, join_slots = -1;
+  int64_t Rcap = -1, table_cap = -1, xcap = -1, join_slots = -1, list_cap = -1;
   bool tiered = false;
   void* out_ids = nullptr;
   void* out_scores = nullptr;
   int64_t out_total = -1;
   bool operator==(const GraphKey& o) const {
     return c == o.c && score_mode == o.score_mode && any_select == o.any_select && rounds == o.rounds && Rcap == o.Rcap &&
-           table_cap == o.table_cap && xcap == o.xcap && join_slots == o.join_slots && tiered == o.tiered && out_ids == o.out_ids && out_scores == o.out_scores &&
+           table_cap == o.table_cap && xcap == o.xcap && join_slots == o.join_slots && list_cap == o.list_cap && tiered == o.tiered && out_ids == o.out_ids && out_scores == o.out_scores &&
            out_total == o.out_total;
   }
 };
@@ -181,21 +183,16 @@ struct Handle {
   int32_t* tour = nullptr;
   int64_t A = 0;
   int32_t* vtx_of_pre = nullptr;
+  double* wup = nullptr;  // per label: weight of the edge to the parent (0: a root)
   void* up = nullptr;  // int4 per label: parent, grandparent, great-grandparent (-1: none), depth
   int64_t* d_vtx_ptr = nullptr;
   int64_t* d_edge_ptr = nullptr;
   int64_t* d_off_ptr = nullptr;
 
   // step 1 outputs
-  int32_t* off_u = nullptr;
-  int32_t* off_v = nullptr;
-  int32_t* off_id = nullptr;
-  double* off_w = nullptr;
   double* rtree = nullptr;  // r(v) = fl(1/w(v, parent v))
   int64_t* blk_a = nullptr; // per-block counters (classification, scans)
-  int64_t* cls_off = nullptr;  // write offsets of the classification's block chunks (counted at init)
   int64_t* blk_b = nullptr;
-  int nblk = 0;
 
   // per label one 32-byte record: P(x) = D(x) * 2^32 + depth(x) (u128; D = exact root distance in units of
   // 2^-S), then of the parent array, inside the label's 32-label group: minimum up to it, minimum after it,
@@ -207,8 +204,9 @@ struct Handle {
   u128* ts_sum = nullptr;        // tree scan: tile sums
 
   // scores
-  uint64_t* key = nullptr;  // FP64 score bits (positive -> order preserving)
-  int32_t* lca = nullptr;   // preorder label of the LCA
+  // by canonical id: FP64 score bits + 1 (not negative -> order preserving), 0 for a tree edge
+  uint64_t* key = nullptr;
+  int32_t* lca = nullptr;  // preorder label of the LCA (off-tree edges)
 
   // selection
   uint32_t* hist = nullptr;  // G * kSelBins
@@ -231,6 +229,11 @@ struct Handle {
   // steps A5 + A6: false: the join; true: the tiers (this attempt's candidates fill the join's cells too much;
   // remembered for later recoveries with (c_mem, mode_mem))
   bool tiered = false;
+  // selection: the edges of the boundary bucket and above (grow-only)
+  int64_t list_cap = 0;
+  int32_t* list_id = nullptr;
+  uint64_t* list_key = nullptr;
+  void* list_tile = nullptr;  // int2 per tile of the edge list: its run in the list
   // candidate buffers (grow-only, capacity Rcap)
   int64_t Rcap = 0;
   // the join: records and probes by rank, cell table, candidates per LCA
@@ -249,7 +252,7 @@ struct Handle {
   int join_blocks = 0, join_pair_blocks = 0;
   // the tiers' buffers below are allocated when a recovery first needs them
   int64_t tier_cap = 0;
-  int32_t* cand_idx = nullptr;     // off-tree index of each candidate (id order within graph)
+  int32_t* cand_idx = nullptr;     // canonical id of each candidate (id order)
   uint64_t* rk[2] = {nullptr, nullptr};  // radix keys ping-pong
   int32_t* rv[2] = {nullptr, nullptr};   // radix values ping-pong
   int32_t* rank_cand = nullptr;    // rank -> candidate index
@@ -544,11 +547,11 @@ int validate_graph(Handle& h, bool acyclic);    // input checks; acyclic: also a
 int build_edge_list(Handle& h);                 // init: canonical edge list from the CSR
 int build_tree_layout(Handle& h);               // init: preorder labels, Euler tour, relabelled edges and parents
 int tree_scan_workspace(Handle& h);             // init: look-back space of the tree scan
-int classify_layout(Handle& h);                 // init: off-tree edges per classification chunk
-int step_classify(Handle& h);                   // A1
+int step_resist(Handle& h);                     // A1: r of the tree edges (off-tree edges: told apart in A3)
 int step_tree(Handle& h);                       // A2
 int step_score(Handle& h, int score_mode);      // A3
 int step_select(Handle& h);                     // A4a: candidate prefix per graph
+int64_t select_tiles(int64_t m);                // its tiles of the edge list
 int sort_setup();                               // per-device kernel attributes of the sort
 int accept_setup();                             // per-device kernel attributes of the block tier
 int coop_rounds(const Handle& h, int c);        // cooperative-tier rounds the next recovery launches
@@ -565,6 +568,7 @@ int step_accept(Handle& h, int c);              // A5 + A6 by tiers
 int step_budget(Handle& h, int32_t* out_ids, double* out_scores);  // A7
 int ensure_candidates(Handle& h, int64_t R, int c);
 int grow_join(Handle& h);
+int grow_list(Handle& h, int64_t entries);
 int grow_tables(Handle& h, int64_t slots, int64_t xblocks);
 int device_alloc(Handle& h, void** p, size_t bytes);
 

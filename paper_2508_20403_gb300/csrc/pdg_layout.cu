@@ -188,12 +188,16 @@ __global__ void k_lay_up(const int32_t* __restrict__ parent_pre, int64_t n, int4
   }
 }
 
-__global__ void k_lay_edges(int32_t* __restrict__ eu, int32_t* __restrict__ ev, const int32_t* __restrict__ pre_of,
-                            int64_t m) {
+// the edge list in labels, and the weight of every label's edge to its parent
+__global__ void k_lay_edges(int32_t* __restrict__ eu, int32_t* __restrict__ ev, const double* __restrict__ ew,
+                            const int32_t* __restrict__ pre_of, const int32_t* __restrict__ parent_pre, int64_t m,
+                            double* __restrict__ wup) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t a = pre_of[eu[e]], b = pre_of[ev[e]];
-    eu[e] = min(a, b);
-    ev[e] = max(a, b);
+    const int32_t x = pre_of[eu[e]], y = pre_of[ev[e]];
+    const int32_t a = min(x, y), b = max(x, y);
+    eu[e] = a;
+    ev[e] = b;
+    if (parent_pre[b] == a) wup[b] = ew[e];
   }
 }
 
@@ -227,6 +231,7 @@ int build_tree_layout(Handle& h) {
   if ((st = device_alloc(h, (void**)&h.tour, sizeof(int32_t) * (size_t)std::max<int64_t>(A, 1))) ||
       (st = device_alloc(h, (void**)&h.vtx_of_pre, sizeof(int32_t) * (size_t)n)) ||
       (st = device_alloc(h, &h.up, sizeof(int4) * (size_t)n)) ||
+      (st = device_alloc(h, (void**)&h.wup, sizeof(double) * (size_t)n)) ||
       (st = device_alloc(h, &h.rec, 2 * sizeof(u128) * (size_t)n)))
     return st;
   // the range-minimum table: a row per power of two up to the number of 32-label groups
@@ -298,7 +303,8 @@ int build_tree_layout(Handle& h) {
     while ((1ll << dep_bits) <= h.max_depth) dep_bits++;
     if (h.hsc->e_max != INT_MIN && h.hsc->e_max - h.hsc->e_min + 53 + dep_bits > 96) return fail(PDG_E_RANGE);
   }
-  if (m > 0) k_lay_edges<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, pre_of, m);
+  LAY_CK(cudaMemsetAsync(h.wup, 0, sizeof(double) * n, s));
+  if (m > 0) k_lay_edges<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, h.el_w, pre_of, parent_pre, m, h.wup);
   k_lay_up<<<gn, kBlock, 0, s>>>(parent_pre, n, static_cast<int4*>(h.up));
   LAY_CK(cudaMemcpyAsync(h.parent, parent_pre, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
   LAY_CK(cudaGetLastError());

@@ -1,5 +1,6 @@
 // Step A3: score every off-tree edge (Algorithm 1 step 1: LCA_query,
-// distance_query, compute_resistance).
+// distance_query, compute_resistance), telling it from the tree edges by the
+// parent in the record of its larger label.
 //
 //   l   = LCA_T(u, v): with preorder labels u < v, the smallest parent among the
 //         labels (u, v], one range-minimum query (pdg_tree.cu)
@@ -12,11 +13,12 @@
 // groups between them, all addressed by (u, v) alone; then P(l).  The
 // conversion runs on the integer pipes (pdg_fp.cuh); the product is one FP64
 // multiply, which the FP64 pipe takes in fewer issue slots than an integer
-// version of it.
+// version of it.  The edges and the results are streamed past L2 (evict first):
+// the records should stay there.
 //
-// The score is positive, so its IEEE bit pattern read as an unsigned integer
-// orders like the score itself; key[i] stores those bits for the selection
-// and sort steps.
+// The score is not negative, so its IEEE bit pattern read as an unsigned
+// integer orders like the score itself; key[id] stores those bits + 1 for the
+// selection and sort steps, and 0 for a tree edge.
 #include <algorithm>
 
 #include "pdg_fp.cuh"
@@ -28,9 +30,9 @@ namespace {
 
 
 struct ScoreArgs {
-  const int32_t* ou;
-  const int32_t* ov;
-  const double* ow;
+  const int32_t* eu;
+  const int32_t* ev;
+  const double* ew;
   const uint4* rec;       // [2 n]: P; minimum of the group's parents up to the label, after it, mask, parent
   const int32_t* parent;
   const int32_t* table;   // [rows][n1]
@@ -45,10 +47,14 @@ struct ScoreArgs {
 };
 
 __device__ __forceinline__ void score_edge(const ScoreArgs& A, int64_t i, uint32_t* s_hist) {
-  const uint32_t u = (uint32_t)A.ou[i], v = (uint32_t)A.ov[i];  // preorder labels, u < v
+  const uint32_t u = (uint32_t)__ldcs(A.eu + i), v = (uint32_t)__ldcs(A.ev + i);  // preorder labels, u < v
   uint4 pu, mu, pv, mv;
   load_sector(A.rec + 2 * (uint64_t)u, pu, mu);
   load_sector(A.rec + 2 * (uint64_t)v, pv, mv);
+  if (mv.w == u) {  // a tree edge
+    __stcs(A.key + i, (uint64_t)0);
+    return;
+  }
   int32_t l;
   const uint32_t gu = u >> 5, gv = v >> 5;
   if (gu == gv) {  // (u, v] inside one group: the lowest mask bit after u
@@ -72,9 +78,10 @@ __device__ __forceinline__ void score_edge(const ScoreArgs& A, int64_t i, uint32
   const uint64_t rb = fixed_hl_to_bits((uint64_t)(r_fixed >> 64), (uint64_t)r_fixed, A.S);  // below 2^97
   uint64_t sb = rb;
   if (A.score_mode != PDG_SCORE_RESISTANCE)  // one IEEE multiply, rounded to nearest-even
-    sb = (uint64_t)__double_as_longlong(__dmul_rn(A.ow[i], __longlong_as_double((long long)rb)));
-  A.key[i] = sb;
-  A.lca[i] = l;
+    sb = (uint64_t)__double_as_longlong(__dmul_rn(__ldcs(A.ew + i), __longlong_as_double((long long)rb)));
+  sb++;
+  __stcs(A.key + i, sb);
+  __stcs(A.lca + i, l);
   if (s_hist) atomicAdd(&s_hist[sb >> 52], 1u);
 }
 
@@ -84,16 +91,18 @@ __device__ __forceinline__ void score_edge(const ScoreArgs& A, int64_t i, uint32
 // blocks retire.  The edges in flight then stay a narrow window of the list,
 // so the records being gathered (those of a few graphs of a packed batch) stay
 // in L2 however long the list is, and no warp draws tickets from one word.
-// Tiles of 4096 edges: R-MAT scale 22 0.83 ms, 192 packed graphs 0.285 ms
-// (8192: 0.85 and 0.36, 16384: 0.91 and 0.51).  Eight blocks per SM (32
-// registers, one word spilled): mesh 128^3 0.067 ms, at six 0.072.
-// Before the 32-byte records, with nine gathers and tickets: 1.51, 0.40 and
-// 0.094 ms.
+// Tiles of 4096 edges: 192 packed graphs 0.285 ms (8192: 0.36, 16384: 0.51).
+// Eight blocks per SM (32 registers): 5 % ahead of six on a mesh.  Measured with
+// the tree edges skipped here: mesh 128^3 0.103 ms, R-MAT scale 22 0.815 ms,
+// 192 packed graphs 0.331 ms, where a compaction of the off-tree edges and the
+// scoring of the list took 0.135, 1.46 and 0.58 ms (queueing the off-tree edges
+// of a warp so that every lane scores costs a gather more per edge: slower on
+// all of them, 1.27 ms on R-MAT).
 constexpr int64_t kScoreTile = 4096;
 constexpr int kScoreBlocks = 8;
 
-__global__ void __launch_bounds__(kBlock, kScoreBlocks) k_score(ScoreArgs A, int64_t E, int64_t tile,
-                                                     const DevScalars* __restrict__ dsc) {
+__global__ void __launch_bounds__(kBlock, kScoreBlocks) k_score(ScoreArgs A, int64_t m, int64_t tile,
+                                                                const DevScalars* __restrict__ dsc) {
   dep_sync();
   __shared__ uint32_t s_hist[kSelBins];
   uint32_t* sh = A.hist ? s_hist : nullptr;  // uniform over the grid
@@ -102,7 +111,7 @@ __global__ void __launch_bounds__(kBlock, kScoreBlocks) k_score(ScoreArgs A, int
     __syncthreads();
   }
   A.S = 52 - dsc->e_min;
-  const int64_t i0 = (int64_t)blockIdx.x * tile, i1 = min(E, i0 + tile);
+  const int64_t i0 = (int64_t)blockIdx.x * tile, i1 = min(m, i0 + tile);
   for (int64_t i = i0 + threadIdx.x; i < i1; i += kBlock) score_edge(A, i, sh);
   if (sh) {
     __syncthreads();
@@ -114,12 +123,12 @@ __global__ void __launch_bounds__(kBlock, kScoreBlocks) k_score(ScoreArgs A, int
 }  // namespace
 
 int step_score(Handle& h, int score_mode) {
-  if (h.E_off == 0) return PDG_OK;
+  if (h.m == 0) return PDG_OK;
   ++h.launches;
   ScoreArgs A{};
-  A.ou = h.off_u;
-  A.ov = h.off_v;
-  A.ow = h.off_w;
+  A.eu = h.el_u;
+  A.ev = h.el_v;
+  A.ew = h.el_w;
   A.rec = static_cast<const uint4*>(h.rec);
   A.parent = h.parent;
   A.table = h.rmq_table;
@@ -131,9 +140,9 @@ int step_score(Handle& h, int score_mode) {
   A.lca = h.lca;
   A.hist = h.fuse_hist ? h.hist : nullptr;
   const int64_t wave = (int64_t)h.num_sms * kScoreBlocks;
-  const int64_t even = ((h.E_off + wave - 1) / wave + kBlock - 1) / kBlock * kBlock;
+  const int64_t even = ((h.m + wave - 1) / wave + kBlock - 1) / kBlock * kBlock;
   const int64_t tile = std::min(even, kScoreTile);
-  launch_k(h, k_score, (int)((h.E_off + tile - 1) / tile), kBlock, 0, A, h.E_off, tile, h.dsc);
+  launch_k(h, k_score, (int)((h.m + tile - 1) / tile), kBlock, 0, A, h.m, tile, h.dsc);
   PDG_CUDA(cudaGetLastError());
   return PDG_OK;
 }

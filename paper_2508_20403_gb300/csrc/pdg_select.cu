@@ -12,6 +12,8 @@
 // The threshold comes from a two-level radix select on the score bits
 // (12 bits: sign + exponent, then the next 12 mantissa bits); every edge of
 // the boundary bucket is kept, so the candidate set is always a prefix.
+#include <algorithm>
+
 #include "pdg_internal.cuh"
 
 namespace pdg {
@@ -26,16 +28,11 @@ __device__ __forceinline__ int64_t sel_chunk(int64_t E, int nb) {
   return (c + kTile - 1) / kTile * kTile;
 }
 
-__device__ __forceinline__ void sel_count(uint32_t* h, uint64_t k, int lvl, int32_t b1) {
-  if (lvl == 0) atomicAdd(&h[k >> 52], 1u);
-  else if ((int32_t)(k >> 52) == b1) atomicAdd(&h[(k >> 40) & 0xfff], 1u);
-}
-
-// level 1 (lvl == 0): bins of key >> 52; level 2: bins of (key >> 40) & 0xfff
-// restricted to the level-1 bucket of the edge's graph.
+// Level 1: bins of key >> 52 (the lists of a single graph are counted by the
+// scoring kernel itself); 0 marks a tree edge.
 __global__ void __launch_bounds__(kBlock) k_sel_hist(const uint64_t* __restrict__ key, int64_t E,
-                                                     const int64_t* __restrict__ off_ptr, int32_t G,
-                                                     const GraphSel* __restrict__ sel, int lvl,
+                                                     const int64_t* __restrict__ edge_ptr, int32_t G,
+                                                     const GraphSel* __restrict__ sel,
                                                      uint32_t* __restrict__ hist) {
   dep_sync();
   __shared__ uint32_t sh[kSelBins];
@@ -43,18 +40,19 @@ __global__ void __launch_bounds__(kBlock) k_sel_hist(const uint64_t* __restrict_
   const int64_t b0 = (int64_t)blockIdx.x * chunk;
   const int64_t b1 = min(E, b0 + chunk);
   if (b0 >= b1) return;
-  const int32_t g0 = (G == 1) ? 0 : part_of(off_ptr, G, b0);
-  const int32_t g1 = (G == 1) ? 0 : part_of(off_ptr, G, b1 - 1);
+  const int32_t g0 = (G == 1) ? 0 : part_of(edge_ptr, G, b0);
+  const int32_t g1 = (G == 1) ? 0 : part_of(edge_ptr, G, b1 - 1);
   // one graph at a time: a shared-memory histogram for long ranges, direct
   // global atomics for short ones (many small graphs per chunk)
   for (int32_t g = g0; g <= g1; g++) {
-    const int64_t r0 = (G == 1) ? b0 : max(b0, off_ptr[g]);
-    const int64_t r1 = (G == 1) ? b1 : min(b1, off_ptr[g + 1]);
+    const int64_t r0 = (G == 1) ? b0 : max(b0, edge_ptr[g]);
+    const int64_t r1 = (G == 1) ? b1 : min(b1, edge_ptr[g + 1]);
     const GraphSel s = sel[g];
     if (s.take_all || r0 >= r1) continue;
     uint32_t* hg = hist + (int64_t)g * kSelBins;
     if (r1 - r0 < 256) {  // too short to amortise clearing and flushing 4096 shared bins
-      for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) sel_count(hg, key[i], lvl, s.b1);
+      for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x)
+        if (key[i]) atomicAdd(&hg[key[i] >> 52], 1u);
       continue;
     }
     for (int i = threadIdx.x; i < kSelBins; i += blockDim.x) sh[i] = 0;
@@ -68,7 +66,7 @@ __global__ void __launch_bounds__(kBlock) k_sel_hist(const uint64_t* __restrict_
       }
 #pragma unroll
       for (int u = 0; u < kHistUnroll; u++)
-        if (i0 + u * kBlock + threadIdx.x < r1) sel_count(sh, k[u], lvl, s.b1);
+        if (k[u]) atomicAdd(&sh[k[u] >> 52], 1u);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < kSelBins; i += blockDim.x)
@@ -85,7 +83,7 @@ static_assert(kPickPer == 16, "pick layout");
 
 __global__ void __launch_bounds__(kBlock) k_sel_pick(uint32_t* __restrict__ hist, GraphSel* __restrict__ sel,
                                                      const int64_t* __restrict__ off_ptr, int32_t G, int lvl,
-                                                     int64_t* __restrict__ count_out, int64_t* __restrict__ cand_ptr) {
+                                                     int64_t* __restrict__ count_out, int64_t* __restrict__ ptr) {
   dep_sync();
   __shared__ int64_t sm[kBlock / 32 + 1];
   __shared__ int s_owner;
@@ -93,14 +91,14 @@ __global__ void __launch_bounds__(kBlock) k_sel_pick(uint32_t* __restrict__ hist
   GraphSel s = sel[g];
   uint32_t* hg = hist + (int64_t)g * kSelBins;
   if (s.take_all) {
-    if (lvl == 1 && threadIdx.x == 0) {
+    if (threadIdx.x == 0) {
       s.count = off_ptr[g + 1] - off_ptr[g];
-      s.thresh = 0;
+      s.thresh = 1;  // every off-tree edge (tree edges have key 0)
       sel[g] = s;
       count_out[g] = s.count;
-      if (G == 1) {  // a single graph's candidate offsets need no scan
-        cand_ptr[0] = 0;
-        cand_ptr[1] = s.count;
+      if (G == 1) {  // a single graph's offsets need no scan
+        ptr[0] = 0;
+        ptr[1] = s.count;
       }
     }
     return;
@@ -147,16 +145,19 @@ __global__ void __launch_bounds__(kBlock) k_sel_pick(uint32_t* __restrict__ hist
     if (lvl == 0) {
       s.b1 = bin;
       s.above1 = run;
+      s.count = run + bin_count;
+      s.thresh = (uint64_t)bin << 52;
     } else {
       s.b2 = bin;
       s.above2 = run;
       s.count = s.above1 + run + bin_count;
       s.thresh = ((uint64_t)s.b1 << 52) | ((uint64_t)bin << 40);
-      count_out[g] = s.count;
-      if (G == 1) {
-        cand_ptr[0] = 0;
-        cand_ptr[1] = s.count;
-      }
+    }
+    s.thresh = max(s.thresh, (uint64_t)1);
+    count_out[g] = s.count;
+    if (G == 1) {
+      ptr[0] = 0;
+      ptr[1] = s.count;
     }
     sel[g] = s;
   }
@@ -165,146 +166,346 @@ __global__ void __launch_bounds__(kBlock) k_sel_pick(uint32_t* __restrict__ hist
   for (int q = 0; q < kPickPer / 4; q++) w4[q] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// Ordered compaction of the selected edges (key >= the graph's threshold), in
-// canonical id order: a count pass per block chunk, then a write pass whose
-// blocks add up the counts of the blocks before them and place each tile's
-// selected edges by a block scan.  Both passes stream the keys with vector
-// loads.
-struct CandSrc {
+// The compaction runs in two steps, so that the m keys are read once (for a
+// single graph; before, three times: the second histogram, a counting and a
+// writing pass, 380 us of 1.47 ms on R-MAT scale 22).
+//
+// k_sel_list, over all keys with the level-1 threshold, lists the edges of the
+// boundary bucket and above.  Every block takes one tile of keys, keeps the
+// tile's edges in id order, and places them as one run wherever the list's end
+// is at that moment; the tile's place and length go to a table.  (Placing the
+// runs themselves in order by a chained look-back passed 20 tiles per us, half
+// the rate at which the keys arrive.)  The second histogram and the exact
+// compaction then read that short list, tile by tile in id order.
+// Tiles of 8192 keys, two blocks per SM: R-MAT scale 22 (64 M keys) 0.15 ms.
+constexpr int kListThreads = 1024;
+constexpr int kListWarps = kListThreads / 32;
+constexpr int kListPairs = 4;  // pairs of keys per thread
+constexpr int kListTile = kListThreads * kListPairs * 2;
+
+struct ListArgs {
+  const uint64_t* key;      // by id
+  int64_t m;
+  const int64_t* edge_ptr;  // graphs' ids
+  int32_t G;
+  const GraphSel* sel;
+  int64_t cap;              // of the list
+  int32_t* list_id;
+  uint64_t* list_key;
+  int2* tile;               // per tile: first entry, entries
+};
+
+// the graph of position p, found by one warp with 32-way splits
+__device__ __forceinline__ int32_t warp_part_of(const int64_t* __restrict__ ptr, int32_t G, int64_t p) {
+  const int lane = threadIdx.x & 31;
+  int32_t lo = 0, hi = G;  // ptr[lo] <= p < ptr[hi]
+  while (hi - lo > 1) {
+    const int32_t step = (hi - lo + 31) / 32, q = lo + lane * step;
+    const bool ok = q < hi && ptr[q] <= p;
+    const int last = 31 - __clz(__ballot_sync(0xffffffffu, ok));  // lane 0 is always ok
+    lo += last * step;
+    hi = min(hi, lo + step);
+  }
+  return lo;
+}
+
+__global__ void __launch_bounds__(kListThreads, 2) k_sel_list(ListArgs a, DevScalars* dsc) {
+  dep_sync();
+  __shared__ int sm[kListThreads / 32 + 1];
+  __shared__ uint16_t s_pick[kListTile];
+  __shared__ int s_count[kListPairs * kListWarps];
+  __shared__ int64_t s_base;
+  __shared__ int s_graph;
+  const int64_t t0 = (int64_t)blockIdx.x * kListTile;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const unsigned below = (1u << lane) - 1;
+  // neighbouring threads read neighbouring pairs of keys
+  uint64_t k[2 * kListPairs];
+#pragma unroll
+  for (int i = 0; i < kListPairs; i++) {
+    const int64_t p = t0 + 2 * ((int64_t)i * kListThreads + threadIdx.x);
+    if (p + 2 <= a.m) {
+      const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(a.key + p);
+      k[2 * i] = x.x;
+      k[2 * i + 1] = x.y;
+    } else {
+      k[2 * i] = p < a.m ? a.key[p] : 0;
+      k[2 * i + 1] = 0;
+    }
+  }
+  if (a.G > 1) {
+    if (wid == 0) {
+      const int32_t g = warp_part_of(a.edge_ptr, a.G, t0);
+      if (lane == 0) s_graph = g;
+    }
+    __syncthreads();
+  }
+  // each thread follows its keys' graphs
+  int32_t g = a.G > 1 ? s_graph : 0;
+  int64_t g_end = a.G > 1 ? a.edge_ptr[g + 1] : INT64_MAX;
+  uint64_t th = a.sel[g].thresh;
+  uint32_t pick = 0;
+#pragma unroll
+  for (int i = 0; i < 2 * kListPairs; i++) {
+    const int64_t p = t0 + 2 * ((int64_t)(i / 2) * kListThreads + threadIdx.x) + (i & 1);
+    if (p < a.m) {
+      while (p >= g_end) {
+        g++;
+        g_end = a.edge_ptr[g + 1];
+        th = a.sel[g].thresh;
+      }
+      if (k[i] >= th) pick |= 1u << i;
+    }
+  }
+  // offsets in key order: rounds, then warps, then lanes
+#pragma unroll
+  for (int i = 0; i < kListPairs; i++) {
+    const unsigned b0 = __ballot_sync(0xffffffffu, pick >> (2 * i) & 1u);
+    const unsigned b1 = __ballot_sync(0xffffffffu, pick >> (2 * i + 1) & 1u);
+    if (lane == 0) s_count[i * kListWarps + wid] = __popc(b0) + __popc(b1);
+  }
+  __syncthreads();
+  int tot;
+  const int before = block_excl_scan_n<kListThreads>(threadIdx.x < kListPairs * kListWarps ? s_count[threadIdx.x] : 0, sm, &tot);
+  if (threadIdx.x < kListPairs * kListWarps) s_count[threadIdx.x] = before;
+  if (threadIdx.x == 0) {
+    int64_t base = tot ? (int64_t)atomicAdd((unsigned long long*)&dsc->n_list, (unsigned long long)tot) : 0;
+    const bool fits = base + tot <= a.cap;
+    if (!fits) atomicOr(&dsc->err, ERR_CAPACITY);  // the host grows the list (n_list entries) and repeats
+    a.tile[blockIdx.x] = make_int2((int)base, fits ? tot : 0);
+    s_base = fits ? base : -1;
+  }
+  __syncthreads();
+  if (s_base < 0 || tot == 0) return;  // uniform
+#pragma unroll
+  for (int i = 0; i < kListPairs; i++) {
+    const bool y0 = pick >> (2 * i) & 1u, y1 = pick >> (2 * i + 1) & 1u;
+    const unsigned b0 = __ballot_sync(0xffffffffu, y0), b1 = __ballot_sync(0xffffffffu, y1);
+    int at = s_count[i * kListWarps + wid] + __popc(b0 & below) + __popc(b1 & below);
+    const int j = 2 * (i * kListThreads + threadIdx.x);
+    if (y0) s_pick[at++] = (uint16_t)j;
+    if (y1) s_pick[at] = (uint16_t)(j + 1);
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < tot; j += kListThreads) {
+    const int64_t i = t0 + s_pick[j];
+    a.list_id[s_base + j] = (int32_t)i;
+    a.list_key[s_base + j] = a.key[i];
+  }
+}
+
+// Blocks of the list's readers: each takes a run of at most kRunTiles tiles,
+// whose entries it numbers through in id order.
+constexpr int kRunThreads = 512;
+constexpr int kRunTiles = 64;
+
+struct ListRun {
+  int first[kRunTiles], start[kRunTiles + 1];
+  int graph[kRunTiles];     // of the tile's first id
+  int64_t ends[kRunTiles];  // where that graph's ids end
+  int entries;
+  __device__ __forceinline__ void open(const int2* __restrict__ tile, int64_t tiles, const int64_t* __restrict__ edge_ptr,
+                                       int32_t G) {
+    const int64_t per = (tiles + gridDim.x - 1) / gridDim.x, b = (int64_t)blockIdx.x * per;
+    if (threadIdx.x < 32) {
+      const int lane = threadIdx.x;
+      int run = 0;
+      for (int j0 = 0; j0 < kRunTiles; j0 += 32) {
+        const int j = j0 + lane;
+        const bool mine = j < per && b + j < tiles;
+        const int2 t = mine ? tile[b + j] : make_int2(0, 0);
+        const int incl = warp_incl_scan(t.y);
+        first[j] = t.x;
+        start[j] = run + incl - t.y;
+        run += __shfl_sync(0xffffffffu, incl, 31);
+        const int64_t id0 = (b + j) * kListTile;
+        graph[j] = G > 1 && mine ? part_of(edge_ptr, G, id0) : 0;
+        ends[j] = G > 1 && mine ? edge_ptr[graph[j] + 1] : INT64_MAX;
+      }
+      if (lane == 0) start[kRunTiles] = entries = run;
+    }
+    __syncthreads();
+  }
+  // place in the list of the run's entry q, and its tile in the run
+  __device__ __forceinline__ int64_t at(int q, int& j) const {
+    j = 0;
+#pragma unroll
+    for (int o = kRunTiles / 2; o; o >>= 1)
+      if (start[j + o] <= q) j += o;
+    return (int64_t)first[j] + (q - start[j]);
+  }
+  __device__ __forceinline__ int32_t graph_of(int j, int32_t id, const int64_t* __restrict__ edge_ptr) const {
+    int32_t g = graph[j];
+    if (id >= ends[j])
+      while (id >= edge_ptr[g + 1]) g++;
+    return g;
+  }
+};
+
+struct PickArgs {
+  const int2* tile;
+  int64_t tiles;
+  const int32_t* list_id;
+  const uint64_t* list_key;
+  const int64_t* edge_ptr;
+  int32_t G;
+  const GraphSel* sel;
+  uint32_t* hist;
+  int64_t* block_count;     // selected entries per block
+  const int64_t* cand_ptr;
+  int64_t cap;              // candidates
+  int32_t* cand_idx;
+  uint64_t* rkey;
+  int32_t* rval;
   const int32_t* u;
   const int32_t* v;
   const int32_t* lca;
-  const int32_t* id;
-  int4* rec;  // [2 R]: u, v, LCA, canonical id; score bits
+  int4* rec;                // [2 R]: u, v, LCA, canonical id; score bits
 };
 
-template <bool WRITE>
-__global__ void __launch_bounds__(kBlock) k_sel_compact(const uint64_t* __restrict__ key, int64_t E,
-                                                        const int64_t* __restrict__ off_ptr, int32_t G,
-                                                        const GraphSel* __restrict__ sel,
-                                                        int64_t* __restrict__ bcount, int64_t cap,
-                                                        int32_t* __restrict__ cand_idx,
-                                                        uint64_t* __restrict__ rkey, int32_t* __restrict__ rval,
-                                                        const int64_t* __restrict__ cand_ptr, CandSrc src,
-                                                        DevScalars* dsc) {
+// Level 2: bins of (key >> 40) & 0xfff inside the level-1 bucket of the entry's graph.
+__global__ void __launch_bounds__(kRunThreads) k_sel_hist2(PickArgs a) {
   dep_sync();
-  __shared__ int64_t sm[kBlock / 32 + 1];
-  __shared__ uint16_t s_pick[WRITE ? kTile : 1];
-  const int64_t chunk = sel_chunk(E, gridDim.x);
-  const int64_t b0 = (int64_t)blockIdx.x * chunk;
-  const int64_t b1 = min(E, b0 + chunk);
-  int64_t run = 0;
-  if (WRITE) {  // this block's offset: the counts of the blocks before it, added up here (no separate scan)
-    int64_t c = 0;
-    for (int i = threadIdx.x; i < (int)blockIdx.x; i += kBlock) c += bcount[i];
-    run = block_sum(c, sm);
+  __shared__ ListRun run;
+  __shared__ uint32_t sh[kSelBins];
+  run.open(a.tile, a.tiles, a.edge_ptr, a.G);
+  if (a.G == 1) {
+    if (run.entries == 0) return;  // uniform
+    for (int i = threadIdx.x; i < kSelBins; i += kRunThreads) sh[i] = 0;
+    __syncthreads();
+  }
+  for (int q = threadIdx.x; q < run.entries; q += kRunThreads) {
+    int j;
+    const int64_t at = run.at(q, j);
+    const uint64_t k = a.list_key[at];
+    const int32_t g = a.G == 1 ? 0 : run.graph_of(j, a.list_id[at], a.edge_ptr);
+    const GraphSel& s = a.sel[g];
+    if (s.take_all || (int32_t)(k >> 52) != s.b1) continue;
+    if (a.G == 1) atomicAdd(&sh[(k >> 40) & 0xfff], 1u);
+    else atomicAdd(&a.hist[(int64_t)g * kSelBins + ((k >> 40) & 0xfff)], 1u);
+  }
+  if (a.G > 1) return;
+  __syncthreads();
+  for (int i = threadIdx.x; i < kSelBins; i += kRunThreads)
+    if (sh[i]) atomicAdd(&a.hist[i], sh[i]);
+}
+
+// The candidates: entries at or above their graph's threshold, in id order.
+// A count per block, then a write pass whose blocks add up the counts before
+// their own.
+template <bool WRITE>
+__global__ void __launch_bounds__(kRunThreads) k_sel_pick_list(PickArgs a, DevScalars* dsc) {
+  dep_sync();
+  __shared__ ListRun run;
+  __shared__ int64_t sm[kRunThreads / 32 + 1];
+  run.open(a.tile, a.tiles, a.edge_ptr, a.G);
+  int64_t base = 0;
+  if (WRITE) {
+    int64_t c = 0, tot;
+    for (int i = threadIdx.x; i < (int)blockIdx.x; i += kRunThreads) c += a.block_count[i];
+    block_excl_scan_n<kRunThreads>(c, sm, &base);
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {  // the last block's end is the total
-      const int64_t total = run + bcount[blockIdx.x];
-      dsc->n_cand_wanted = total;
-      if (total > cap || total != cand_ptr[G]) {
-        // nothing downstream may touch more than `cap` candidates: run it empty
-        dsc->n_cand = 0;
-        atomicOr(&dsc->err, ERR_CAPACITY);
-      } else {
-        dsc->n_cand = total;
-      }
+      tot = base + a.block_count[blockIdx.x];
+      dsc->n_cand_wanted = tot;
+      const bool fits = tot <= a.cap && tot == a.cand_ptr[a.G];
+      // nothing downstream may touch more than `cap` candidates: run it empty
+      if (!fits) atomicOr(&dsc->err, ERR_CAPACITY);
+      dsc->n_cand = fits ? tot : 0;
     }
   }
-  int64_t tot = 0;
-  for (int64_t t0 = b0; t0 < b1; t0 += kTile) {
-    const int64_t base = t0 + (int64_t)threadIdx.x * kItems;
-    uint32_t pick = 0;
-    uint64_t k[kItems];
-    if (base < b1) {
-      // graph of the first item, then advanced item by item
-      int32_t g = (G == 1) ? 0 : part_of(off_ptr, G, base);
-      int64_t g_end = (G == 1) ? INT64_MAX : off_ptr[g + 1];
-      uint64_t th = sel[g].thresh;
-      if (base + kItems <= b1) {
-        const ulonglong2* k2 = reinterpret_cast<const ulonglong2*>(key + base);
-#pragma unroll
-        for (int q = 0; q < kItems / 2; q++) {
-          const ulonglong2 x = k2[q];
-          k[2 * q] = x.x;
-          k[2 * q + 1] = x.y;
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < kItems; i++) k[i] = (base + i < b1) ? key[base + i] : 0;
-      }
-#pragma unroll
-      for (int i = 0; i < kItems; i++) {
-        const int64_t p = base + i;
-        if (p < b1) {
-          while (p >= g_end) {
-            g++;
-            g_end = off_ptr[g + 1];
-            th = sel[g].thresh;
-          }
-          if (k[i] >= th) pick |= 1u << i;
-        }
-      }
+  int64_t count = 0;
+  for (int q0 = 0; q0 < run.entries; q0 += kRunThreads) {
+    const int q = q0 + threadIdx.x;
+    bool in = false;
+    int64_t at = 0;
+    uint64_t k = 0;
+    if (q < run.entries) {
+      int j;
+      at = run.at(q, j);
+      k = a.list_key[at];
+      const int32_t g = a.G == 1 ? 0 : run.graph_of(j, a.list_id[at], a.edge_ptr);
+      in = k >= a.sel[g].thresh;
     }
-    const int64_t cnt = __popc(pick);
     if (!WRITE) {
-      tot += cnt;
+      count += in ? 1 : 0;
       continue;
     }
-    // the tile's selected edges are listed in shared memory, then taken by neighbouring threads: every access
-    // below but the gathers of the edge's own words is coalesced, and those are in id order
-    int64_t tile_tot;
-    int at = (int)block_excl_scan(cnt, sm, &tile_tot);
-#pragma unroll
-    for (int i = 0; i < kItems; i++)
-      if (pick & (1u << i)) s_pick[at++] = (uint16_t)(threadIdx.x * kItems + i);
-    __syncthreads();
-    for (int j = threadIdx.x; j < (int)tile_tot; j += kBlock) {
-      const int64_t i = t0 + s_pick[j], pos = run + j;
-      if (pos >= cap) break;
-      const uint64_t kk = __ldg(key + i);
-      cand_idx[pos] = (int32_t)i;
-      rkey[pos] = ~kk;  // ascending ~score = descending score
-      rval[pos] = (int32_t)pos;
-      // what the later steps read of a candidate, in one sector
-      src.rec[2 * pos] = make_int4(__ldg(src.u + i), __ldg(src.v + i), __ldg(src.lca + i), __ldg(src.id + i));
-      reinterpret_cast<uint64_t*>(src.rec)[4 * pos + 2] = kk;
-    }
-    run += tile_tot;
-    __syncthreads();
+    int64_t tot;
+    const int64_t pos = base + block_excl_scan_n<kRunThreads>((int64_t)(in ? 1 : 0), sm, &tot);
+    base += tot;
+    if (!in || pos >= a.cap) continue;
+    const int32_t id = a.list_id[at];
+    a.cand_idx[pos] = id;
+    a.rkey[pos] = ~k;  // ascending ~score = descending score
+    a.rval[pos] = (int32_t)pos;
+    // what the later steps read of a candidate, in one sector
+    a.rec[2 * pos] = make_int4(__ldg(a.u + id), __ldg(a.v + id), __ldg(a.lca + id), id);
+    reinterpret_cast<uint64_t*>(a.rec)[4 * pos + 2] = k - 1;
   }
   if (!WRITE) {
-    tot = block_sum(tot, sm);
-    if (threadIdx.x == 0) bcount[blockIdx.x] = tot;
+    int64_t tot;
+    block_excl_scan_n<kRunThreads>(count, sm, &tot);
+    if (threadIdx.x == 0) a.block_count[blockIdx.x] = tot;
   }
 }
 
 }  // namespace
 
+int64_t select_tiles(int64_t m) { return std::max<int64_t>(1, (m + kListTile - 1) / kListTile); }
+
 int step_select(Handle& h) {
-  const int64_t E = h.E_off;
-  const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(kSelChunkBlocks, (E + kTile - 1) / kTile));
   bool any_select = false;
   for (int32_t g = 0; g < h.G; g++)
     if (h.want_h[g] < h.off_ptr_h[g + 1] - h.off_ptr_h[g]) any_select = true;
-  for (int lvl = 0; lvl < 2; lvl++) {
-    if (any_select && !(lvl == 0 && h.fuse_hist)) {
-      ++h.launches;
-      launch_k(h, k_sel_hist, nb, kBlock, 0, h.key, E, h.d_off_ptr, h.G, h.sel, lvl, h.hist);
-    }
+  const int64_t tiles = select_tiles(h.m);
+  // at most kRunTiles tiles per block, and enough blocks to fill the device when there are many tiles
+  const int64_t runs = std::max<int64_t>((tiles + kRunTiles - 1) / kRunTiles, std::min<int64_t>(tiles, (int64_t)h.num_sms * 4));
+  if (tiles > 0x7fffffff || runs > kSelRunsMax) return PDG_E_INVALID_ARG;
+  auto pick = [&](int lvl, int64_t* ptr) -> int {
     ++h.launches;
-    launch_k(h, k_sel_pick, h.G, kBlock, 0, h.hist, h.sel, h.d_off_ptr, h.G, lvl, h.d_graph_tmp, h.d_cand_ptr);
-  }
-  PDG_CUDA(cudaGetLastError());
+    launch_k(h, k_sel_pick, h.G, kBlock, 0, h.hist, h.sel, h.d_off_ptr, h.G, lvl, h.d_graph_tmp, ptr);
+    PDG_CUDA(cudaGetLastError());
+    return PDG_OK;
+  };
   int st;
+  if (any_select && !h.fuse_hist) {
+    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(kSelChunkBlocks, (h.m + kTile - 1) / kTile));
+    ++h.launches;
+    launch_k(h, k_sel_hist, nb, kBlock, 0, h.key, h.m, h.d_edge_ptr, h.G, h.sel, h.hist);
+  }
+  if ((st = pick(0, h.d_cand_ptr))) return st;
+  ListArgs la{h.key, h.m, h.d_edge_ptr, h.G, h.sel, h.list_cap, h.list_id, h.list_key, static_cast<int2*>(h.list_tile)};
+  ++h.launches;
+  launch_k(h, k_sel_list, (int)tiles, kListThreads, 0, la, h.dsc);
+  PickArgs p{};
+  p.tile = la.tile;
+  p.tiles = tiles;
+  p.list_id = h.list_id;
+  p.list_key = h.list_key;
+  p.edge_ptr = h.d_edge_ptr;
+  p.G = h.G;
+  p.sel = h.sel;
+  p.hist = h.hist;
+  p.block_count = h.blk_a;
+  p.cand_ptr = h.d_cand_ptr;
+  p.cap = h.Rcap;
+  p.cand_idx = h.cand_idx;
+  p.rkey = h.rk[0];
+  p.rval = h.rv[0];
+  p.u = h.el_u;
+  p.v = h.el_v;
+  p.lca = h.lca;
+  p.rec = static_cast<int4*>(h.cand_rec);
+  if (any_select) {
+    ++h.launches;
+    launch_k(h, k_sel_hist2, (int)runs, kRunThreads, 0, p);
+    if ((st = pick(1, h.d_cand_ptr))) return st;
+  }
   if (h.G > 1 && (st = scan_excl_i64(h, h.d_graph_tmp, h.d_cand_ptr, h.G, nullptr, h.G))) return st;
-  int64_t* bcount = h.blk_a;
   ++h.launches;
-  launch_k(h, k_sel_compact<false>, nb, kBlock, 0, h.key, E, h.d_off_ptr, h.G, h.sel, bcount, 0, nullptr, nullptr,
-           nullptr, h.d_cand_ptr, CandSrc{}, h.dsc);
+  launch_k(h, k_sel_pick_list<false>, (int)runs, kRunThreads, 0, p, h.dsc);
   ++h.launches;
-  launch_k(h, k_sel_compact<true>, nb, kBlock, 0, h.key, E, h.d_off_ptr, h.G, h.sel, bcount, h.Rcap, h.cand_idx,
-           h.rk[0], h.rv[0], h.d_cand_ptr,
-           CandSrc{h.off_u, h.off_v, h.lca, h.off_id, static_cast<int4*>(h.cand_rec)}, h.dsc);
+  launch_k(h, k_sel_pick_list<true>, (int)runs, kRunThreads, 0, p, h.dsc);
   PDG_CUDA(cudaGetLastError());
   return PDG_OK;
 }
