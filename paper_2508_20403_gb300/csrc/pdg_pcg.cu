@@ -41,29 +41,28 @@ __global__ void k_pc_tflag(const int32_t* __restrict__ eu, const int32_t* __rest
 }
 
 __global__ void k_pc_cut(const int32_t* __restrict__ rev, const int64_t* __restrict__ tptr,
-                         const int32_t* __restrict__ tdeg, int32_t root, int32_t* __restrict__ succ,
-                         int32_t* __restrict__ rd) {
-  if (blockIdx.x == 0 && threadIdx.x == 0 && tdeg[root] > 0) {
-    const int32_t tail = rev[tptr[root] + tdeg[root] - 1];
-    succ[tail] = -1;
-    rd[tail] = 0;
-  }
+                         const int32_t* __restrict__ tdeg, int32_t root, int32_t* __restrict__ succ, RankSpace r) {
+  const bool first = threadIdx.x == 0 && tdeg[root] > 0;  // one warp
+  if (first) succ[rev[tptr[root] + tdeg[root] - 1]] = -1;
+  rank_add_head(first, (int32_t)tptr[root], r.heads, r.n_heads);
 }
 
 // entry / exit positions of every non-root vertex and the weight of the edge above it
 __global__ void k_pc_times(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
                            const double* __restrict__ ew, const uint8_t* __restrict__ tflag,
                            const int32_t* __restrict__ arc_uv, const int32_t* __restrict__ rev,
-                           const int32_t* __restrict__ rd, const int64_t* __restrict__ tptr, int64_t n, int64_t m,
-                           int32_t* __restrict__ tin, int32_t* __restrict__ tout, double* __restrict__ wup) {
+                           const uint64_t* __restrict__ own, const uint64_t* __restrict__ walk,
+                           const int64_t* __restrict__ tptr, int64_t n, int64_t m, int32_t* __restrict__ tin,
+                           int32_t* __restrict__ tout, double* __restrict__ wup) {
   const int64_t last = tptr[n] - 1;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
     if (!tflag[e]) continue;
     const int32_t a1 = arc_uv[e], a2 = rev[a1];
-    const bool down1 = rd[a1] > rd[a2];  // u -> v comes first: u is the parent
+    const int32_t r1 = arc_rank(own, walk, a1), r2 = arc_rank(own, walk, a2);
+    const bool down1 = r1 > r2;  // u -> v comes first: u is the parent
     const int32_t child = down1 ? ev[e] : eu[e];
-    tin[child] = (int32_t)(last - rd[down1 ? a1 : a2]);
-    tout[child] = (int32_t)(last - rd[down1 ? a2 : a1]);
+    tin[child] = (int32_t)(last - max(r1, r2));
+    tout[child] = (int32_t)(last - min(r1, r2));
     wup[child] = ew[e];
   }
 }
@@ -420,7 +419,8 @@ int pcg_quality(Handle& h, const int32_t* ids, int64_t k, const double* b, doubl
   if (T > kScanTile) return fail(PDG_E_INVALID_ARG);      // one block scans the tile sums
   uint8_t* tflag = nullptr;
   int32_t *tdeg = nullptr, *cur = nullptr, *tadj = nullptr, *rev = nullptr, *arc_uv = nullptr;
-  int32_t *succ[2] = {nullptr, nullptr}, *rd[2] = {nullptr, nullptr}, *tin = nullptr, *tout = nullptr;
+  int32_t *succ = nullptr, *tin = nullptr, *tout = nullptr;
+  RankSpace rank;
   int32_t *ea = nullptr, *eb = nullptr, *seen = nullptr, *flags = nullptr, *icnt = nullptr, *iedge = nullptr;
   int64_t *tptr = nullptr, *iptr = nullptr;
   double *wup = nullptr, *Y = nullptr, *E = nullptr, *Z = nullptr, *E2 = nullptr, *sums = nullptr, *ewk = nullptr;
@@ -428,8 +428,8 @@ int pcg_quality(Handle& h, const int32_t* ids, int64_t k, const double* b, doubl
   double *z = nullptr, *p = nullptr, *Ap = nullptr, *t = nullptr, *u = nullptr, *yv = nullptr, *sv = nullptr;
   double *qv = nullptr, *part = nullptr, *dsc = nullptr;
   if (!talloc(&tflag, m) || !talloc(&tdeg, n) || !talloc(&cur, n) || !talloc(&tptr, n + 1) ||
-      !talloc(&tadj, A) || !talloc(&rev, A) || !talloc(&arc_uv, m) || !talloc(&succ[0], A) || !talloc(&succ[1], A) ||
-      !talloc(&rd[0], A) || !talloc(&rd[1], A) || !talloc(&tin, n) || !talloc(&tout, n) || !talloc(&wup, n) ||
+      !talloc(&tadj, A) || !talloc(&rev, A) || !talloc(&arc_uv, m) || !talloc(&succ, A) ||
+      !rank_space(rank, A, 1, s, talloc) || !talloc(&tin, n) || !talloc(&tout, n) || !talloc(&wup, n) ||
       !talloc(&Y, A + 1) || !talloc(&E, A + 1) || !talloc(&Z, A + 1) || !talloc(&E2, A + 1) || !talloc(&sums, T) ||
       !talloc(&ea, k) || !talloc(&eb, k) || !talloc(&ewk, k) || !talloc(&seen, m) || !talloc(&flags, 4) ||
       !talloc(&icnt, n) || !talloc(&iptr, n + 1) || !talloc(&iedge, 2 * k) || !talloc(&C, k * k) ||
@@ -457,16 +457,11 @@ int pcg_quality(Handle& h, const int32_t* ids, int64_t k, const double* b, doubl
   k_tour_fix_rev<<<gn, kBlock, 0, s>>>(tptr, tadj, n, rev);
   k_tour_fix_arcs<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, tflag, m, tptr, tadj, arc_uv);
   const int ga = grid_for(h, std::max<int64_t>(A, 1));
-  k_st_succ<<<ga, kBlock, 0, s>>>(tadj, rev, tptr, tdeg, n, succ[0], rd[0]);
-  k_pc_cut<<<1, 32, 0, s>>>(rev, tptr, tdeg, root, succ[0], rd[0]);
-  int bits = 1;
-  while ((1ll << bits) <= A) bits++;
-  int c = 0;
-  for (int it = 0; it < bits; it++) {
-    k_st_rank<<<ga, kBlock, 0, s>>>(succ[c], rd[c], succ[c ^ 1], rd[c ^ 1], tptr, n);
-    c ^= 1;
-  }
-  k_pc_times<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, h.el_w, tflag, arc_uv, rev, rd[c], tptr, n, m, tin, tout, wup);
+  k_st_succ<<<ga, kBlock, 0, s>>>(tadj, rev, tptr, tdeg, n, succ);
+  k_pc_cut<<<1, 32, 0, s>>>(rev, tptr, tdeg, root, succ, rank);
+  const uint64_t* walk = rank_lists(h, succ, tptr + n, rank, s);
+  k_pc_times<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, h.el_w, tflag, arc_uv, rev, rank.own, walk, tptr, n, m, tin, tout,
+                                   wup);
   // the grounded tree solve x = L_T^-1 y
   const int64_t NA = A + 1;
   const int tiles = (int)T;

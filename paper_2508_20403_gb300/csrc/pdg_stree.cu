@@ -12,15 +12,15 @@
 // Each tree is rooted at the maximum-degree vertex of its component (ties:
 // smaller id) and returned as a parent array.
 //
-// Forest: Boruvka rounds.  Every component finds its maximum incident edge
-// leaving it (an atomicMax on the key bits, then an atomicMin on the edge id
-// among the edges carrying that key), hooks to the component across it (two
-// components that chose the same edge: the smaller id stays the root; with a
-// strict order no longer cycle exists), and pointer jumping relabels the
-// vertices.  Rooting: an Euler tour of the forest (arc x->y is followed by
-// the arc after y->x in y's tree adjacency, cut at each root) ranked by
-// pointer jumping; of the two arcs of a tree edge, the earlier one runs from
-// the parent to the child.
+// Forest: Boruvka rounds over the edges that still join two trees.  Every tree
+// finds its maximum edge (an atomicMax on the key bits, then an atomicMin on
+// the edge id among the edges carrying that key), hooks to the tree across it
+// (two trees that chose the same edge: the smaller id stays the root; with a
+// strict order no longer cycle exists), and a filter writes the next round's
+// list with the new roots.  Rooting: an Euler tour of the forest (arc x->y is
+// followed by the arc after y->x in y's tree adjacency, cut at each root),
+// ranked; of the two arcs of a tree edge, the earlier one runs from the parent
+// to the child.
 #include <climits>
 #include <cmath>
 #include <type_traits>
@@ -34,6 +34,7 @@ namespace pdg {
 namespace {
 
 constexpr int32_t kNoEdge = INT_MAX;
+constexpr int kStRounds = 40;
 
 __device__ __forceinline__ unsigned long long degree_key(const int64_t* __restrict__ row_ptr, int64_t v) {
   // larger degree first, then smaller id
@@ -60,6 +61,100 @@ __global__ void k_st_bfs(const int64_t* __restrict__ row_ptr, const int32_t* __r
     }
   }
   if (__any_sync(0xffffffffu, any) && (threadIdx.x & 31) == 0) *grew = 1;
+}
+
+// Levels of narrow frontiers in one cluster of eight blocks: the frontier is a
+// queue, eight lanes take a vertex, and a cluster barrier ends a level (about
+// 3.4 us, the chain of queue, row, neighbour and distance loads, instead of a
+// launch that looks at every vertex: 560 levels of a triangulation of 300,000
+// points take 2.0 ms, and took 3.5 ms of kernels and 0.9 ms between them).  It ends where the frontier is empty or wider than
+// kBfsNarrow, and leaves the level and the frontier's size behind.
+constexpr int kBfsCluster = 8, kBfsThreads = 1024, kBfsNarrow = 4096, kBfsLocal = 4096, kBfsLong = 256;
+
+struct BfsState {
+  int32_t level, width;
+  int32_t count[3];  // frontier sizes: of level l at l % 3
+};
+
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__global__ void __cluster_dims__(kBfsCluster, 1, 1) __launch_bounds__(kBfsThreads)
+    k_st_bfs_narrow(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int32_t* dist, int32_t* q0,
+                    int32_t* q1, BfsState* st, int64_t n) {
+  __shared__ int32_t s_out[kBfsLocal];
+  __shared__ int32_t s_long[64];
+  __shared__ int s_n, s_nlong, s_base;
+  const int rank = blockIdx.x;  // one cluster
+  const int sub = threadIdx.x & 7;
+  int level = *(volatile int32_t*)&st->level;
+  int width = 0;
+  for (;; level++) {
+    width = *(volatile int32_t*)&st->count[level % 3];
+    if (width == 0 || width > kBfsNarrow || level >= n) break;  // uniform over the cluster
+    if (threadIdx.x == 0) {
+      s_n = s_nlong = 0;
+      if (rank == 0) *(volatile int32_t*)&st->count[(level + 2) % 3] = 0;
+    }
+    __syncthreads();
+    const int32_t* in = (level & 1) ? q1 : q0;
+    int32_t* out = (level & 1) ? q0 : q1;
+    auto visit = [&](int32_t u) {
+      if (*(volatile int32_t*)&dist[u] >= 0 || atomicCAS(&dist[u], -1, level + 1) != -1) return;
+      const int at = atomicAdd(&s_n, 1);
+      if (at < kBfsLocal) s_out[at] = u;
+      else out[atomicAdd(&st->count[(level + 1) % 3], 1)] = u;
+    };
+    for (int i = (rank * kBfsThreads + (int)threadIdx.x) >> 3; i < width; i += kBfsCluster * kBfsThreads / 8) {
+      const int32_t v = __ldcg(in + i);
+      const int64_t b = row_ptr[v], e = row_ptr[v + 1];
+      if (e - b > kBfsLong) {  // a long row is shared by the whole block below
+        int at = 64;
+        if (sub == 0) at = atomicAdd(&s_nlong, 1);
+        at = __shfl_sync(0xffu << (threadIdx.x & 24), at, threadIdx.x & 24);  // the eight lanes of this vertex
+        if (at < 64) {
+          if (sub == 0) s_long[at] = v;
+          continue;
+        }
+      }
+      for (int64_t p = b + sub; p < e; p += 8) visit(col[p]);
+    }
+    __syncthreads();
+    for (int k = 0; k < min(s_nlong, 64); k++) {
+      const int32_t v = s_long[k];
+      for (int64_t p = row_ptr[v] + threadIdx.x; p < row_ptr[v + 1]; p += kBfsThreads) visit(col[p]);
+    }
+    __syncthreads();
+    const int mine = min(s_n, kBfsLocal);
+    if (threadIdx.x == 0 && mine) s_base = atomicAdd(&st->count[(level + 1) % 3], mine);
+    __syncthreads();
+    for (int i = threadIdx.x; i < mine; i += kBfsThreads) out[s_base + i] = s_out[i];
+    cluster_barrier();
+  }
+  if (rank == 0 && threadIdx.x == 0) {
+    st->level = level;
+    st->width = width;
+  }
+}
+
+// the frontier of `level` as a queue, after levels that were run over all vertices
+__global__ void k_st_bfs_collect(const int32_t* __restrict__ dist, int64_t n, int32_t level, int32_t* __restrict__ q0,
+                                 int32_t* __restrict__ q1, BfsState* st) {
+  int32_t* q = (level & 1) ? q1 : q0;
+  const int lane = threadIdx.x & 31;
+  if (blockIdx.x == 0 && threadIdx.x == 0) st->level = level;  // (the counts are zero)
+  for (int64_t v0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); v0 < n;
+       v0 += (int64_t)gridDim.x * blockDim.x) {  // warp-uniform
+    const int64_t v = v0 + lane;
+    const bool in = v < n && dist[v] == level;
+    const unsigned b = __ballot_sync(0xffffffffu, in);
+    if (!b) continue;
+    int at = 0;
+    if (lane == 0) at = atomicAdd(&st->count[level % 3], __popc(b));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (in) q[at + __popc(b & ((1u << lane) - 1))] = (int32_t)v;
+  }
 }
 
 __global__ void k_st_unreached(const int32_t* __restrict__ dist, int64_t n, int32_t* flag) {
@@ -89,88 +184,178 @@ __global__ void k_st_keys_weff(const int32_t* __restrict__ eu, const int32_t* __
   }
 }
 
-__global__ void k_st_iota(int32_t* __restrict__ a, int64_t n) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
-    a[v] = (int32_t)v;
+// ---- Boruvka over a shrinking list of the edges that still join two trees.
+// Every kernel of a round is bound by its random accesses (150 G sectors/s), so
+// what counts is how many edges a round touches: on mesh 128^3 (6.2 M edges, 11
+// rounds) 1.0 ms; all edges in every round, with the vertices relabelled by
+// pointer jumping in between, took 1.4 ms.
+
+// nxt is a union-find forest over the vertices: a tree's root points at itself
+__device__ __forceinline__ int32_t st_find(int32_t* nxt, int32_t v) {
+  int32_t r = v, p = nxt[r];
+  while (p != r) {
+    r = p;
+    p = nxt[r];
+  }
+  if (nxt[v] != r) nxt[v] = r;  // a shorter path for the next search; an ancestor either way
+  return r;
 }
 
-__global__ void k_st_reset_best(unsigned long long* __restrict__ bk, int32_t* __restrict__ bid, int64_t n) {
+__global__ void k_st_start(int32_t* __restrict__ nxt, unsigned long long* __restrict__ bk, int32_t* __restrict__ bid,
+                           int64_t n, int64_t* __restrict__ counts, int64_t m) {
+  if (blockIdx.x == 0 && threadIdx.x <= kStRounds) counts[threadIdx.x] = threadIdx.x == 0 ? m : 0;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
+    nxt[v] = (int32_t)v;
     bk[v] = 0;
     bid[v] = kNoEdge;
   }
 }
 
-__global__ void k_st_best_key(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
-                              const uint64_t* __restrict__ key, const int32_t* __restrict__ comp, int64_t m,
-                              unsigned long long* bk) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t cu = comp[eu[e]], cv = comp[ev[e]];
-    if (cu == cv) continue;
-    const unsigned long long k = key[e];
-    if (k > bk[cu]) atomicMax(&bk[cu], k);
-    if (k > bk[cv]) atomicMax(&bk[cv], k);
+// the edges of a round: the trees at their ends, key, canonical id (null: the place in the list)
+struct StEdges {
+  const int32_t* u;
+  const int32_t* v;
+  const uint64_t* key;
+  const int32_t* id;
+  const int64_t* count;
+  __device__ __forceinline__ int32_t id_of(int64_t i) const { return id ? id[i] : (int32_t)i; }
+};
+
+__global__ void k_st_best_key(StEdges e, unsigned long long* bk) {
+  const int64_t m = *e.count;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t u = e.u[i], v = e.v[i];
+    const unsigned long long k = e.key[i];
+    if (k > bk[u]) atomicMax(&bk[u], k);
+    if (k > bk[v]) atomicMax(&bk[v], k);
   }
 }
 
-__global__ void k_st_best_id(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
-                             const uint64_t* __restrict__ key, const int32_t* __restrict__ comp, int64_t m,
-                             const unsigned long long* __restrict__ bk, int32_t* bid) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t cu = comp[eu[e]], cv = comp[ev[e]];
-    if (cu == cv) continue;
-    const unsigned long long k = key[e];
-    if (k == bk[cu]) atomicMin(&bid[cu], (int32_t)e);
-    if (k == bk[cv]) atomicMin(&bid[cv], (int32_t)e);
+__global__ void k_st_best_id(StEdges e, const unsigned long long* __restrict__ bk, int32_t* bid) {
+  const int64_t m = *e.count;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t u = e.u[i], v = e.v[i];
+    const unsigned long long k = e.key[i];
+    if (k == bk[u]) atomicMin(&bid[u], e.id_of(i));
+    if (k == bk[v]) atomicMin(&bid[v], e.id_of(i));
   }
 }
 
-// every component root hooks across its chosen edge; the edge joins the tree
-__global__ void k_st_hook(const int32_t* __restrict__ comp, const int32_t* __restrict__ bid,
-                          const int32_t* __restrict__ eu, const int32_t* __restrict__ ev, int64_t n,
-                          int32_t* __restrict__ nxt, uint8_t* __restrict__ tflag, int32_t* hooks) {
-  int any = 0;
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
-    if (comp[c] != (int32_t)c) continue;
-    const int32_t e = bid[c];
-    if (e == kNoEdge) {
-      nxt[c] = (int32_t)c;
-      continue;
-    }
-    const int32_t cu = comp[eu[e]], cv = comp[ev[e]];
-    const int32_t other = (cu == (int32_t)c) ? cv : cu;
-    tflag[e] = 1;
-    any = 1;
-    // two components that chose the same edge: the smaller id stays a root
-    nxt[c] = (bid[other] == e && (int32_t)c < other) ? (int32_t)c : other;
+// Every tree hooks across its chosen edge, which joins the forest; of two trees
+// that chose the same edge the smaller id stays a root (a strict order allows
+// no longer cycle).  A tree's edge is one entry of the list, so that entry does
+// the hooking.
+__global__ void k_st_hook(StEdges e, const int32_t* __restrict__ bid, int32_t* __restrict__ nxt,
+                          uint8_t* __restrict__ tflag) {
+  const int64_t m = *e.count;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t u = e.u[i], v = e.v[i], id = e.id_of(i);
+    const bool bu = bid[u] == id, bv = bid[v] == id;
+    if (!bu && !bv) continue;
+    tflag[id] = 1;
+    if (bu && !(bv && u < v)) nxt[u] = v;
+    if (bv && !(bu && v < u)) nxt[v] = u;
   }
-  if (__any_sync(0xffffffffu, any) && (threadIdx.x & 31) == 0) *hooks = 1;
 }
 
-// pointer jumping over the hooks (in place: a jump only shortens a path)
-__global__ void k_st_jump(const int32_t* __restrict__ comp, int32_t* nxt, int64_t n, int32_t* changed) {
-  int any = 0;
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
-    if (comp[c] != (int32_t)c) continue;
-    const int32_t a = nxt[c];
-    const int32_t b = nxt[a];
-    if (a != b) {
-      nxt[c] = b;
-      any = 1;
-    }
-  }
-  if (__any_sync(0xffffffffu, any) && (threadIdx.x & 31) == 0) *changed = 1;
-}
-
-__global__ void k_st_relabel(int32_t* comp, const int32_t* __restrict__ nxt, int64_t n) {
+// Every vertex points at its root, and the roots' choices are reset (worth a pass while the edges outnumber the
+// vertices: each of an edge's two searches is then one load, and it writes nothing at random).
+__global__ void k_st_compress(int32_t* nxt, int64_t n, unsigned long long* __restrict__ bk, int32_t* __restrict__ bid) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
-    comp[v] = nxt[comp[v]];
+    if (st_find(nxt, (int32_t)v) == (int32_t)v) {
+      bk[v] = 0;
+      bid[v] = kNoEdge;
+    }
 }
 
-__global__ void k_st_comp_root(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ comp, int64_t n,
-                               unsigned long long* rk) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
-    atomicMax(&rk[comp[v]], degree_key(row_ptr, v));
+// The edges that still join two trees, with those trees' roots; without a
+// k_st_compress before it, the roots' choices are reset here (roots without
+// such an edge take no part any more).  A block's survivors are one run of the
+// next list.
+__global__ void __launch_bounds__(kBlock) k_st_filter(StEdges e, int32_t* nxt, int32_t* __restrict__ ou,
+                                                      int32_t* __restrict__ ov, uint64_t* __restrict__ okey,
+                                                      int32_t* __restrict__ oid, int64_t* count,
+                                                      bool reset, unsigned long long* __restrict__ bk,
+                                                      int32_t* __restrict__ bid) {
+  __shared__ int sm[kBlock / 32 + 1];
+  __shared__ unsigned long long s_base;
+  const int64_t m = *e.count;
+  constexpr int kPer = 4;
+  for (int64_t i0 = (int64_t)blockIdx.x * kBlock * kPer; i0 < m; i0 += (int64_t)gridDim.x * kBlock * kPer) {
+    int32_t u[kPer], v[kPer];
+    int mine = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; k++) {
+      const int64_t i = i0 + k * kBlock + threadIdx.x;
+      u[k] = v[k] = -1;
+      if (i < m) {
+        const int32_t a = st_find(nxt, e.u[i]), b = st_find(nxt, e.v[i]);
+        if (a != b) {
+          u[k] = a;
+          v[k] = b;
+          mine++;
+          if (reset) {
+            bk[a] = 0;
+            bk[b] = 0;
+            bid[a] = kNoEdge;
+            bid[b] = kNoEdge;
+          }
+        }
+      }
+    }
+    int tot;
+    int at = block_excl_scan(mine, sm, &tot);
+    if (threadIdx.x == 0) s_base = tot ? atomicAdd((unsigned long long*)count, (unsigned long long)tot) : 0;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kPer; k++) {
+      if (u[k] < 0) continue;
+      const int64_t i = i0 + k * kBlock + threadIdx.x, o = (int64_t)s_base + at++;
+      ou[o] = u[k];
+      ov[o] = v[k];
+      okey[o] = e.key[i];
+      oid[o] = e.id_of(i);
+    }
+    __syncthreads();
+  }
+}
+
+// the root of every vertex's tree, and its vertex of maximum degree: a thread keeps the maximum while the tree stays
+// the same, and a block whose threads all end in one tree makes one addition to its word (mesh 128^3, one tree: 24 us;
+// an addition per vertex, all to that word, took 1340)
+__global__ void __launch_bounds__(kBlock) k_st_comp_root(const int64_t* __restrict__ row_ptr, int32_t* nxt,
+                                                         int32_t* __restrict__ comp, int64_t n, unsigned long long* rk) {
+  __shared__ unsigned long long s_best;
+  __shared__ int32_t s_comp;
+  __shared__ int s_mixed;
+  int32_t cur = -1;
+  unsigned long long best = 0;
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t c = st_find(nxt, (int32_t)v);
+    comp[v] = c;
+    if (c != cur) {
+      if (cur >= 0) atomicMax(&rk[cur], best);
+      cur = c;
+      best = 0;
+    }
+    best = max(best, degree_key(row_ptr, v));
+  }
+  if (threadIdx.x == 0) {
+    s_best = 0;
+    s_comp = cur;
+    s_mixed = 0;
+  }
+  __syncthreads();
+  if (cur >= 0 && cur != s_comp) s_mixed = 1;
+  __syncthreads();
+  if (s_mixed) {
+    if (cur >= 0) atomicMax(&rk[cur], best);
+    return;
+  }
+  for (int o = 16; o; o >>= 1) best = max(best, __shfl_down_sync(0xffffffffu, best, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(&s_best, best);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_comp >= 0) atomicMax(&rk[s_comp], s_best);
 }
 
 __device__ __forceinline__ bool is_root(const int32_t* __restrict__ comp, const unsigned long long* __restrict__ rk,
@@ -182,13 +367,13 @@ __device__ __forceinline__ bool is_root(const int32_t* __restrict__ comp, const 
 // root's first arc
 __global__ void k_st_cut(const int32_t* __restrict__ comp, const unsigned long long* __restrict__ rk,
                          const int64_t* __restrict__ tptr, const int32_t* __restrict__ tdeg,
-                         const int32_t* __restrict__ rev, int64_t n, int32_t* __restrict__ succ,
-                         int32_t* __restrict__ rd) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-    if (tdeg[v] == 0 || !is_root(comp, rk, v)) continue;
-    const int32_t tail = rev[tptr[v] + tdeg[v] - 1];
-    succ[tail] = -1;
-    rd[tail] = 0;
+                         const int32_t* __restrict__ rev, int64_t n, int32_t* __restrict__ succ, RankSpace r) {
+  for (int64_t v0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); v0 < n;
+       v0 += (int64_t)gridDim.x * blockDim.x) {  // warp-uniform
+    const int64_t v = v0 + (threadIdx.x & 31);
+    const bool root = v < n && tdeg[v] > 0 && is_root(comp, rk, v);
+    if (root) succ[rev[tptr[v] + tdeg[v] - 1]] = -1;
+    rank_add_head(root, root ? (int32_t)tptr[v] : 0, r.heads, r.n_heads);
   }
 }
 
@@ -196,12 +381,12 @@ __global__ void k_st_cut(const int32_t* __restrict__ comp, const unsigned long l
 // from the parent to the child
 __global__ void k_st_parent(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
                             const uint8_t* __restrict__ tflag, const int32_t* __restrict__ arc_uv,
-                            const int32_t* __restrict__ rev, const int32_t* __restrict__ rd, int64_t m,
-                            int32_t* __restrict__ parent) {
+                            const int32_t* __restrict__ rev, const uint64_t* __restrict__ own,
+                            const uint64_t* __restrict__ walk, int64_t m, int32_t* __restrict__ parent) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
     if (!tflag[e]) continue;
     const int32_t a = arc_uv[e];
-    if (rd[a] > rd[rev[a]]) parent[ev[e]] = eu[e];
+    if (arc_rank(own, walk, a) > arc_rank(own, walk, rev[a])) parent[ev[e]] = eu[e];
     else parent[eu[e]] = ev[e];
   }
 }
@@ -232,8 +417,12 @@ int spanning_tree(Handle& h, int tree_kind, int32_t* parent) {
   };
   uint64_t* key = nullptr;
   int32_t *comp = nullptr, *nxt = nullptr, *bid = nullptr, *dist = nullptr, *tdeg = nullptr, *cur = nullptr;
-  int32_t *tadj = nullptr, *rev = nullptr, *arc_uv = nullptr, *succ[2] = {nullptr, nullptr};
-  int32_t *rd[2] = {nullptr, nullptr}, *flags = nullptr;
+  int32_t *tadj = nullptr, *rev = nullptr, *arc_uv = nullptr, *succ = nullptr, *flags = nullptr;
+  int32_t *lu[2] = {nullptr, nullptr}, *lv[2] = {nullptr, nullptr}, *lid[2] = {nullptr, nullptr};
+  uint64_t* lkey[2] = {nullptr, nullptr};
+  int64_t* counts = nullptr;
+  BfsState* bfs = nullptr;
+  RankSpace rank;
   unsigned long long *bk = nullptr, *rk = nullptr;
   uint8_t* tflag = nullptr;
   int64_t* tptr = nullptr;
@@ -241,9 +430,11 @@ int spanning_tree(Handle& h, int tree_kind, int32_t* parent) {
   const int64_t A = 2 * std::max<int64_t>(n - 1, 0);  // arcs of a spanning forest, at most
   if (!talloc(&key, m) || !talloc(&comp, n) || !talloc(&nxt, n) || !talloc(&bid, n) || !talloc(&bk, n) ||
       !talloc(&rk, n) || !talloc(&tflag, m) || !talloc(&tdeg, n) || !talloc(&cur, n) || !talloc(&tptr, n + 1) ||
-      !talloc(&tadj, A) || !talloc(&rev, A) || !talloc(&arc_uv, m) || !talloc(&succ[0], A) || !talloc(&succ[1], A) ||
-      !talloc(&rd[0], A) || !talloc(&rd[1], A) || !talloc(&flags, 64) ||
-      (tree_kind == PDG_TREE_FEGRASS && !talloc(&dist, n))) {
+      !talloc(&tadj, A) || !talloc(&rev, A) || !talloc(&arc_uv, m) || !talloc(&succ, A) ||
+      !rank_space(rank, A, std::max<int64_t>(n / 2, 1), s, talloc) || !talloc(&flags, 64) ||
+      !talloc(&counts, kStRounds + 1) || !talloc(&lu[0], m) || !talloc(&lv[0], m) || !talloc(&lid[0], m) ||
+      !talloc(&lkey[0], m) || !talloc(&lu[1], m) || !talloc(&lv[1], m) || !talloc(&lid[1], m) || !talloc(&lkey[1], m) ||
+      (tree_kind == PDG_TREE_FEGRASS && (!talloc(&dist, n) || !talloc(&bfs, 1)))) {
     cudaGetLastError();
     cleanup();
     return PDG_E_OOM;
@@ -270,20 +461,33 @@ int spanning_tree(Handle& h, int tree_kind, int32_t* parent) {
       return fail(PDG_E_CUDA);
     const int32_t root = (int32_t)(0xffffffffull - (bh & 0xffffffffull));
     const int64_t maxdeg = (int64_t)(bh >> 32);
-    // unweighted BFS distances from the root, 16 levels per host check
+    // unweighted BFS distances from the root: narrow frontiers in one kernel, wide ones level by level over all
+    // vertices, 16 levels per host check
     ST_CK(cudaMemsetAsync(dist, 0xff, sizeof(int32_t) * n, s));
     ST_CK(cudaMemsetAsync(dist + root, 0, sizeof(int32_t), s));
+    BfsState* hst = reinterpret_cast<BfsState*>(h.hsc);
     bool done = false;
-    for (int64_t level = 0; level <= n && !done; level += 16) {
+    int32_t level = 0;
+    while (!done) {
+      if (level > n) return fail(PDG_E_CUDA);
+      ST_CK(cudaMemsetAsync(bfs, 0, sizeof(BfsState), s));
+      k_st_bfs_collect<<<gn, kBlock, 0, s>>>(dist, n, level, nxt, comp, bfs);
+      k_st_bfs_narrow<<<kBfsCluster, kBfsThreads, 0, s>>>(h.row_ptr, h.col, dist, nxt, comp, bfs, n);
+      if (cudaMemcpyAsync(hst, bfs, sizeof(BfsState), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+          cudaStreamSynchronize(s) != cudaSuccess)
+        return fail(PDG_E_CUDA);
+      level = hst->level;
+      if (hst->width == 0) break;
       ST_CK(cudaMemsetAsync(flags, 0, sizeof(int32_t) * 16, s));
-      for (int i = 0; i < 16; i++) k_st_bfs<<<gn, kBlock, 0, s>>>(h.row_ptr, h.col, n, dist, (int32_t)(level + i), flags + i);
+      for (int i = 0; i < 16; i++) k_st_bfs<<<gn, kBlock, 0, s>>>(h.row_ptr, h.col, n, dist, level + i, flags + i);
       if (!read_flags(16)) return fail(PDG_E_CUDA);
       done = hflags[15] == 0;
+      level += 16;
     }
     ST_CK(cudaMemsetAsync(flags, 0, sizeof(int32_t), s));
     k_st_unreached<<<gn, kBlock, 0, s>>>(dist, n, flags);
     if (!read_flags(1)) return fail(PDG_E_CUDA);
-    if (!done || hflags[0]) return fail(PDG_E_INVALID_ARG);  // not connected
+    if (hflags[0]) return fail(PDG_E_INVALID_ARG);  // not connected
     // log of the degrees, from the host math library (one table, both sides of every comparison)
     std::vector<double> lh((size_t)maxdeg + 1, 0.0);
     for (int64_t d = 1; d <= maxdeg; d++) lh[d] = std::log((double)d);
@@ -294,35 +498,33 @@ int spanning_tree(Handle& h, int tree_kind, int32_t* parent) {
   } else {
     k_st_keys_weight<<<gm, kBlock, 0, s>>>(h.el_w, m, key);
   }
-  // 2. Boruvka rounds
-  k_st_iota<<<gn, kBlock, 0, s>>>(comp, n);
+  // 2. Boruvka rounds; the host looks at the number of edges left every few rounds
+  k_st_start<<<gn, kBlock, 0, s>>>(nxt, bk, bid, n, counts, m);
   ST_CK(cudaMemsetAsync(tflag, 0, (size_t)std::max<int64_t>(m, 1), s));
-  bool merged_all = false;
-  for (int round = 0; round < 64; round++) {
-    k_st_reset_best<<<gn, kBlock, 0, s>>>(bk, bid, n);
-    k_st_best_key<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, key, comp, m, bk);
-    k_st_best_id<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, key, comp, m, bk, bid);
-    ST_CK(cudaMemsetAsync(flags, 0, sizeof(int32_t), s));
-    k_st_hook<<<gn, kBlock, 0, s>>>(comp, bid, h.el_u, h.el_v, n, nxt, tflag, flags);
-    if (!read_flags(1)) return fail(PDG_E_CUDA);
-    if (hflags[0] == 0) {
-      merged_all = true;
-      break;
+  int64_t left = m;
+  for (int round = 0; left > 0; round++) {
+    if (round >= kStRounds) return fail(PDG_E_CUDA);  // every round at least halves the trees
+    const int i = round & 1;
+    const StEdges e = round == 0 ? StEdges{h.el_u, h.el_v, key, nullptr, counts}
+                                 : StEdges{lu[i], lv[i], lkey[i], lid[i], counts + round};
+    const int gl = grid_for(h, left);
+    k_st_best_key<<<gl, kBlock, 0, s>>>(e, bk);
+    k_st_best_id<<<gl, kBlock, 0, s>>>(e, bk, bid);
+    k_st_hook<<<gl, kBlock, 0, s>>>(e, bid, nxt, tflag);
+    const bool pass = left > n;
+    if (pass) k_st_compress<<<gn, kBlock, 0, s>>>(nxt, n, bk, bid);
+    k_st_filter<<<gl, kBlock, 0, s>>>(e, nxt, lu[i ^ 1], lv[i ^ 1], lkey[i ^ 1], lid[i ^ 1], counts + round + 1, !pass, bk,
+                                      bid);
+    if (round < 2 || round % 3 == 1) {
+      if (cudaMemcpyAsync(h.hsc, counts + round + 1, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+          cudaStreamSynchronize(s) != cudaSuccess)
+        return fail(PDG_E_CUDA);
+      left = *reinterpret_cast<int64_t*>(h.hsc);
     }
-    bool flat = false;
-    for (int it = 0; it < 64 && !flat; it += 4) {
-      ST_CK(cudaMemsetAsync(flags, 0, sizeof(int32_t) * 4, s));
-      for (int i = 0; i < 4; i++) k_st_jump<<<gn, kBlock, 0, s>>>(comp, nxt, n, flags + i);
-      if (!read_flags(4)) return fail(PDG_E_CUDA);
-      flat = hflags[3] == 0;
-    }
-    if (!flat) return fail(PDG_E_CUDA);
-    k_st_relabel<<<gn, kBlock, 0, s>>>(comp, nxt, n);
   }
-  if (!merged_all) return fail(PDG_E_CUDA);
   // 3. roots, tree adjacency, Euler tour
   ST_CK(cudaMemsetAsync(rk, 0, sizeof(unsigned long long) * n, s));
-  k_st_comp_root<<<gn, kBlock, 0, s>>>(h.row_ptr, comp, n, rk);
+  k_st_comp_root<<<std::min(gn, h.num_sms * 4), kBlock, 0, s>>>(h.row_ptr, nxt, comp, n, rk);
   ST_CK(cudaMemsetAsync(tdeg, 0, sizeof(int32_t) * n, s));
   ST_CK(cudaMemsetAsync(cur, 0, sizeof(int32_t) * n, s));
   k_st_tdeg<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, tflag, m, tdeg);
@@ -336,17 +538,11 @@ int spanning_tree(Handle& h, int tree_kind, int32_t* parent) {
   }
   k_st_fill<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, tflag, m, tptr, cur, tadj, rev, arc_uv);
   const int ga = grid_for(h, std::max<int64_t>(A, 1));
-  k_st_succ<<<ga, kBlock, 0, s>>>(tadj, rev, tptr, tdeg, n, succ[0], rd[0]);
-  k_st_cut<<<gn, kBlock, 0, s>>>(comp, rk, tptr, tdeg, rev, n, succ[0], rd[0]);
-  int bits = 1;
-  while ((1ll << bits) <= A) bits++;
-  int c = 0;
-  for (int r = 0; r < bits; r++) {
-    k_st_rank<<<ga, kBlock, 0, s>>>(succ[c], rd[c], succ[c ^ 1], rd[c ^ 1], tptr, n);
-    c ^= 1;
-  }
+  k_st_succ<<<ga, kBlock, 0, s>>>(tadj, rev, tptr, tdeg, n, succ);
+  k_st_cut<<<gn, kBlock, 0, s>>>(comp, rk, tptr, tdeg, rev, n, succ, rank);
+  const uint64_t* walk = rank_lists(h, succ, tptr + n, rank, s);
   ST_CK(cudaMemsetAsync(parent, 0xff, sizeof(int32_t) * n, s));
-  k_st_parent<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, tflag, arc_uv, rev, rd[c], m, parent);
+  k_st_parent<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, tflag, arc_uv, rev, rank.own, walk, m, parent);
   if (cudaGetLastError() != cudaSuccess) return fail(PDG_E_CUDA);
   cleanup();
   return PDG_OK;
