@@ -27,38 +27,70 @@ __global__ void k_val_rowptr(const int64_t* __restrict__ row_ptr, int64_t n, Dev
     if (row_ptr[u] > row_ptr[u + 1]) atomicOr(&dsc->err, ERR_NOT_CSR);
 }
 
-// Every thread takes kValRun consecutive entries: one search for the row of the
-// first, then the row advances with the entries.
-constexpr int kValRun = 8;
+// Every warp takes kValRun * 32 consecutive entries: one search for the row of
+// the first, then 32 entries at a time, each lane finding its row among the
+// next 32 row ends (one coalesced load, five shuffles).  Only the entries above
+// the diagonal look for their mirror image: distinct ones have distinct images
+// below it (rows are strictly increasing), so the matrix is symmetric when all
+// are found and there are as many entries below as above (dsc->active counts
+// the difference).  Bound by those searches: 12.5 M entries of mesh 128^3 take
+// 195 us; a search for every entry, a thread taking eight in a row, took 260.
+constexpr int kValRun = 16;
 
 __global__ void __launch_bounds__(kBlock) k_val_entries(const int64_t* __restrict__ row_ptr,
                                                         const int32_t* __restrict__ col,
                                                         const double* __restrict__ w, int64_t n, int64_t nnz,
                                                         const int64_t* __restrict__ vtx_ptr, int32_t G,
                                                         DevScalars* dsc) {
+  __shared__ int s_diff;
+  if (threadIdx.x == 0) s_diff = 0;
+  __syncthreads();
   const double lo = ldexp(1.0, -900), hi = ldexp(1.0, 900);
-  int err = 0;
-  for (int64_t p0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kValRun; p0 < nnz;
-       p0 += (int64_t)gridDim.x * blockDim.x * kValRun) {
-    int64_t u = row_of(row_ptr, n, p0);
-    for (int64_t p = p0; p < p0 + kValRun && p < nnz; p++) {
-    while (row_ptr[u + 1] <= p) u++;  // empty rows are passed over (row_ptr is monotone: checked before)
-    const int32_t v = col[p];
-    const double x = w[p];
-    if (!(x >= lo && x <= hi)) err |= ERR_BAD_WEIGHT;
-    if (v < 0 || v >= n || v == u) {
-      err |= ERR_NOT_CSR;
-      continue;
-    }
-    if (p + 1 < row_ptr[u + 1] && !(col[p + 1] > v)) err |= ERR_NOT_CSR;
-    if (graph_of_vertex(vtx_ptr, G, u) != graph_of_vertex(vtx_ptr, G, v)) err |= ERR_CROSS_GRAPH;
-    const int64_t b = row_ptr[v], e = row_ptr[v + 1];
-    const int64_t q = lower_bound_i32(col, b, e, (int32_t)u);
-    if (q >= e || col[q] != (int32_t)u || __double_as_longlong(w[q]) != __double_as_longlong(x))
-      err |= ERR_NOT_SYMMETRIC;
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  int err = 0, diff = 0;
+  for (int64_t p0 = warp * 32 * kValRun; p0 < nnz; p0 += warps * 32 * kValRun) {
+    int64_t row = row_of(row_ptr, n, p0);  // of the round's first entry
+    for (int64_t b0 = p0; b0 < min(nnz, p0 + 32 * kValRun); b0 += 32) {
+      const int64_t p = b0 + lane;
+      const bool in = p < nnz;
+      // the row ends after this row's start; an entry's row lies as many rows on as ends are not beyond it
+      const int64_t end = row + 1 + lane <= n ? row_ptr[row + 1 + lane] : nnz;
+      int k = 0;
+#pragma unroll
+      for (int o = 16; o; o >>= 1)
+        if (__shfl_sync(0xffffffffu, end, k + o - 1) <= p) k += o;
+      int64_t u = row + k, u_end = __shfl_sync(0xffffffffu, end, k);
+      const int32_t v = in ? col[p] : 0;
+      int32_t next = __shfl_down_sync(0xffffffffu, v, 1);
+      if (in) {
+        while (u_end <= p) u_end = row_ptr[++u + 1];  // past many empty rows (row_ptr is monotone: checked before)
+        if (lane == 31 && p + 1 < nnz) next = col[p + 1];
+        const double x = w[p];
+        if (!(x >= lo && x <= hi)) err |= ERR_BAD_WEIGHT;
+        if (v < 0 || v >= n || v == u) {
+          err |= ERR_NOT_CSR;
+        } else {
+          if (p + 1 < u_end && !(next > v)) err |= ERR_NOT_CSR;
+          if (graph_of_vertex(vtx_ptr, G, u) != graph_of_vertex(vtx_ptr, G, v)) err |= ERR_CROSS_GRAPH;
+          diff += u < v ? 1 : -1;
+          if (u < v) {
+            const int64_t b = row_ptr[v], e = row_ptr[v + 1];
+            const int64_t q = lower_bound_i32(col, b, e, (int32_t)u);
+            if (q >= e || col[q] != (int32_t)u || __double_as_longlong(w[q]) != __double_as_longlong(x))
+              err |= ERR_NOT_SYMMETRIC;
+          }
+        }
+      }
+      row = __shfl_sync(0xffffffffu, u, 31);  // (not used after a round that ends the entries)
     }
   }
   if (err) atomicOr(&dsc->err, err);
+  diff = __reduce_add_sync(0xffffffffu, diff);
+  if (lane == 0 && diff) atomicAdd(&s_diff, diff);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_diff) atomicAdd((unsigned long long*)&dsc->active, (unsigned long long)(long long)s_diff);
 }
 
 __global__ void k_val_parent(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
@@ -151,7 +183,8 @@ int validate_csr(Handle& h) {
   if (h.hsc->err) return PDG_E_NOT_CSR;  // the entry checks below search rows: only on a monotone row_ptr
   if (h.nnz > 0) k_val_entries<<<grid, kBlock, 0, h.stream>>>(h.row_ptr, h.col, h.w, n, h.nnz, h.d_vtx_ptr, h.G, h.dsc);
   if (!fetch()) return check_cuda(cudaGetLastError());
-  const int err = h.hsc->err;
+  int err = h.hsc->err;
+  if (h.hsc->active != 0) err |= ERR_NOT_SYMMETRIC;
   if (err & ERR_NOT_CSR) return PDG_E_NOT_CSR;
   if (err & ERR_BAD_WEIGHT) return PDG_E_BAD_WEIGHT;
   if (err & ERR_CROSS_GRAPH) return PDG_E_INVALID_ARG;
@@ -201,6 +234,7 @@ int validate_graph(Handle& h, bool acyclic) {
     return check_cuda(cudaGetLastError());
   }
   int err = h.hsc->err;
+  if (h.hsc->active != 0) err |= ERR_NOT_SYMMETRIC;
   for (int64_t r : roots_h)
     if (r != 1) err |= ERR_NOT_A_TREE;
   if (acyclic && !(err & (ERR_NOT_CSR | ERR_BAD_WEIGHT | ERR_NOT_A_TREE | ERR_CROSS_GRAPH))) {
