@@ -396,6 +396,7 @@ void sparsifier_free(pdg_handle hp) {
   }
   if (h.gstream) cudaStreamDestroy(h.gstream);
   pinned_release(h.hsc, sizeof(DevScalars));
+  pinned_release(h.pcg_host, sizeof(double) * kPcgParts);
   HostStage& s = hp->stage;
   const size_t G = (size_t)std::max(s.G, 1);
   pinned_release(s.sel, sizeof(GraphSel) * G);
@@ -489,7 +490,7 @@ int sparsify_batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_
       cudaMemcpyAsync(h.d_vtx_ptr, vtx_ptr, sizeof(int64_t) * (num_graphs + 1), cudaMemcpyHostToDevice, h.stream) !=
           cudaSuccess)
     return fail(PDG_E_CUDA);
-  if ((st = validate_graph(h, false))) return fail(st);  // acyclicity, depth and range: build_tree_layout
+  if ((st = validate_graph(h))) return fail(st);  // acyclicity, depth and range: build_tree_layout
   // per-graph edge counts from the row offsets at the graph boundaries
   std::vector<int64_t> rp_at(num_graphs + 1);
   {
@@ -671,7 +672,9 @@ static int pcg_entry(int64_t n, const int64_t* row_ptr, const int32_t* col, cons
   const int64_t vp[2] = {0, n};
   int32_t* d_ids = nullptr;
   double* d_b = nullptr;
-  if (!(h.hsc = static_cast<DevScalars*>(pinned_alloc(sizeof(DevScalars))))) return fail(PDG_E_OOM);
+  if (!(h.hsc = static_cast<DevScalars*>(pinned_alloc(sizeof(DevScalars)))) ||
+      !(h.pcg_host = static_cast<double*>(pinned_alloc(sizeof(double) * kPcgParts))))
+    return fail(PDG_E_OOM);
   if ((st = alloc_n(h, &h.dsc, 1)) || (st = alloc_n(h, &h.row_ptr, n + 1)) || (st = alloc_n(h, &h.col, h.nnz)) ||
       (st = alloc_n(h, &h.w, h.nnz)) || (st = alloc_n(h, &h.parent, n)) || (st = alloc_n(h, &h.d_vtx_ptr, 2)) ||
       (st = alloc_n(h, &h.blk_a, 10240)) || (st = alloc_n(h, &h.blk_b, 2048)) ||
@@ -685,7 +688,7 @@ static int pcg_entry(int64_t n, const int64_t* row_ptr, const int32_t* col, cons
       cudaMemcpyAsync(d_b, b, sizeof(double) * n, kind, h.stream) != cudaSuccess ||
       cudaMemcpyAsync(h.d_vtx_ptr, vp, sizeof(vp), cudaMemcpyHostToDevice, h.stream) != cudaSuccess)
     return fail(PDG_E_CUDA);
-  if ((st = validate_graph(h, true))) return fail(st);
+  if ((st = validate_graph(h))) return fail(st);  // acyclicity, depth and range: pcg_quality
   if ((st = alloc_n(h, &h.el_u, std::max<int64_t>(h.m, 1))) || (st = alloc_n(h, &h.el_v, std::max<int64_t>(h.m, 1))) ||
       (st = alloc_n(h, &h.el_w, std::max<int64_t>(h.m, 1))) || (st = build_edge_list(h)))
     return fail(st);

@@ -3,6 +3,7 @@
 // the device helpers they share and the handle layout.
 #pragma once
 
+#include <climits>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -85,7 +86,7 @@ struct DevScalars {
   int64_t max_seg;      // largest subtask
   int64_t big_regs;     // registrations the cooperative tier will make
   int64_t undecided;    // cooperative tier: still undecided after a round
-  int64_t active;       // validation: vertices whose pointer jump is not done
+  int64_t active;       // validation: entries above the diagonal minus entries below
   int64_t max_depth;
   int32_t radix_sel;    // radix sort: which ping-pong buffer holds the keys
   int32_t radix_skip;   // radix sort: the current digit is uniform
@@ -102,6 +103,13 @@ struct DevScalars {
   unsigned long long join_conf;   // join: (marker, candidate) pairs found
   int64_t finish_left;  // cooperative tier: candidates the rounds left to the serial finisher
 };
+
+// the fixed-point range of exact root distances: 2^(e_max - e_min + 53) per edge, `depth` edges
+inline bool exact_range(const DevScalars& d, int64_t depth) {
+  int bits = 0;
+  while ((1ll << bits) <= depth) bits++;
+  return d.e_max == INT_MIN || d.e_max - d.e_min + 53 + bits <= 96;
+}
 
 // Programmatic dependent launch.  A kernel started by launch_k may be put on
 // the SMs as the kernel before it on the stream drains (its blocks exiting),
@@ -309,6 +317,7 @@ struct Handle {
 
   DevScalars* dsc = nullptr;   // device
   DevScalars* hsc = nullptr;   // pinned host mirror
+  double* pcg_host = nullptr;  // pinned: kPcgParts sums of the PCG measure
   int64_t stats[12] = {0};
   int64_t launches = 0;  // kernels launched by the current recovery
   // CUDA-graph replay of a whole recovery (opt.use_graph)
@@ -543,7 +552,7 @@ int scan_excl_u32(Handle& h, const uint32_t* in, int64_t* out, const int64_t* n_
 int scan_excl_u8(Handle& h, const uint8_t* in, int64_t* out, const int64_t* n_dev, int64_t n_max);
 
 // steps
-int validate_graph(Handle& h, bool acyclic);    // input checks; acyclic: also acyclicity, max depth, range
+int validate_graph(Handle& h);  // input checks; the tours check acyclicity and range
 int build_edge_list(Handle& h);                 // init: canonical edge list from the CSR
 int build_tree_layout(Handle& h);               // init: preorder labels, Euler tour, relabelled edges and parents
 int tree_scan_workspace(Handle& h);             // init: look-back space of the tree scan
@@ -557,6 +566,7 @@ int accept_setup();                             // per-device kernel attributes 
 int coop_rounds(const Handle& h, int c);        // cooperative-tier rounds the next recovery launches
 int validate_csr(Handle& h);                    // CSR shape, symmetry and weights only
 int spanning_tree(Handle& h, int tree_kind, int32_t* parent);  // parent array of the generated tree (device)
+constexpr int kPcgParts = 256;
 constexpr int64_t kPcgMaxEdges = 8192;  // recovered edges of the PCG quality measure (dense k x k capacitance)
 // device ids and b; host results (hist: nullable, the relative residual after each iteration;
 // z0: nullable, the preconditioner applied to the centred right-hand side, n values)

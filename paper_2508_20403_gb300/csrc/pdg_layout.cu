@@ -267,11 +267,8 @@ int build_tree_layout(Handle& h) {
     LAY_CK(cudaMemcpyAsync(h.hsc, h.dsc, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
     LAY_CK(cudaStreamSynchronize(s));
     if (hbad) return fail(PDG_E_NOT_A_TREE);  // the parent links are not a tree the tour covers (a cycle)
-    // the fixed-point range of the exact root distances: 2^(e_max - e_min + 53) per edge, max_depth edges
     h.max_depth = h.hsc->max_depth;
-    int dep_bits = 0;
-    while ((1ll << dep_bits) <= h.max_depth) dep_bits++;
-    if (h.hsc->e_max != INT_MIN && h.hsc->e_max - h.hsc->e_min + 53 + dep_bits > 96) return fail(PDG_E_RANGE);
+    if (!exact_range(*h.hsc, h.max_depth)) return fail(PDG_E_RANGE);
   }
   LAY_CK(cudaMemsetAsync(h.wup, 0, sizeof(double) * n, s));
   if (m > 0) k_lay_edges<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, h.el_w, pre_of, parent_pre, m, h.wup);
