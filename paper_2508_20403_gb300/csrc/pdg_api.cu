@@ -65,7 +65,7 @@ int device_alloc(Handle& h, void** p, size_t bytes) {
   return PDG_OK;
 }
 
-static void device_release(Handle& h, void* p) {
+void device_release(Handle& h, void* p) {
   if (!p) return;
   auto it = std::find(h.allocs.begin(), h.allocs.end(), p);
   if (it != h.allocs.end()) h.allocs.erase(it);
@@ -183,7 +183,7 @@ int ensure_scan_status(Handle& h, int64_t n_max) {
   const int64_t tiles = (std::max<int64_t>(n_max, 1) + kTile - 1) / kTile;
   if (h.scan_ctr == nullptr) {
     int st = alloc_n(h, &h.scan_ctr, 2);
-    if (st) return st;
+    if (st || (st = alloc_n(h, &h.scan_sums, kScanSums))) return st;
     PDG_CUDA(cudaMemsetAsync(h.scan_ctr, 0, 2 * sizeof(uint32_t), h.stream));
   }
   if (tiles <= h.scan_tiles_cap) return PDG_OK;

@@ -201,6 +201,8 @@ struct Handle {
   double* rtree = nullptr;  // r(v) = fl(1/w(v, parent v))
   int64_t* blk_a = nullptr; // per-block counters (classification, scans)
   int64_t* blk_b = nullptr;
+  int32_t* up_count = nullptr;  // validation: entries above the diagonal, per chunk of kValChunk entries
+  int64_t* up_off = nullptr;    // and before it
 
   // per label one 32-byte record: P(x) = D(x) * 2^32 + depth(x) (u128; D = exact root distance in units of
   // 2^-S), then of the parent array, inside the label's 32-label group: minimum up to it, minimum after it,
@@ -271,6 +273,7 @@ struct Handle {
   uint32_t* radix_counters = nullptr;  // per pass: tile ticket (and one spare word)
   uint64_t* scan_status = nullptr;     // single-pass scan: flag | value per tile, zero between scans
   uint32_t* scan_ctr = nullptr;        // single-pass scan: tile ticket, blocks finished
+  int64_t* scan_sums = nullptr;        // two-launch scan: [kScanSums] tile sums
   int64_t scan_tiles_cap = 0;
   uint32_t* radix_dtot = nullptr;      // 256
   // records in (lca, rank) order
@@ -545,6 +548,7 @@ struct DepScope {
 
 // device-wide exclusive scan: out[i] = sum in[0..i), out[N] = total.
 // N may live on the device (n_dev != nullptr) or be given on the host.
+constexpr int kScanSums = 4096;
 int ensure_scan_status(Handle& h, int64_t n_max);  // scans of up to n_max elements can run
 int scan_excl_i64(Handle& h, const int64_t* in, int64_t* out, int64_t n_host, const int64_t* n_dev, int64_t n_max);
 int scan_excl_i32(Handle& h, const int32_t* in, int64_t* out, int64_t n_host, const int64_t* n_dev, int64_t n_max);
@@ -553,7 +557,7 @@ int scan_excl_u8(Handle& h, const uint8_t* in, int64_t* out, const int64_t* n_de
 
 // steps
 int validate_graph(Handle& h);  // input checks; the tours check acyclicity and range
-int build_edge_list(Handle& h);                 // init: canonical edge list from the CSR
+int build_edge_list(Handle& h);                 // init: canonical edge list from the CSR, after validation
 int build_tree_layout(Handle& h);               // init: preorder labels, Euler tour, relabelled edges and parents
 int tree_scan_workspace(Handle& h);             // init: look-back space of the tree scan
 int step_resist(Handle& h);                     // A1: r of the tree edges (off-tree edges: told apart in A3)
@@ -581,5 +585,6 @@ int grow_join(Handle& h);
 int grow_list(Handle& h, int64_t entries);
 int grow_tables(Handle& h, int64_t slots, int64_t xblocks);
 int device_alloc(Handle& h, void** p, size_t bytes);
+void device_release(Handle& h, void* p);
 
 }  // namespace pdg

@@ -63,53 +63,82 @@ __global__ void k_st_bfs(const int64_t* __restrict__ row_ptr, const int32_t* __r
   if (__any_sync(0xffffffffu, any) && (threadIdx.x & 31) == 0) *grew = 1;
 }
 
-// Levels of narrow frontiers in one cluster of eight blocks: the frontier is a
-// queue, eight lanes take a vertex, and a cluster barrier ends a level (about
-// 3.4 us, the chain of queue, row, neighbour and distance loads, instead of a
-// launch that looks at every vertex: 560 levels of a triangulation of 300,000
-// points take 2.0 ms, and took 3.5 ms of kernels and 0.9 ms between them).  It ends where the frontier is empty or wider than
-// kBfsNarrow, and leaves the level and the frontier's size behind.
-constexpr int kBfsCluster = 8, kBfsThreads = 1024, kBfsNarrow = 4096, kBfsLocal = 4096, kBfsLong = 256;
+// Levels of narrow frontiers in one cluster of 16 blocks, or eight where 16 do
+// not fit together.  Every block keeps
+// what it discovers in a queue in its shared memory; the next level's vertices
+// are the blocks' queues one after another, read across the cluster, eight lanes
+// to a vertex.  A cluster barrier ends a level, and the queues' lengths go with
+// it.  A level costs the chain of loads from queue, row and neighbours, the
+// compare-and-swap and the barrier, 2.0 us on average (with the queue and its length in
+// global memory, and the distance looked at before the swap, 3.4 us; a launch
+// that looks at every vertex took 6).  It ends where the frontier is empty or
+// wider than kBfsNarrow; the distances then say what the frontier is.
+constexpr int kBfsThreads = 512, kBfsNarrow = 4096, kBfsLong = 256;
 
 struct BfsState {
   int32_t level, width;
-  int32_t count[3];  // frontier sizes: of level l at l % 3
 };
 
 __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-__global__ void __cluster_dims__(kBfsCluster, 1, 1) __launch_bounds__(kBfsThreads)
-    k_st_bfs_narrow(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int32_t* dist, int32_t* q0,
-                    int32_t* q1, BfsState* st, int64_t n) {
-  __shared__ int32_t s_out[kBfsLocal];
+// the address that a block's own shared variable has in block `rank` of the cluster
+__device__ __forceinline__ uint32_t cluster_address(const void* own, int rank) {
+  uint32_t at;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(own)), "r"(rank));
+  return at;
+}
+
+template <int kBfsCluster>
+__global__ void __launch_bounds__(kBfsThreads)
+    k_st_bfs_narrow(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int32_t* dist,
+                    const int32_t* __restrict__ first, BfsState* st) {
+  __shared__ int32_t s_queue[2][kBfsNarrow];       // of level l: l & 1
+  __shared__ int32_t s_count[2][kBfsCluster];      // lengths of all blocks' queues
   __shared__ int32_t s_long[64];
-  __shared__ int s_n, s_nlong, s_base;
+  __shared__ int s_n, s_nlong;
   const int rank = blockIdx.x;  // one cluster
   const int sub = threadIdx.x & 7;
-  int level = *(volatile int32_t*)&st->level;
-  int width = 0;
+  int level = st->level, width = st->width;
+  if (width == 0 || width > kBfsNarrow) return;  // (all blocks)
+  {
+    const int share = (width + kBfsCluster - 1) / kBfsCluster, p = level & 1;
+    if (threadIdx.x < kBfsCluster) s_count[p][threadIdx.x] = max(0, min(share, width - (int)threadIdx.x * share));
+    for (int i = threadIdx.x; i < share && rank * share + i < width; i += kBfsThreads)
+      s_queue[p][i] = first[rank * share + i];
+  }
+  __syncthreads();
+  cluster_barrier();
   for (;; level++) {
-    width = *(volatile int32_t*)&st->count[level % 3];
-    if (width == 0 || width > kBfsNarrow || level >= n) break;  // uniform over the cluster
-    if (threadIdx.x == 0) {
-      s_n = s_nlong = 0;
-      if (rank == 0) *(volatile int32_t*)&st->count[(level + 2) % 3] = 0;
+    const int p = level & 1;
+    int end[kBfsCluster];  // of the blocks' parts of the frontier
+    width = 0;
+#pragma unroll
+    for (int b = 0; b < kBfsCluster; b++) {
+      width += s_count[p][b];
+      end[b] = width;
     }
+    if (width == 0 || width > kBfsNarrow) break;  // uniform over the cluster
+    if (threadIdx.x == 0) s_n = s_nlong = 0;
     __syncthreads();
-    const int32_t* in = (level & 1) ? q1 : q0;
-    int32_t* out = (level & 1) ? q0 : q1;
     auto visit = [&](int32_t u) {
-      if (*(volatile int32_t*)&dist[u] >= 0 || atomicCAS(&dist[u], -1, level + 1) != -1) return;
+      if (atomicCAS(&dist[u], -1, level + 1) != -1) return;
       const int at = atomicAdd(&s_n, 1);
-      if (at < kBfsLocal) s_out[at] = u;
-      else out[atomicAdd(&st->count[(level + 1) % 3], 1)] = u;
+      if (at < kBfsNarrow) s_queue[p ^ 1][at] = u;  // (a longer queue ends the loop)
     };
     for (int i = (rank * kBfsThreads + (int)threadIdx.x) >> 3; i < width; i += kBfsCluster * kBfsThreads / 8) {
-      const int32_t v = __ldcg(in + i);
-      const int64_t b = row_ptr[v], e = row_ptr[v + 1];
-      if (e - b > kBfsLong) {  // a long row is shared by the whole block below
+      int b = 0, before = 0;
+#pragma unroll
+      for (int k = 0; k < kBfsCluster - 1; k++)
+        if (i >= end[k]) {
+          b = k + 1;
+          before = end[k];
+        }
+      int32_t v;
+      asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(cluster_address(&s_queue[p][i - before], b)) : "memory");
+      const int64_t r0 = row_ptr[v], r1 = row_ptr[v + 1];
+      if (r1 - r0 > kBfsLong) {  // a long row is shared by the whole block below
         int at = 64;
         if (sub == 0) at = atomicAdd(&s_nlong, 1);
         at = __shfl_sync(0xffu << (threadIdx.x & 24), at, threadIdx.x & 24);  // the eight lanes of this vertex
@@ -118,19 +147,18 @@ __global__ void __cluster_dims__(kBfsCluster, 1, 1) __launch_bounds__(kBfsThread
           continue;
         }
       }
-      for (int64_t p = b + sub; p < e; p += 8) visit(col[p]);
+      for (int64_t q = r0 + sub; q < r1; q += 8) visit(col[q]);
     }
     __syncthreads();
     for (int k = 0; k < min(s_nlong, 64); k++) {
       const int32_t v = s_long[k];
-      for (int64_t p = row_ptr[v] + threadIdx.x; p < row_ptr[v + 1]; p += kBfsThreads) visit(col[p]);
+      for (int64_t q = row_ptr[v] + threadIdx.x; q < row_ptr[v + 1]; q += kBfsThreads) visit(col[q]);
     }
     __syncthreads();
-    const int mine = min(s_n, kBfsLocal);
-    if (threadIdx.x == 0 && mine) s_base = atomicAdd(&st->count[(level + 1) % 3], mine);
-    __syncthreads();
-    for (int i = threadIdx.x; i < mine; i += kBfsThreads) out[s_base + i] = s_out[i];
-    cluster_barrier();
+    if (threadIdx.x < kBfsCluster)
+      asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cluster_address(&s_count[p ^ 1][rank], threadIdx.x)), "r"(s_n)
+                   : "memory");
+    cluster_barrier();  // the last access to another block's memory lies before it
   }
   if (rank == 0 && threadIdx.x == 0) {
     st->level = level;
@@ -138,12 +166,33 @@ __global__ void __cluster_dims__(kBfsCluster, 1, 1) __launch_bounds__(kBfsThread
   }
 }
 
-// the frontier of `level` as a queue, after levels that were run over all vertices
-__global__ void k_st_bfs_collect(const int32_t* __restrict__ dist, int64_t n, int32_t level, int32_t* __restrict__ q0,
-                                 int32_t* __restrict__ q1, BfsState* st) {
-  int32_t* q = (level & 1) ? q1 : q0;
+template <int CLUSTER>
+cudaError_t launch_bfs_narrow(const Handle& h, int32_t* dist, const int32_t* first, BfsState* st, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = CLUSTER;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.gridDim = dim3(CLUSTER);
+  cfg.blockDim = dim3(kBfsThreads);
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  const int64_t* row_ptr = h.row_ptr;
+  const int32_t* col = h.col;
+  if (CLUSTER > 8) {  // more than every device takes
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_st_bfs_narrow<CLUSTER>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaLaunchKernelEx(&cfg, k_st_bfs_narrow<CLUSTER>, row_ptr, col, dist, first, st);
+}
+
+// the frontier of `level` as a queue, as far as it goes in there (st->width is zero)
+__global__ void k_st_bfs_collect(const int32_t* __restrict__ dist, int64_t n, int32_t level, int32_t* __restrict__ queue,
+                                 BfsState* st) {
   const int lane = threadIdx.x & 31;
-  if (blockIdx.x == 0 && threadIdx.x == 0) st->level = level;  // (the counts are zero)
+  if (blockIdx.x == 0 && threadIdx.x == 0) st->level = level;
   for (int64_t v0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); v0 < n;
        v0 += (int64_t)gridDim.x * blockDim.x) {  // warp-uniform
     const int64_t v = v0 + lane;
@@ -151,9 +200,9 @@ __global__ void k_st_bfs_collect(const int32_t* __restrict__ dist, int64_t n, in
     const unsigned b = __ballot_sync(0xffffffffu, in);
     if (!b) continue;
     int at = 0;
-    if (lane == 0) at = atomicAdd(&st->count[level % 3], __popc(b));
+    if (lane == 0) at = atomicAdd(&st->width, __popc(b));
     at = __shfl_sync(0xffffffffu, at, 0);
-    if (in) q[at + __popc(b & ((1u << lane) - 1))] = (int32_t)v;
+    if (in) queue[at + __popc(b & ((1u << lane) - 1))] = (int32_t)v;
   }
 }
 
@@ -471,8 +520,11 @@ int spanning_tree(Handle& h, int tree_kind, int32_t* parent) {
     while (!done) {
       if (level > n) return fail(PDG_E_CUDA);
       ST_CK(cudaMemsetAsync(bfs, 0, sizeof(BfsState), s));
-      k_st_bfs_collect<<<gn, kBlock, 0, s>>>(dist, n, level, nxt, comp, bfs);
-      k_st_bfs_narrow<<<kBfsCluster, kBfsThreads, 0, s>>>(h.row_ptr, h.col, dist, nxt, comp, bfs, n);
+      k_st_bfs_collect<<<gn, kBlock, 0, s>>>(dist, n, level, nxt, bfs);
+      if (launch_bfs_narrow<16>(h, dist, nxt, bfs, s) != cudaSuccess) {
+        cudaGetLastError();
+        ST_CK(launch_bfs_narrow<8>(h, dist, nxt, bfs, s));
+      }
       if (cudaMemcpyAsync(hst, bfs, sizeof(BfsState), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
           cudaStreamSynchronize(s) != cudaSuccess)
         return fail(PDG_E_CUDA);
@@ -511,7 +563,7 @@ int spanning_tree(Handle& h, int tree_kind, int32_t* parent) {
     k_st_best_key<<<gl, kBlock, 0, s>>>(e, bk);
     k_st_best_id<<<gl, kBlock, 0, s>>>(e, bk, bid);
     k_st_hook<<<gl, kBlock, 0, s>>>(e, bid, nxt, tflag);
-    const bool pass = left > n;
+    const bool pass = left > n / 2;
     if (pass) k_st_compress<<<gn, kBlock, 0, s>>>(nxt, n, bk, bid);
     k_st_filter<<<gl, kBlock, 0, s>>>(e, nxt, lu[i ^ 1], lv[i ^ 1], lkey[i ^ 1], lid[i ^ 1], counts + round + 1, !pass, bk,
                                       bid);

@@ -33,15 +33,51 @@ __global__ void k_val_rowptr(const int64_t* __restrict__ row_ptr, int64_t n, Dev
 // the diagonal look for their mirror image: distinct ones have distinct images
 // below it (rows are strictly increasing), so the matrix is symmetric when all
 // are found and there are as many entries below as above (dsc->active counts
-// the difference).  Bound by those searches: 12.5 M entries of mesh 128^3 take
-// 195 us; a search for every entry, a thread taking eight in a row, took 260.
-constexpr int kValRun = 16;
+// the difference).  Bound by the latency of those searches (eight blocks an SM, 32
+// registers, against seven: 150 us, 270): 12.5 M entries of mesh 128^3 take 150
+// us; a search for every entry, a thread taking eight in a row, took 260.
+// The count of the entries above the diagonal in every chunk goes to the
+// canonical edge list, which is made of them.
+constexpr int kValRun = 16, kValChunk = 32 * kValRun;
 
-__global__ void __launch_bounds__(kBlock) k_val_entries(const int64_t* __restrict__ row_ptr,
+// Row of CSR entry p (largest u with row_ptr[u] <= p), found by one warp with
+// 32-way splits: about log32(n) dependent loads instead of log2(n).
+__device__ __forceinline__ int64_t warp_row_of(const int64_t* __restrict__ row_ptr, int64_t n, int64_t p) {
+  const int lane = threadIdx.x & 31;
+  int64_t lo = 0, hi = n;  // row_ptr[lo] <= p < row_ptr[hi]
+  while (hi - lo > 1) {
+    const int64_t step = (hi - lo + 31) / 32;
+    const int64_t q = lo + lane * step;
+    const bool ok = q < hi && __ldg(row_ptr + q) <= p;
+    const int last = 31 - __clz(__ballot_sync(0xffffffffu, ok));  // lane 0 is always ok
+    lo += last * step;
+    hi = min(hi, lo + step);
+  }
+  return lo;
+}
+
+// Row of entry p = (round's first entry) + lane, for a round whose first entry lies in `row`: its row lies as many rows
+// on as of the next 32 row ends are not beyond it.  *u_end: where that row ends (for p < nnz).
+__device__ __forceinline__ int64_t warp_entry_row(const int64_t* __restrict__ row_ptr, int64_t n, int64_t nnz,
+                                                  int64_t row, int64_t p, int64_t* u_end) {
+  const int lane = threadIdx.x & 31;
+  const int64_t end = row + 1 + lane <= n ? row_ptr[row + 1 + lane] : nnz;
+  int k = 0;
+#pragma unroll
+  for (int o = 16; o; o >>= 1)
+    if (__shfl_sync(0xffffffffu, end, k + o - 1) <= p) k += o;
+  int64_t u = row + k;
+  *u_end = __shfl_sync(0xffffffffu, end, k);
+  if (p < nnz)
+    while (*u_end <= p) *u_end = row_ptr[++u + 1];  // past many empty rows (row_ptr is monotone: checked before)
+  return u;
+}
+
+__global__ void __launch_bounds__(kBlock, 8) k_val_entries(const int64_t* __restrict__ row_ptr,
                                                         const int32_t* __restrict__ col,
                                                         const double* __restrict__ w, int64_t n, int64_t nnz,
                                                         const int64_t* __restrict__ vtx_ptr, int32_t G,
-                                                        DevScalars* dsc) {
+                                                        int32_t* __restrict__ up_count, DevScalars* dsc) {
   __shared__ int s_diff;
   if (threadIdx.x == 0) s_diff = 0;
   __syncthreads();
@@ -50,22 +86,17 @@ __global__ void __launch_bounds__(kBlock) k_val_entries(const int64_t* __restric
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int err = 0, diff = 0;
-  for (int64_t p0 = warp * 32 * kValRun; p0 < nnz; p0 += warps * 32 * kValRun) {
-    int64_t row = row_of(row_ptr, n, p0);  // of the round's first entry
-    for (int64_t b0 = p0; b0 < min(nnz, p0 + 32 * kValRun); b0 += 32) {
+  for (int64_t p0 = warp * kValChunk; p0 < nnz; p0 += warps * kValChunk) {
+    int64_t row = warp_row_of(row_ptr, n, p0);  // of the round's first entry
+    int up = 0;
+    for (int64_t b0 = p0; b0 < min(nnz, p0 + kValChunk); b0 += 32) {
       const int64_t p = b0 + lane;
       const bool in = p < nnz;
-      // the row ends after this row's start; an entry's row lies as many rows on as ends are not beyond it
-      const int64_t end = row + 1 + lane <= n ? row_ptr[row + 1 + lane] : nnz;
-      int k = 0;
-#pragma unroll
-      for (int o = 16; o; o >>= 1)
-        if (__shfl_sync(0xffffffffu, end, k + o - 1) <= p) k += o;
-      int64_t u = row + k, u_end = __shfl_sync(0xffffffffu, end, k);
+      int64_t u_end;
+      const int64_t u = warp_entry_row(row_ptr, n, nnz, row, p, &u_end);
       const int32_t v = in ? col[p] : 0;
       int32_t next = __shfl_down_sync(0xffffffffu, v, 1);
       if (in) {
-        while (u_end <= p) u_end = row_ptr[++u + 1];  // past many empty rows (row_ptr is monotone: checked before)
         if (lane == 31 && p + 1 < nnz) next = col[p + 1];
         const double x = w[p];
         if (!(x >= lo && x <= hi)) err |= ERR_BAD_WEIGHT;
@@ -76,6 +107,7 @@ __global__ void __launch_bounds__(kBlock) k_val_entries(const int64_t* __restric
           if (graph_of_vertex(vtx_ptr, G, u) != graph_of_vertex(vtx_ptr, G, v)) err |= ERR_CROSS_GRAPH;
           diff += u < v ? 1 : -1;
           if (u < v) {
+            up++;
             const int64_t b = row_ptr[v], e = row_ptr[v + 1];
             const int64_t q = lower_bound_i32(col, b, e, (int32_t)u);
             if (q >= e || col[q] != (int32_t)u || __double_as_longlong(w[q]) != __double_as_longlong(x))
@@ -85,12 +117,48 @@ __global__ void __launch_bounds__(kBlock) k_val_entries(const int64_t* __restric
       }
       row = __shfl_sync(0xffffffffu, u, 31);  // (not used after a round that ends the entries)
     }
+    up = __reduce_add_sync(0xffffffffu, up);
+    if (lane == 0) up_count[p0 / kValChunk] = up;
   }
   if (err) atomicOr(&dsc->err, err);
   diff = __reduce_add_sync(0xffffffffu, diff);
   if (lane == 0 && diff) atomicAdd(&s_diff, diff);
   __syncthreads();
   if (threadIdx.x == 0 && s_diff) atomicAdd((unsigned long long*)&dsc->active, (unsigned long long)(long long)s_diff);
+}
+
+// The canonical edge list: every entry above the diagonal in row-major order, which is the entries' order, so a warp
+// appends the ones of its chunk (columns in range, as many as counted: validated).  Reads the CSR once and writes the
+// list, 250 MB for mesh 128^3: 68 us (with a thread's loads eight entries apart and a second pass over the columns to
+// count, 133).
+__global__ void __launch_bounds__(kBlock) k_edge_list(const int64_t* __restrict__ row_ptr,
+                                                      const int32_t* __restrict__ col, const double* __restrict__ w,
+                                                      int64_t n, int64_t nnz, const int64_t* __restrict__ up_off,
+                                                      int32_t* __restrict__ eu, int32_t* __restrict__ ev,
+                                                      double* __restrict__ ew) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t p0 = warp * kValChunk; p0 < nnz; p0 += warps * kValChunk) {
+    int64_t row = warp_row_of(row_ptr, n, p0), at = up_off[p0 / kValChunk];
+    for (int64_t b0 = p0; b0 < min(nnz, p0 + kValChunk); b0 += 32) {
+      const int64_t p = b0 + lane;
+      const int32_t v = p < nnz ? col[p] : 0;
+      const double x = p < nnz ? w[p] : 0.0;
+      int64_t u_end;
+      const int64_t u = warp_entry_row(row_ptr, n, nnz, row, p, &u_end);
+      const bool up = p < nnz && u < v;
+      const unsigned b = __ballot_sync(0xffffffffu, up);
+      if (up) {
+        const int64_t o = at + __popc(b & ((1u << lane) - 1));
+        eu[o] = (int32_t)u;
+        ev[o] = v;
+        ew[o] = x;
+      }
+      at += __popc(b);
+      row = __shfl_sync(0xffffffffu, u, 31);
+    }
+  }
 }
 
 __global__ void k_val_parent(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
@@ -137,6 +205,33 @@ __global__ void k_val_reset(DevScalars* dsc) {
 
 }  // namespace
 
+static int64_t entry_chunks(const Handle& h) { return (h.nnz + kValChunk - 1) / kValChunk; }
+
+static int entry_grid(const Handle& h) { return grid_for(h, 32 * entry_chunks(h)); }
+
+static int alloc_chunks(Handle& h) {
+  int st = device_alloc(h, reinterpret_cast<void**>(&h.up_count), sizeof(int32_t) * (size_t)entry_chunks(h));
+  if (!st)
+    st = device_alloc(h, reinterpret_cast<void**>(&h.up_off), sizeof(int64_t) * (size_t)(entry_chunks(h) + 1));
+  return st;
+}
+
+int build_edge_list(Handle& h) {
+  if (h.nnz == 0) return PDG_OK;
+  const int64_t chunks = entry_chunks(h);
+  int st = ensure_scan_status(h, chunks);
+  if (st || (st = scan_excl_i32(h, h.up_count, h.up_off, chunks, nullptr, chunks))) return st;
+  ++h.launches;
+  k_edge_list<<<entry_grid(h), kBlock, 0, h.stream>>>(h.row_ptr, h.col, h.w, h.n, h.nnz, h.up_off, h.el_u, h.el_v,
+                                                      h.el_w);
+  PDG_CUDA(cudaGetLastError());
+  device_release(h, h.up_count);
+  device_release(h, h.up_off);
+  h.up_count = nullptr;
+  h.up_off = nullptr;
+  return PDG_OK;
+}
+
 // The CSR checks alone (spanning-tree generation has no parent array yet).
 int validate_csr(Handle& h) {
   const int64_t n = h.n;
@@ -149,7 +244,11 @@ int validate_csr(Handle& h) {
   k_val_rowptr<<<grid, kBlock, 0, h.stream>>>(h.row_ptr, n, h.dsc);
   if (!fetch()) return check_cuda(cudaGetLastError());
   if (h.hsc->err) return PDG_E_NOT_CSR;  // the entry checks below search rows: only on a monotone row_ptr
-  if (h.nnz > 0) k_val_entries<<<grid, kBlock, 0, h.stream>>>(h.row_ptr, h.col, h.w, n, h.nnz, h.d_vtx_ptr, h.G, h.dsc);
+  if (h.nnz > 0) {
+    if (const int st = alloc_chunks(h)) return st;
+    k_val_entries<<<entry_grid(h), kBlock, 0, h.stream>>>(h.row_ptr, h.col, h.w, n, h.nnz, h.d_vtx_ptr, h.G, h.up_count,
+                                                          h.dsc);
+  }
   if (!fetch()) return check_cuda(cudaGetLastError());
   int err = h.hsc->err;
   if (h.hsc->active != 0) err |= ERR_NOT_SYMMETRIC;
@@ -172,7 +271,11 @@ int validate_graph(Handle& h) {
   k_val_rowptr<<<grid, kBlock, 0, h.stream>>>(h.row_ptr, n, h.dsc);
   if (!fetch()) return check_cuda(cudaGetLastError());
   if (h.hsc->err) return PDG_E_NOT_CSR;
-  if (h.nnz > 0) k_val_entries<<<grid, kBlock, 0, h.stream>>>(h.row_ptr, h.col, h.w, n, h.nnz, h.d_vtx_ptr, h.G, h.dsc);
+  if (h.nnz > 0) {
+    if (const int st = alloc_chunks(h)) return st;
+    k_val_entries<<<entry_grid(h), kBlock, 0, h.stream>>>(h.row_ptr, h.col, h.w, n, h.nnz, h.d_vtx_ptr, h.G, h.up_count,
+                                                          h.dsc);
+  }
   int64_t* roots = nullptr;
   int st = PDG_OK;
   auto cleanup = [&]() { cudaFreeAsync(roots, h.stream); };
