@@ -65,7 +65,8 @@ typedef struct pdg_options {
      options shape decide only candidate sets whose cells are too full for it. */
   int32_t warp_tier_max;    /* subtasks with 2..warp_tier_max candidates get one warp each (<= 32) */
   int64_t k_override;       /* >= 0: use this budget instead of floor(alpha*|V|) */
-  double candidate_factor;  /* first candidate prefix holds about factor*k edges (>= 1) */
+  double candidate_factor;  /* first candidate prefix holds about factor*k edges (>= 1); with 1.5 or more, 3*k while k is
+                               small and no earlier recovery of the handle tells what does */
   int32_t max_rounds;       /* rounds of the cooperative (hash) tier before the serial finisher */
   int32_t use_graph;        /* 1: capture the recovery pipeline in a CUDA graph and replay it */
   int64_t spin_limit;       /* iteration bound of every device-side wait */

@@ -197,6 +197,8 @@ int ensure_scan_status(Handle& h, int64_t n_max) {
   return PDG_OK;
 }
 
+constexpr int64_t kFirstLong = 1 << 15;  // largest budget of a graph whose first prefix is 3 k
+
 static int ensure_tiers(Handle& h, int c);
 
 int ensure_candidates(Handle& h, int64_t R, int c) {
@@ -227,7 +229,9 @@ int ensure_candidates(Handle& h, int64_t R, int c) {
   }
   if ((st = ensure_scan_status(h, h.Rcap + 1))) return st;
   // the selection's list: a power of two of the scores, usually a few times the candidates
-  if (h.list_cap < std::min<int64_t>(Rmax, 4 * h.Rcap) && (st = grow_list(h, 4 * h.Rcap))) return st;
+  // (R-MAT graphs: 8 to 40 times, which an eighth of the edges holds; it is 1.5 bytes an edge)
+  const int64_t list = std::min(Rmax, std::max({4 * h.Rcap, Rmax / 8, (int64_t)1 << 19}));
+  if (h.list_cap < list && (st = grow_list(h, list))) return st;
   return h.tiered ? ensure_tiers(h, c) : PDG_OK;
 }
 
@@ -782,6 +786,8 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
   // budgets and initial prefix sizes
   std::vector<int64_t> kg(G), eoff(G);
   int64_t total_k = 0;
+  std::vector<int64_t> rung(G, 0), first_long(G, 0);  // factor * k; the longer first prefix of a call without memory
+  int64_t longer = 0;
   for (int32_t g = 0; g < G; g++) {
     const int64_t ng = h.vtx_ptr_h[g + 1] - h.vtx_ptr_h[g];
     eoff[g] = h.off_ptr_h[g + 1] - h.off_ptr_h[g];
@@ -800,12 +806,24 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
     total_k += take;
     int64_t want = (int64_t)std::ceil((double)k * h.opt.candidate_factor) + 32;
     if (want < k) want = k;
-    if (h.k_mem[g] == k && h.c_mem == c && h.mode_mem == h.opt.score_mode) want = std::max(want, h.want_mem[g]);
+    rung[g] = want;
+    const bool known = h.k_mem[g] == k && h.c_mem == c && h.mode_mem == h.opt.score_mode;
+    if (known) want = std::max(want, h.want_mem[g]);
+    else if (k <= kFirstLong && h.opt.candidate_factor >= 1.5) longer += (first_long[g] = std::max(want, 3 * k + 32)) - want;
     h.want_h[g] = std::min(want, eoff[g]);
     s.k[g] = k;
     s.out_ptr[g] = user_out_ptr[g];
   }
   s.out_ptr[G] = user_out_ptr[G];
+  // A first prefix that turns out too short costs a second attempt, some 200 us, and more candidates cost little while
+  // all of them are few (80,000-point triangulation, k = 4000: 12,000 candidates 200 us, 24,000 209; 8,300 to 16,600 of
+  // mesh 48^3 5 us more, 13,600 to 27,100 of R-MAT scale 17 35 us).  So a call without memory of an earlier one starts
+  // with 3 k, which does for triangulations, geometric graphs and resistance scores where 1.5 k does not; the memory is
+  // of the short prefix where that would have done.  Of large budgets more candidates cost as much as the attempt that
+  // they may save, and 1.5 k does for the largest meshes and R-MAT graphs: it stays their first prefix.
+  if (longer <= 2 * kFirstLong)
+    for (int32_t g = 0; g < G; g++)
+      if (first_long[g] > 0) h.want_h[g] = std::min(first_long[g], eoff[g]);
   const int64_t out_total = user_out_ptr[G];
   // output staging (device) when the caller's buffers are host memory
   int32_t* dev_ids = out_ids;
@@ -901,6 +919,7 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
       GraphSel& gs = s.sel[g];
       std::memset(&gs, 0, sizeof(gs));
       gs.want = h.want_h[g];
+      gs.rung = rung[g];
       gs.take_all = (h.want_h[g] >= eoff[g]) ? 1 : 0;
       need += gs.take_all ? eoff[g] : h.want_h[g];
       if (!gs.take_all) any_select = true;
@@ -947,7 +966,7 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
       continue;
     }
     if ((err & ERR_TABLE) && !h.tiered) {  // the cells outgrew the table
-      h.join_factor *= 2;
+      h.join_factor *= 4;
       if ((st = grow_join(h))) return st;
       first = false;
       continue;
@@ -983,12 +1002,12 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
     bool again = false;
     for (int32_t g = 0; g < G; g++)
       if (s.gstat[g] == G_RETRY) {
-        h.want_h[g] = std::min(eoff[g], std::max<int64_t>(h.want_h[g] * 4, 64));
+        h.want_h[g] = std::min(eoff[g], std::max<int64_t>(h.want_h[g] * 2, 64));  // 3 k mostly does
         again = true;
       }
     if (!again) {
       for (int32_t g = 0; g < G; g++) {
-        h.want_mem[g] = h.want_h[g];
+        h.want_mem[g] = s.gstat[g] == G_OK_SHORT ? std::min(rung[g], h.want_h[g]) : h.want_h[g];
         h.k_mem[g] = kg[g];
       }
       h.c_mem = c;

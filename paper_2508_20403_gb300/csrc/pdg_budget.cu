@@ -66,7 +66,9 @@ __global__ void __launch_bounds__(kBlock) k_budget_write(
   for (int64_t g = tid; g < G; g += nth) {
     const int64_t cnt = scan[cand_ptr[g + 1]] - scan[cand_ptr[g]];
     const int64_t k = kk[g];
-    gstat[g] = (cnt >= k) ? G_OK : (sel[g].take_all ? G_UNDER : G_RETRY);
+    const int64_t c0 = cand_ptr[g], c1 = cand_ptr[g + 1];
+    const bool short_does = scan[min(c1, c0 + sel[g].rung)] - scan[c0] >= k;
+    gstat[g] = (cnt >= k) ? (short_does ? G_OK_SHORT : G_OK) : (sel[g].take_all ? G_UNDER : G_RETRY);
     gcount[g] = min(cnt, k);
   }
   for (int64_t r = tid; r < N; r += nth) {

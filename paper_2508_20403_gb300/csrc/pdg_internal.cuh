@@ -61,7 +61,8 @@ enum : int {
 enum : uint8_t { ST_UNDECIDED = 0, ST_ACCEPTED = 1, ST_REJECTED = 2, ST_ACCEPTED_NEW = 3 };
 
 // per-graph outcome of the budget cut
-enum : int32_t { G_OK = 0, G_UNDER = 1, G_RETRY = 2 };
+// (G_OK_SHORT: a prefix of GraphSel::rung candidates would have done)
+enum : int32_t { G_OK = 0, G_UNDER = 1, G_RETRY = 2, G_OK_SHORT = 3 };
 
 // Scalars that kernels produce and the host reads back in one copy.
 // Errors that invalidate the current attempt: the host discards it (and
@@ -147,6 +148,7 @@ struct GraphSel {
   int32_t b1, b2;
   int32_t take_all;
   int32_t pad;
+  int64_t rung;     // candidate_factor * k
 };
 
 // What a captured recovery graph depends on besides the pinned parameters it
