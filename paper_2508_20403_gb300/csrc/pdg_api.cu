@@ -201,6 +201,56 @@ constexpr int64_t kFirstLong = 1 << 15;  // largest budget of a graph whose firs
 
 static int ensure_tiers(Handle& h, int c);
 
+// A device array of the caller's that kernels can read where it is (memory of another device, or of another kind, is
+// copied).
+static bool in_place(const Handle& h, const void* p, size_t alignment) {
+  cudaPointerAttributes a;
+  if (reinterpret_cast<uintptr_t>(p) % alignment) return false;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == h.device;
+}
+
+// From this many entries on, host weights are copied beside the work on the structure: 2^20 take 40 us to come, what
+// that costs more (the places of the mirror images, one more pass over the edges) some 10.  Mesh 128^3, 100 MB of
+// weights: init and recovery 2700 -> 2360 us.
+constexpr int64_t kLateWeights = 1 << 20;
+
+// The CSR arrays of an init (h.n, h.nnz set): the caller's own where kernels can read them, else copies.  They are only
+// read, in the order of h.stream, and not after the entry point has returned.
+static int take_csr(Handle& h, const int64_t* row_ptr, const int32_t* col, const double* w, int mem_kind) {
+  if (mem_kind == PDG_MEM_DEVICE && h.nnz > 0 && in_place(h, row_ptr, 8) && in_place(h, col, 4) && in_place(h, w, 8)) {
+    h.csr_borrowed = true;
+    h.row_ptr = const_cast<int64_t*>(row_ptr);
+    h.col = const_cast<int32_t*>(col);
+    h.w = const_cast<double*>(w);
+    return PDG_OK;
+  }
+  const cudaMemcpyKind kind = (mem_kind == PDG_MEM_HOST) ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
+  int st;
+  if ((st = alloc_n(h, &h.row_ptr, h.n + 1)) || (st = alloc_n(h, &h.col, h.nnz)) || (st = alloc_n(h, &h.w, h.nnz)))
+    return st;
+  if (cudaMemcpyAsync(h.row_ptr, row_ptr, sizeof(int64_t) * (h.n + 1), kind, h.stream) != cudaSuccess ||
+      (h.nnz && cudaMemcpyAsync(h.col, col, sizeof(int32_t) * h.nnz, kind, h.stream) != cudaSuccess) ||
+      (h.nnz && !h.w_pending && cudaMemcpyAsync(h.w, w, sizeof(double) * h.nnz, kind, h.stream) != cudaSuccess))
+    return PDG_E_CUDA;
+  return PDG_OK;
+}
+
+static void drop_csr(Handle& h) {
+  if (!h.csr_borrowed) {
+    device_release(h, h.row_ptr);
+    device_release(h, h.col);
+    if (!h.w_pending) device_release(h, h.w);
+  }
+  h.csr_borrowed = false;
+  h.row_ptr = nullptr;
+  h.col = nullptr;
+  if (!h.w_pending) h.w = nullptr;
+}
+
 int ensure_candidates(Handle& h, int64_t R, int c) {
   const int64_t Rmax = std::max<int64_t>(h.E_off, 1);
   R = std::min<int64_t>(std::max<int64_t>(R, 1), Rmax);
@@ -385,6 +435,7 @@ void sparsifier_free(pdg_handle hp) {
   int prev = 0;
   cudaGetDevice(&prev);
   cudaSetDevice(h.device);
+  if (h.sstream) cudaStreamSynchronize(h.sstream);  // weights may be on their way
   for (void* p : h.allocs) cudaFreeAsync(p, h.stream);
   h.allocs.clear();
   cudaStreamSynchronize(h.stream);  // pinned staging below may be reused at once
@@ -395,7 +446,6 @@ void sparsifier_free(pdg_handle hp) {
   if (h.ev_fork) cudaEventDestroy(h.ev_fork);
   if (h.ev_join) cudaEventDestroy(h.ev_join);
   if (h.sstream) {
-    cudaStreamSynchronize(h.sstream);
     cudaStreamDestroy(h.sstream);
   }
   if (h.gstream) cudaStreamDestroy(h.gstream);
@@ -483,17 +533,37 @@ int sparsify_batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_
   if (!(h.hsc = static_cast<DevScalars*>(pinned_alloc(sizeof(DevScalars))))) return fail(PDG_E_OOM);
   if ((st = alloc_n(h, &h.dsc, 1))) return fail(st);
   if (cudaMemsetAsync(h.dsc, 0, sizeof(DevScalars), h.stream) != cudaSuccess) return fail(PDG_E_CUDA);
-  if ((st = alloc_n(h, &h.row_ptr, n + 1)) || (st = alloc_n(h, &h.col, h.nnz)) || (st = alloc_n(h, &h.w, h.nnz)) ||
-      (st = alloc_n(h, &h.parent, n)) || (st = alloc_n(h, &h.d_vtx_ptr, num_graphs + 1)) ||
-      (st = alloc_n(h, &h.blk_a, 10240)) || (st = alloc_n(h, &h.blk_b, 2048)))
+  if (mem_kind == PDG_MEM_HOST && h.nnz >= kLateWeights && h.sstream) {
+    const size_t before = h.device_bytes;
+    h.w_pending = alloc_n(h, &h.w_mirror, h.nnz) == PDG_OK && alloc_n(h, &h.w_place, h.m) == PDG_OK;
+    h.device_bytes = before;  // (given back during init)
+    if (!h.w_pending) {  // no room for the places: the weights come first
+      cudaGetLastError();
+      device_release(h, h.w_mirror);
+      h.w_mirror = nullptr;
+    }
+  }
+  if ((st = alloc_n(h, &h.parent, n)) || (st = alloc_n(h, &h.d_vtx_ptr, num_graphs + 1)) ||
+      (st = alloc_n(h, &h.blk_a, 10240)) || (st = alloc_n(h, &h.blk_b, 2048)) ||
+      (st = take_csr(h, row_ptr, col, w, mem_kind)))
     return fail(st);
-  if (cudaMemcpyAsync(h.row_ptr, row_ptr, sizeof(int64_t) * (n + 1), kind, h.stream) != cudaSuccess ||
-      (h.nnz && cudaMemcpyAsync(h.col, col, sizeof(int32_t) * h.nnz, kind, h.stream) != cudaSuccess) ||
-      (h.nnz && cudaMemcpyAsync(h.w, w, sizeof(double) * h.nnz, kind, h.stream) != cudaSuccess) ||
-      cudaMemcpyAsync(h.parent, parent, sizeof(int32_t) * n, kind, h.stream) != cudaSuccess ||
+  if (cudaMemcpyAsync(h.parent, parent, sizeof(int32_t) * n, kind, h.stream) != cudaSuccess ||
       cudaMemcpyAsync(h.d_vtx_ptr, vtx_ptr, sizeof(int64_t) * (num_graphs + 1), cudaMemcpyHostToDevice, h.stream) !=
           cudaSuccess)
     return fail(PDG_E_CUDA);
+  if (h.w_pending && (cudaEventRecord(h.ev_fork, h.stream) != cudaSuccess ||
+                      cudaStreamWaitEvent(h.sstream, h.ev_fork, 0) != cudaSuccess ||
+                      cudaMemcpyAsync(h.w, w, sizeof(double) * h.nnz, kind, h.sstream) != cudaSuccess ||
+                      cudaEventRecord(h.ev_join, h.sstream) != cudaSuccess))
+    return fail(PDG_E_CUDA);
+  // weights that are refused come before what is wrong with the tree
+  auto fail_tree = [&](int code) {
+    if (h.w_pending && finish_weights(h) == PDG_OK &&
+        cudaMemcpyAsync(h.hsc, h.dsc, sizeof(DevScalars), cudaMemcpyDeviceToHost, h.stream) == cudaSuccess &&
+        cudaStreamSynchronize(h.stream) == cudaSuccess && late_weight_status(h) != PDG_OK)
+      code = late_weight_status(h);
+    return fail(code);
+  };
   if ((st = validate_graph(h))) return fail(st);  // acyclicity, depth and range: build_tree_layout
   // per-graph edge counts from the row offsets at the graph boundaries
   std::vector<int64_t> rp_at(num_graphs + 1);
@@ -512,19 +582,14 @@ int sparsify_batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_
   if ((st = alloc_n(h, &h.el_u, std::max<int64_t>(h.m, 1))) || (st = alloc_n(h, &h.el_v, std::max<int64_t>(h.m, 1))) ||
       (st = alloc_n(h, &h.el_w, std::max<int64_t>(h.m, 1))) || (st = build_edge_list(h)))
     return fail(st);
-  device_release(h, h.row_ptr);
-  device_release(h, h.col);
-  device_release(h, h.w);
-  h.row_ptr = nullptr;
-  h.col = nullptr;
-  h.w = nullptr;
+  drop_csr(h);
   h.edge_ptr_h.assign(num_graphs + 1, 0);
   h.off_ptr_h.assign(num_graphs + 1, 0);
   for (int32_t g = 0; g < num_graphs; g++) {
     const int64_t entries = rp_at[g + 1] - rp_at[g];
-    if (entries % 2) return fail(PDG_E_NOT_SYMMETRIC);
+    if (entries % 2) return fail_tree(PDG_E_NOT_SYMMETRIC);
     const int64_t mg = entries / 2, ng = vtx_ptr[g + 1] - vtx_ptr[g];
-    if (mg < ng - 1) return fail(PDG_E_NOT_A_TREE);
+    if (mg < ng - 1) return fail_tree(PDG_E_NOT_A_TREE);
     h.edge_ptr_h[g + 1] = h.edge_ptr_h[g] + mg;
     h.off_ptr_h[g + 1] = h.off_ptr_h[g] + (mg - ng + 1);
   }
@@ -544,7 +609,8 @@ int sparsify_batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_
       (st = ensure_scan_status(h, std::max<int64_t>(n, num_graphs) + 1)))
     return fail(st);
   // the tree's layout: preorder labels, Euler tour, the relabelled edge list, parents and tree weights
-  if ((st = build_tree_layout(h)) || (st = tree_scan_workspace(h))) return fail(st);
+  if ((st = build_tree_layout(h))) return fail_tree(st);
+  if ((st = tree_scan_workspace(h))) return fail(st);
   HostStage& s = hp->stage;
   s.G = num_graphs;
   s.sel = static_cast<GraphSel*>(pinned_alloc(sizeof(GraphSel) * num_graphs));
@@ -560,8 +626,13 @@ int sparsify_batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_
       cudaMemsetAsync(h.hist, 0, sizeof(uint32_t) * (size_t)num_graphs * kSelBins, h.stream) != cudaSuccess ||
       cudaMemsetAsync(h.radix_dtot, 0, sizeof(uint32_t) * 256, h.stream) != cudaSuccess ||
       cudaMemsetAsync(h.radix_hist, 0, sizeof(uint32_t) * kRadixHistWords, h.stream) != cudaSuccess ||
+      (h.w_late && cudaMemcpyAsync(h.hsc, h.dsc, sizeof(DevScalars), cudaMemcpyDeviceToHost, h.stream) != cudaSuccess) ||
       cudaStreamSynchronize(h.stream) != cudaSuccess)
     return fail(PDG_E_CUDA);
+  if (h.w_late) {
+    if ((st = late_weight_status(h))) return fail(st);
+    if (!exact_range(*h.hsc, h.max_depth)) return fail(PDG_E_RANGE);
+  }
   h.want_h.assign(num_graphs, 0);
   h.want_mem.assign(num_graphs, 0);
   h.k_mem.assign(num_graphs, -1);
@@ -590,7 +661,6 @@ int pdg_spanning_tree(int64_t n, const int64_t* row_ptr, const int32_t* col, con
     sparsifier_free(hp);
     return code;
   };
-  const cudaMemcpyKind kind = (mem_kind == PDG_MEM_HOST) ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   int64_t ends[2];
   if (mem_kind == PDG_MEM_HOST) {
     ends[0] = row_ptr[0];
@@ -609,14 +679,11 @@ int pdg_spanning_tree(int64_t n, const int64_t* row_ptr, const int32_t* col, con
   int st = PDG_OK;
   const int64_t vp[2] = {0, n};
   if (!(h.hsc = static_cast<DevScalars*>(pinned_alloc(sizeof(DevScalars))))) return fail(PDG_E_OOM);
-  if ((st = alloc_n(h, &h.dsc, 1)) || (st = alloc_n(h, &h.row_ptr, n + 1)) || (st = alloc_n(h, &h.col, h.nnz)) ||
-      (st = alloc_n(h, &h.w, h.nnz)) || (st = alloc_n(h, &h.parent, n)) || (st = alloc_n(h, &h.d_vtx_ptr, 2)) ||
+  if ((st = alloc_n(h, &h.dsc, 1)) || (st = take_csr(h, row_ptr, col, w, mem_kind)) ||
+      (st = alloc_n(h, &h.parent, n)) || (st = alloc_n(h, &h.d_vtx_ptr, 2)) ||
       (st = alloc_n(h, &h.blk_a, 10240)) || (st = alloc_n(h, &h.blk_b, 2048)))
     return fail(st);
-  if (cudaMemcpyAsync(h.row_ptr, row_ptr, sizeof(int64_t) * (n + 1), kind, h.stream) != cudaSuccess ||
-      (h.nnz && cudaMemcpyAsync(h.col, col, sizeof(int32_t) * h.nnz, kind, h.stream) != cudaSuccess) ||
-      (h.nnz && cudaMemcpyAsync(h.w, w, sizeof(double) * h.nnz, kind, h.stream) != cudaSuccess) ||
-      cudaMemcpyAsync(h.d_vtx_ptr, vp, sizeof(vp), cudaMemcpyHostToDevice, h.stream) != cudaSuccess)
+  if (cudaMemcpyAsync(h.d_vtx_ptr, vp, sizeof(vp), cudaMemcpyHostToDevice, h.stream) != cudaSuccess)
     return fail(PDG_E_CUDA);
   if ((st = validate_csr(h))) return fail(st);
   if ((st = alloc_n(h, &h.el_u, std::max<int64_t>(h.m, 1))) || (st = alloc_n(h, &h.el_v, std::max<int64_t>(h.m, 1))) ||
@@ -679,15 +746,11 @@ static int pcg_entry(int64_t n, const int64_t* row_ptr, const int32_t* col, cons
   if (!(h.hsc = static_cast<DevScalars*>(pinned_alloc(sizeof(DevScalars)))) ||
       !(h.pcg_host = static_cast<double*>(pinned_alloc(sizeof(double) * kPcgParts))))
     return fail(PDG_E_OOM);
-  if ((st = alloc_n(h, &h.dsc, 1)) || (st = alloc_n(h, &h.row_ptr, n + 1)) || (st = alloc_n(h, &h.col, h.nnz)) ||
-      (st = alloc_n(h, &h.w, h.nnz)) || (st = alloc_n(h, &h.parent, n)) || (st = alloc_n(h, &h.d_vtx_ptr, 2)) ||
+  if ((st = alloc_n(h, &h.dsc, 1)) || (st = take_csr(h, row_ptr, col, w, mem_kind)) || (st = alloc_n(h, &h.parent, n)) || (st = alloc_n(h, &h.d_vtx_ptr, 2)) ||
       (st = alloc_n(h, &h.blk_a, 10240)) || (st = alloc_n(h, &h.blk_b, 2048)) ||
       (st = alloc_n(h, &d_ids, std::max<int64_t>(n_edges, 1))) || (st = alloc_n(h, &d_b, n)))
     return fail(st);
-  if (cudaMemcpyAsync(h.row_ptr, row_ptr, sizeof(int64_t) * (n + 1), kind, h.stream) != cudaSuccess ||
-      (h.nnz && cudaMemcpyAsync(h.col, col, sizeof(int32_t) * h.nnz, kind, h.stream) != cudaSuccess) ||
-      (h.nnz && cudaMemcpyAsync(h.w, w, sizeof(double) * h.nnz, kind, h.stream) != cudaSuccess) ||
-      cudaMemcpyAsync(h.parent, parent, sizeof(int32_t) * n, kind, h.stream) != cudaSuccess ||
+  if (cudaMemcpyAsync(h.parent, parent, sizeof(int32_t) * n, kind, h.stream) != cudaSuccess ||
       (n_edges && cudaMemcpyAsync(d_ids, edge_ids, sizeof(int32_t) * n_edges, kind, h.stream) != cudaSuccess) ||
       cudaMemcpyAsync(d_b, b, sizeof(double) * n, kind, h.stream) != cudaSuccess ||
       cudaMemcpyAsync(h.d_vtx_ptr, vp, sizeof(vp), cudaMemcpyHostToDevice, h.stream) != cudaSuccess)

@@ -55,6 +55,7 @@ enum : int {
   ERR_TABLE = 256,
   ERR_BOUNDS = 512,  // a saved index was out of range (checked and skipped; bounds_site says where)
   ERR_DENSE = 1024,  // the join's cells are too full: the attempt is repeated with the tiers
+  ERR_NOT_CSR_ROWS = 2048,  // row_ptr is not monotone (with ERR_NOT_CSR)
 };
 
 // candidate state in the cooperative tier
@@ -104,6 +105,13 @@ struct DevScalars {
   unsigned long long join_conf;   // join: (marker, candidate) pairs found
   int64_t finish_left;  // cooperative tier: candidates the rounds left to the serial finisher
 };
+
+// binary exponent of r = fl(1/w) for a normal w in [2^-900, 2^900]: -e for w = 2^e, else -e - 1 (1/w of the next double
+// above 2^e already lies two ulps below 2^-e)
+__host__ __device__ inline int resist_exponent(unsigned long long w_bits) {
+  const int e = (int)((w_bits >> 52) & 0x7ff) - 1023;
+  return (w_bits & 0xfffffffffffffull) ? -e - 1 : -e;
+}
 
 // the fixed-point range of exact root distances: 2^(e_max - e_min + 53) per edge, `depth` edges
 inline bool exact_range(const DevScalars& d, int64_t depth) {
@@ -203,6 +211,11 @@ struct Handle {
   double* rtree = nullptr;  // r(v) = fl(1/w(v, parent v))
   int64_t* blk_a = nullptr; // per-block counters (classification, scans)
   int64_t* blk_b = nullptr;
+  bool csr_borrowed = false;  // init: row_ptr, col and w are the caller's device arrays
+  // init from host memory: the weights are still on their way (sstream, ev_join) while the structure is worked on
+  bool w_pending = false, w_late = false;
+  uint32_t* w_mirror = nullptr;  // [nnz] place of the mirror image of the entries above the diagonal
+  uint2* w_place = nullptr;      // [m] per edge: its entry and that one's mirror image
   int32_t* up_count = nullptr;  // validation: entries above the diagonal, per chunk of kValChunk entries
   int64_t* up_off = nullptr;    // and before it
 
@@ -559,6 +572,8 @@ int scan_excl_u8(Handle& h, const uint8_t* in, int64_t* out, const int64_t* n_de
 
 // steps
 int validate_graph(Handle& h);  // input checks; the tours check acyclicity and range
+int finish_weights(Handle& h);  // weights that came late: waits, checks, fills the edge list
+int late_weight_status(Handle& h);  // after finish_weights: PDG_OK or what the weights are refused for
 int build_edge_list(Handle& h);                 // init: canonical edge list from the CSR, after validation
 int build_tree_layout(Handle& h);               // init: preorder labels, Euler tour, relabelled edges and parents
 int tree_scan_workspace(Handle& h);             // init: look-back space of the tree scan

@@ -178,6 +178,25 @@ __global__ void k_lay_edges(int32_t* __restrict__ eu, int32_t* __restrict__ ev, 
   }
 }
 
+// exponent range of the tree edges' resistances, where the weights came after the validation (weights that are refused
+// do not matter)
+__global__ void k_lay_range(const double* __restrict__ wup, int64_t n, DevScalars* dsc) {
+  int lo = INT_MAX, hi = INT_MIN;
+  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
+    const double w = wup[x];
+    if (w == 0.0) continue;  // a root
+    const int e = resist_exponent((unsigned long long)__double_as_longlong(w));
+    lo = min(lo, e);
+    hi = max(hi, e);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if ((threadIdx.x & 31) == 0 && lo != INT_MAX) {
+    atomicMin(&dsc->e_min, lo);
+    atomicMax(&dsc->e_max, hi);
+  }
+}
+
 }  // namespace
 
 int build_tree_layout(Handle& h) {
@@ -271,7 +290,9 @@ int build_tree_layout(Handle& h) {
     if (!exact_range(*h.hsc, h.max_depth)) return fail(PDG_E_RANGE);
   }
   LAY_CK(cudaMemsetAsync(h.wup, 0, sizeof(double) * n, s));
+  if ((st = finish_weights(h))) return fail(st);
   if (m > 0) k_lay_edges<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, h.el_w, pre_of, parent_pre, m, h.wup);
+  if (h.w_late) k_lay_range<<<gn, kBlock, 0, s>>>(h.wup, n, h.dsc);
   k_lay_up<<<gn, kBlock, 0, s>>>(parent_pre, n, static_cast<int4*>(h.up));
   LAY_CK(cudaMemcpyAsync(h.parent, parent_pre, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
   LAY_CK(cudaGetLastError());

@@ -24,7 +24,7 @@ __device__ __forceinline__ int32_t graph_of_vertex(const int64_t* __restrict__ v
 
 __global__ void k_val_rowptr(const int64_t* __restrict__ row_ptr, int64_t n, DevScalars* dsc) {
   for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += (int64_t)gridDim.x * blockDim.x)
-    if (row_ptr[u] > row_ptr[u + 1]) atomicOr(&dsc->err, ERR_NOT_CSR);
+    if (row_ptr[u] > row_ptr[u + 1]) atomicOr(&dsc->err, ERR_NOT_CSR | ERR_NOT_CSR_ROWS);
 }
 
 // Every warp takes kValRun * 32 consecutive entries: one search for the row of
@@ -73,11 +73,16 @@ __device__ __forceinline__ int64_t warp_entry_row(const int64_t* __restrict__ ro
   return u;
 }
 
+// WEIGHTS: all checks at once; else (the weights have not come yet) those of the structure, and the places of the mirror
+// images are kept, unless row_ptr was found bad.
+template <bool WEIGHTS>
 __global__ void __launch_bounds__(kBlock, 8) k_val_entries(const int64_t* __restrict__ row_ptr,
                                                         const int32_t* __restrict__ col,
                                                         const double* __restrict__ w, int64_t n, int64_t nnz,
                                                         const int64_t* __restrict__ vtx_ptr, int32_t G,
-                                                        int32_t* __restrict__ up_count, DevScalars* dsc) {
+                                                        int32_t* __restrict__ up_count,
+                                                        uint32_t* __restrict__ mirror, DevScalars* dsc) {
+  if (!WEIGHTS && (*(volatile int32_t*)&dsc->err & ERR_NOT_CSR_ROWS)) return;
   __shared__ int s_diff;
   if (threadIdx.x == 0) s_diff = 0;
   __syncthreads();
@@ -98,8 +103,11 @@ __global__ void __launch_bounds__(kBlock, 8) k_val_entries(const int64_t* __rest
       int32_t next = __shfl_down_sync(0xffffffffu, v, 1);
       if (in) {
         if (lane == 31 && p + 1 < nnz) next = col[p + 1];
-        const double x = w[p];
-        if (!(x >= lo && x <= hi)) err |= ERR_BAD_WEIGHT;
+        double x = 0.0;
+        if (WEIGHTS) {
+          x = w[p];
+          if (!(x >= lo && x <= hi)) err |= ERR_BAD_WEIGHT;
+        }
         if (v < 0 || v >= n || v == u) {
           err |= ERR_NOT_CSR;
         } else {
@@ -110,8 +118,11 @@ __global__ void __launch_bounds__(kBlock, 8) k_val_entries(const int64_t* __rest
             up++;
             const int64_t b = row_ptr[v], e = row_ptr[v + 1];
             const int64_t q = lower_bound_i32(col, b, e, (int32_t)u);
-            if (q >= e || col[q] != (int32_t)u || __double_as_longlong(w[q]) != __double_as_longlong(x))
+            if (q >= e || col[q] != (int32_t)u ||
+                (WEIGHTS && __double_as_longlong(w[q]) != __double_as_longlong(x)))
               err |= ERR_NOT_SYMMETRIC;
+            else if (!WEIGHTS)
+              mirror[p] = (uint32_t)q;
           }
         }
       }
@@ -131,11 +142,14 @@ __global__ void __launch_bounds__(kBlock, 8) k_val_entries(const int64_t* __rest
 // appends the ones of its chunk (columns in range, as many as counted: validated).  Reads the CSR once and writes the
 // list, 250 MB for mesh 128^3: 68 us (with a thread's loads eight entries apart and a second pass over the columns to
 // count, 133).
+// Without WEIGHTS the places of an edge's two entries are kept for k_edge_weights.
+template <bool WEIGHTS>
 __global__ void __launch_bounds__(kBlock) k_edge_list(const int64_t* __restrict__ row_ptr,
                                                       const int32_t* __restrict__ col, const double* __restrict__ w,
                                                       int64_t n, int64_t nnz, const int64_t* __restrict__ up_off,
-                                                      int32_t* __restrict__ eu, int32_t* __restrict__ ev,
-                                                      double* __restrict__ ew) {
+                                                      const uint32_t* __restrict__ mirror, int32_t* __restrict__ eu,
+                                                      int32_t* __restrict__ ev, double* __restrict__ ew,
+                                                      uint2* __restrict__ place) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -144,7 +158,7 @@ __global__ void __launch_bounds__(kBlock) k_edge_list(const int64_t* __restrict_
     for (int64_t b0 = p0; b0 < min(nnz, p0 + kValChunk); b0 += 32) {
       const int64_t p = b0 + lane;
       const int32_t v = p < nnz ? col[p] : 0;
-      const double x = p < nnz ? w[p] : 0.0;
+      const double x = WEIGHTS && p < nnz ? w[p] : 0.0;
       int64_t u_end;
       const int64_t u = warp_entry_row(row_ptr, n, nnz, row, p, &u_end);
       const bool up = p < nnz && u < v;
@@ -153,7 +167,8 @@ __global__ void __launch_bounds__(kBlock) k_edge_list(const int64_t* __restrict_
         const int64_t o = at + __popc(b & ((1u << lane) - 1));
         eu[o] = (int32_t)u;
         ev[o] = v;
-        ew[o] = x;
+        if (WEIGHTS) ew[o] = x;
+        else place[o] = make_uint2((uint32_t)p, mirror[p]);
       }
       at += __popc(b);
       row = __shfl_sync(0xffffffffu, u, 31);
@@ -161,6 +176,24 @@ __global__ void __launch_bounds__(kBlock) k_edge_list(const int64_t* __restrict_
   }
 }
 
+// The edges' weights, once they have come, and their checks: an entry below the diagonal has to be its image's equal,
+// bit by bit, so every weight is looked at.
+__global__ void __launch_bounds__(kBlock) k_edge_weights(const double* __restrict__ w, const uint2* __restrict__ place,
+                                                         int64_t m, double* __restrict__ ew, DevScalars* dsc) {
+  const double lo = ldexp(1.0, -900), hi = ldexp(1.0, 900);
+  int err = 0;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
+    const uint2 at = place[e];
+    const double x = w[at.x], y = w[at.y];
+    if (!(x >= lo && x <= hi) || !(y >= lo && y <= hi)) err |= ERR_BAD_WEIGHT;
+    if (__double_as_longlong(x) != __double_as_longlong(y)) err |= ERR_NOT_SYMMETRIC;
+    ew[e] = x;
+  }
+  if (err) atomicOr(&dsc->err, err);
+}
+
+// WEIGHTS: also the exponent range of the tree edges' resistances
+template <bool WEIGHTS>
 __global__ void k_val_parent(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                              const double* __restrict__ w, const int32_t* __restrict__ parent, int64_t n,
                              const int64_t* __restrict__ vtx_ptr, int32_t G, DevScalars* dsc,
@@ -183,8 +216,8 @@ __global__ void k_val_parent(const int64_t* __restrict__ row_ptr, const int32_t*
       err |= ERR_NOT_A_TREE;
       continue;
     }
-    const double r = 1.0 / w[q];
-    const int ex = (int)((__double_as_longlong(r) >> 52) & 0x7ff) - 1023;
+    if (!WEIGHTS) continue;
+    const int ex = resist_exponent((unsigned long long)__double_as_longlong(w[q]));
     lmin = min(lmin, ex);
     lmax = max(lmax, ex);
   }
@@ -222,13 +255,41 @@ int build_edge_list(Handle& h) {
   int st = ensure_scan_status(h, chunks);
   if (st || (st = scan_excl_i32(h, h.up_count, h.up_off, chunks, nullptr, chunks))) return st;
   ++h.launches;
-  k_edge_list<<<entry_grid(h), kBlock, 0, h.stream>>>(h.row_ptr, h.col, h.w, h.n, h.nnz, h.up_off, h.el_u, h.el_v,
-                                                      h.el_w);
+  if (h.w_pending)
+    k_edge_list<false><<<entry_grid(h), kBlock, 0, h.stream>>>(h.row_ptr, h.col, nullptr, h.n, h.nnz, h.up_off,
+                                                               h.w_mirror, h.el_u, h.el_v, nullptr, h.w_place);
+  else
+    k_edge_list<true><<<entry_grid(h), kBlock, 0, h.stream>>>(h.row_ptr, h.col, h.w, h.n, h.nnz, h.up_off, nullptr,
+                                                              h.el_u, h.el_v, h.el_w, nullptr);
   PDG_CUDA(cudaGetLastError());
   device_release(h, h.up_count);
   device_release(h, h.up_off);
   h.up_count = nullptr;
   h.up_off = nullptr;
+  return PDG_OK;
+}
+
+int finish_weights(Handle& h) {
+  if (!h.w_pending) return PDG_OK;
+  h.w_pending = false;
+  h.w_late = true;
+  PDG_CUDA(cudaStreamWaitEvent(h.stream, h.ev_join, 0));
+  ++h.launches;
+  k_edge_weights<<<grid_for(h, h.m), kBlock, 0, h.stream>>>(h.w, h.w_place, h.m, h.el_w, h.dsc);
+  PDG_CUDA(cudaGetLastError());
+  device_release(h, h.w_mirror);
+  device_release(h, h.w_place);
+  device_release(h, h.w);
+  h.w_mirror = nullptr;
+  h.w_place = nullptr;
+  h.w = nullptr;
+  return PDG_OK;
+}
+
+// (h.hsc holds the scalars as they were after finish_weights)
+int late_weight_status(Handle& h) {
+  if (h.hsc->err & ERR_BAD_WEIGHT) return PDG_E_BAD_WEIGHT;
+  if (h.hsc->err & ERR_NOT_SYMMETRIC) return PDG_E_NOT_SYMMETRIC;
   return PDG_OK;
 }
 
@@ -246,8 +307,8 @@ int validate_csr(Handle& h) {
   if (h.hsc->err) return PDG_E_NOT_CSR;  // the entry checks below search rows: only on a monotone row_ptr
   if (h.nnz > 0) {
     if (const int st = alloc_chunks(h)) return st;
-    k_val_entries<<<entry_grid(h), kBlock, 0, h.stream>>>(h.row_ptr, h.col, h.w, n, h.nnz, h.d_vtx_ptr, h.G, h.up_count,
-                                                          h.dsc);
+    k_val_entries<true><<<entry_grid(h), kBlock, 0, h.stream>>>(h.row_ptr, h.col, h.w, n, h.nnz, h.d_vtx_ptr, h.G,
+                                                                h.up_count, nullptr, h.dsc);
   }
   if (!fetch()) return check_cuda(cudaGetLastError());
   int err = h.hsc->err;
@@ -259,6 +320,39 @@ int validate_csr(Handle& h) {
   return PDG_OK;
 }
 
+constexpr int PDG_RETRY_WITH_WEIGHTS = 1000;
+
+// The checks that need no weights; PDG_RETRY_WITH_WEIGHTS when one of them fails (but row_ptr's).
+static int validate_structure(Handle& h, int grid) {
+  k_val_reset<<<1, 1, 0, h.stream>>>(h.dsc);
+  k_val_rowptr<<<grid, kBlock, 0, h.stream>>>(h.row_ptr, h.n, h.dsc);
+  k_val_entries<false><<<entry_grid(h), kBlock, 0, h.stream>>>(h.row_ptr, h.col, nullptr, h.n, h.nnz, h.d_vtx_ptr, h.G,
+                                                               h.up_count, h.w_mirror, h.dsc);
+  if (cudaMemcpyAsync(h.hsc, h.dsc, sizeof(DevScalars), cudaMemcpyDeviceToHost, h.stream) != cudaSuccess ||
+      cudaStreamSynchronize(h.stream) != cudaSuccess)
+    return check_cuda(cudaGetLastError());
+  if (h.hsc->err & ERR_NOT_CSR) return PDG_E_NOT_CSR;
+  if (h.hsc->err || h.hsc->active != 0) return PDG_RETRY_WITH_WEIGHTS;
+  int64_t* roots = nullptr;
+  if (cudaMallocAsync((void**)&roots, sizeof(int64_t) * h.G, h.stream) != cudaSuccess) {
+    cudaGetLastError();
+    return PDG_E_OOM;
+  }
+  cudaMemsetAsync(roots, 0, sizeof(int64_t) * h.G, h.stream);
+  k_val_parent<false><<<grid, kBlock, 0, h.stream>>>(h.row_ptr, h.col, nullptr, h.parent, h.n, h.d_vtx_ptr, h.G, h.dsc,
+                                                     roots);
+  std::vector<int64_t> roots_h(h.G);
+  const bool ok =
+      cudaMemcpyAsync(roots_h.data(), roots, sizeof(int64_t) * h.G, cudaMemcpyDeviceToHost, h.stream) == cudaSuccess &&
+      cudaMemcpyAsync(h.hsc, h.dsc, sizeof(DevScalars), cudaMemcpyDeviceToHost, h.stream) == cudaSuccess &&
+      cudaStreamSynchronize(h.stream) == cudaSuccess;
+  cudaFreeAsync(roots, h.stream);
+  if (!ok) return check_cuda(cudaGetLastError());
+  bool tree = h.hsc->err == 0;
+  for (int64_t r : roots_h) tree = tree && r == 1;
+  return tree ? PDG_OK : PDG_RETRY_WITH_WEIGHTS;
+}
+
 int validate_graph(Handle& h) {
   const int64_t n = h.n;
   const int grid = grid_for(h, std::max<int64_t>(n, h.nnz));
@@ -267,14 +361,21 @@ int validate_graph(Handle& h) {
     return cudaMemcpyAsync(h.hsc, h.dsc, sizeof(DevScalars), cudaMemcpyDeviceToHost, h.stream) == cudaSuccess &&
            cudaStreamSynchronize(h.stream) == cudaSuccess;
   };
+  if (h.nnz > 0)
+    if (const int st = alloc_chunks(h)) return st;
+  if (h.w_pending) {  // the structure alone; whatever is wrong with it, the weights may be refused for something else
+    const int st = validate_structure(h, grid);
+    if (st != PDG_RETRY_WITH_WEIGHTS) return st;
+    h.w_pending = false;
+    if (cudaStreamWaitEvent(h.stream, h.ev_join, 0) != cudaSuccess) return check_cuda(cudaGetLastError());
+  }
   k_val_reset<<<1, 1, 0, h.stream>>>(h.dsc);
   k_val_rowptr<<<grid, kBlock, 0, h.stream>>>(h.row_ptr, n, h.dsc);
   if (!fetch()) return check_cuda(cudaGetLastError());
   if (h.hsc->err) return PDG_E_NOT_CSR;
   if (h.nnz > 0) {
-    if (const int st = alloc_chunks(h)) return st;
-    k_val_entries<<<entry_grid(h), kBlock, 0, h.stream>>>(h.row_ptr, h.col, h.w, n, h.nnz, h.d_vtx_ptr, h.G, h.up_count,
-                                                          h.dsc);
+    k_val_entries<true><<<entry_grid(h), kBlock, 0, h.stream>>>(h.row_ptr, h.col, h.w, n, h.nnz, h.d_vtx_ptr, h.G,
+                                                                h.up_count, nullptr, h.dsc);
   }
   int64_t* roots = nullptr;
   int st = PDG_OK;
@@ -284,7 +385,7 @@ int validate_graph(Handle& h) {
     return PDG_E_OOM;
   }
   cudaMemsetAsync(roots, 0, sizeof(int64_t) * h.G, h.stream);
-  k_val_parent<<<grid, kBlock, 0, h.stream>>>(h.row_ptr, h.col, h.w, h.parent, n, h.d_vtx_ptr, h.G, h.dsc, roots);
+  k_val_parent<true><<<grid, kBlock, 0, h.stream>>>(h.row_ptr, h.col, h.w, h.parent, n, h.d_vtx_ptr, h.G, h.dsc, roots);
   std::vector<int64_t> roots_h(h.G);
   if (cudaMemcpyAsync(roots_h.data(), roots, sizeof(int64_t) * h.G, cudaMemcpyDeviceToHost, h.stream) != cudaSuccess ||
       !fetch()) {
