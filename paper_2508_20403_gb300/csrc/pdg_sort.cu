@@ -654,7 +654,170 @@ __global__ void __launch_bounds__(kCoThreads) k_sort_coop(CoopSortArgs a) {
   if (blockIdx.x == 0 && threadIdx.x == 0) a.dsc->radix_sel = cur;
 }
 
+// ---------------------------------------------------------------- few candidates
+//
+// A radix pass costs 5 to 7 us of barriers and scans however few keys it moves, eight of them 40 to 55.  Up to
+// kMgMax candidates (of capacity) of one graph are ordered by tiles instead: a block sorts a tile (bitonic: the strides
+// up to 32 in registers, the others in shared memory), then a key's rank is its place in its tile plus, for every other tile, the
+// keys there that come before it, found by eight lanes that each search up to four tiles at a time.  Ties are broken by
+// the place in the input, as the stable passes do.  The searches, N x tiles x 12 loads from L1 and L2, bound the second
+// kernel, the shuffles of the tile sort the first: tiles of 512 for the fewest candidates, which sort in 6 us, of 2048
+// (17 us) for the most, where more tiles would be searched.  332 candidates 38 -> 8 us, 12,000 55 -> 18, 13,600 (tiles
+// of 2048) 53 -> 35; 55,000 would take 59, against 56 in eight passes, so the line lies below that.
+constexpr int64_t kMgMax = 65536;
+
+struct MgItem {
+  uint64_t key;
+  int32_t at;  // place in the tile
+};
+
+__device__ __forceinline__ bool mg_less(const MgItem& a, const MgItem& b) {
+  return a.key < b.key || (a.key == b.key && a.at < b.at);
+}
+
+// element i of a pair (i, i ^ o) in the merge of width w keeps the smaller one where `up`
+__device__ __forceinline__ void mg_lane_step(MgItem& x, int o, bool keep_small) {
+  const MgItem y{__shfl_xor_sync(0xffffffffu, x.key, o), __shfl_xor_sync(0xffffffffu, x.at, o)};
+  if (mg_less(y, x) == keep_small) x = y;
+}
+
+// strides 32 (if w > 32) down to 1 of the merge of width w; the warp holds the elements e and e + 32 of its 64
+__device__ __forceinline__ void mg_warp_steps(MgItem& x0, MgItem& x1, int e, int w) {
+  const int lane = threadIdx.x & 31;
+  if (w >= 64) {
+    const bool up = (e & w) == 0;
+    if (mg_less(x1, x0) == up) {
+      const MgItem t = x0;
+      x0 = x1;
+      x1 = t;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    if (o >= w) continue;
+    const bool low = (lane & o) == 0;
+    mg_lane_step(x0, o, low == ((e & w) == 0));
+    mg_lane_step(x1, o, low == (((e + 32) & w) == 0));
+  }
+}
+
+template <int kMgTile>
+__global__ void __launch_bounds__(kMgTile / 2) k_tile_sort(const uint64_t* __restrict__ keys,
+                                                          const int32_t* __restrict__ vals, uint64_t* __restrict__ out_k,
+                                                          int32_t* __restrict__ out_v, int32_t* __restrict__ rank_cand,
+                                                          const DevScalars* dsc) {
+  dep_sync();
+  if (attempt_aborted(dsc)) return;
+  __shared__ uint64_t s_key[kMgTile];
+  __shared__ int32_t s_at[kMgTile];
+  const int64_t N = dsc->n_cand, t0 = (int64_t)blockIdx.x * kMgTile;
+  if (t0 >= N) return;
+  const int len = (int)min((int64_t)kMgTile, N - t0);
+  const int e = (threadIdx.x >> 5) * 64 + (threadIdx.x & 31);
+  MgItem x0{e < len ? keys[t0 + e] : ~0ull, e}, x1{e + 32 < len ? keys[t0 + e + 32] : ~0ull, e + 32};
+  for (int w = 2; w <= 64; w <<= 1) mg_warp_steps(x0, x1, e, w);
+  for (int w = 128; w <= kMgTile; w <<= 1) {
+    s_key[e] = x0.key;
+    s_at[e] = x0.at;
+    s_key[e + 32] = x1.key;
+    s_at[e + 32] = x1.at;
+    __syncthreads();
+    for (int o = w >> 1; o >= 64; o >>= 1) {
+      const int a = 2 * o * ((int)threadIdx.x / o) + (int)threadIdx.x % o, b = a + o;
+      const MgItem x{s_key[a], s_at[a]}, y{s_key[b], s_at[b]};
+      if (mg_less(y, x) == ((a & w) == 0)) {
+        s_key[a] = y.key;
+        s_at[a] = y.at;
+        s_key[b] = x.key;
+        s_at[b] = x.at;
+      }
+      __syncthreads();
+    }
+    x0 = {s_key[e], s_at[e]};
+    x1 = {s_key[e + 32], s_at[e + 32]};
+    mg_warp_steps(x0, x1, e, w);  // (the warp's own 64 elements: what it writes next no other warp reads before)
+  }
+  const bool alone = N <= kMgTile;
+#pragma unroll
+  for (int h = 0; h < 2; h++) {
+    const MgItem& x = h ? x1 : x0;
+    const int i = e + 32 * h;
+    if (i >= len) continue;  // (the padding's places are the last)
+    const int32_t v = vals[t0 + x.at];
+    if (alone) {
+      rank_cand[i] = v;
+    } else {
+      out_k[t0 + i] = x.key;
+      out_v[t0 + i] = v;
+    }
+  }
+}
+
+constexpr int kMgWays = 4;
+
+template <int kMgTile>
+__global__ void __launch_bounds__(kBlock) k_tile_rank(const uint64_t* keys, const int32_t* __restrict__ vals,
+                                                      int32_t* __restrict__ rank_cand, const DevScalars* dsc) {
+  dep_sync();
+  if (attempt_aborted(dsc)) return;
+  const int64_t N = dsc->n_cand;
+  if (N <= kMgTile) return;  // ranked already
+  const int tiles = (int)((N + kMgTile - 1) / kMgTile);
+  const int sub = threadIdx.x & 7;
+  const int64_t groups = (int64_t)gridDim.x * (kBlock / 8);
+  const int64_t rounds = (N + groups - 1) / groups;
+  int64_t s = (int64_t)blockIdx.x * (kBlock / 8) + (threadIdx.x >> 3);
+  for (int64_t r = 0; r < rounds; r++, s += groups) {  // warp-uniform
+    const bool in = s < N;
+    const uint64_t key = in ? keys[s] : 0;
+    const int own = (int)(s / kMgTile);
+    int before = 0;
+    for (int u0 = sub; u0 < tiles; u0 += 8 * kMgWays) {
+      int pos[kMgWays], len[kMgWays];
+#pragma unroll
+      for (int q = 0; q < kMgWays; q++) {
+        const int u = u0 + 8 * q;
+        pos[q] = 0;
+        len[q] = !in || u >= tiles || u == own ? 0 : (int)min((int64_t)kMgTile, N - (int64_t)u * kMgTile);
+      }
+#pragma unroll
+      for (int h = kMgTile / 2; h >= 0; h = h == 1 ? 0 : h == 0 ? -1 : h >> 1) {
+        // h = 0: the last step, which the place kMgTile needs
+#pragma unroll
+        for (int q = 0; q < kMgWays; q++) {
+          const int u = u0 + 8 * q, probe = h ? pos[q] + h - 1 : pos[q];
+          if (probe >= len[q]) continue;
+          const uint64_t k = keys[(int64_t)u * kMgTile + probe];
+          if (k < key || (u < own && k == key)) pos[q] += h ? h : 1;
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kMgWays; q++) before += pos[q];
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    if (in && sub == 0) rank_cand[before + (int)(s % kMgTile)] = vals[s];
+  }
+}
+
 }  // namespace
+
+template <int TILE>
+static void launch_sort_tiles(Handle& h) {
+  launch_k(h, k_tile_sort<TILE>, (int)((h.Rcap + TILE - 1) / TILE), TILE / 2, 0, h.rk[0], h.rv[0], h.rk[1], h.rv[1],
+           h.rank_cand, h.dsc);
+  const int grid = (int)std::min<int64_t>((int64_t)h.num_sms * 8, (8 * h.Rcap + kBlock - 1) / kBlock);
+  launch_k(h, k_tile_rank<TILE>, grid, kBlock, 0, h.rk[1], h.rv[1], h.rank_cand, h.dsc);
+}
+
+static int step_sort_tiles(Handle& h) {
+  h.launches += 2;
+  if (h.Rcap <= 16 * 512) launch_sort_tiles<512>(h);
+  else if (h.Rcap <= 32 * 1024) launch_sort_tiles<1024>(h);
+  else launch_sort_tiles<2048>(h);
+  PDG_CUDA(cudaGetLastError());
+  return PDG_OK;
+}
 
 // blocks of the one-launch sort that fit on the device at once (0: not available)
 static int coop_sort_grid() {
@@ -726,6 +889,8 @@ static int step_sort_coop(Handle& h, int grid_max) {
 }
 
 int step_sort(Handle& h) {
+  // (the first radix buffer holds the keys: the selection left them there)
+  if (h.opt.sort_one_launch && h.G == 1 && !h.tiered && h.Rcap <= kMgMax) return step_sort_tiles(h);
   // one cooperative launch when every tile of the candidate capacity has its own resident block
   const int cgrid = h.opt.sort_one_launch ? coop_sort_grid() : 0;
   if (cgrid > 0 && (h.Rcap + kCoTile - 1) / kCoTile <= cgrid &&
