@@ -7,6 +7,9 @@ sort whatever its tile size); only the time changes.  The tuner times recoveries
   block_tier_max  subtasks of T_w+1..T_b candidates get one block (0: none; larger ones go cooperative),
   sort_tile_keys  keys per scatter tile of the one-sweep radix sort,
 
+(the tiers decide only candidate sets whose cells are too full for the join, the one-sweep sort orders only sets
+beyond the one-launch sort: elsewhere the settings change nothing)
+
 by coordinate descent from the library defaults, checks that every setting returned the default's edges, and
 caches the winner in a JSON file keyed by the GPU (name and SM count) and a coarse graph class (size, mean degree,
 degree skew, graphs per batch).  `options_for` reads the cache; a graph class with no entry gets the defaults.
