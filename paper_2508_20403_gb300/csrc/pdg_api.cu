@@ -251,14 +251,35 @@ static void drop_csr(Handle& h) {
   if (!h.w_pending) h.w = nullptr;
 }
 
-int ensure_candidates(Handle& h, int64_t R, int c) {
-  const int64_t Rmax = std::max<int64_t>(h.E_off, 1);
-  R = std::min<int64_t>(std::max<int64_t>(R, 1), Rmax);
+// releases a buffer and forgets it
+template <typename T>
+static void drop(Handle& h, T*& p) {
+  device_release(h, p);
+  p = nullptr;
+}
+
+template <typename... T>
+static void drop_all(Handle& h, T*&... p) {
+  (drop(h, p), ...);
+}
+
+static void drop_tiers(Handle& h) {
+  drop_all(h, h.lsort_rank, h.rec_u, h.rec_v, h.rec_anc, h.rec_du, h.rec_dv, h.rec_rank, h.rec_lca, h.rec_b, h.state,
+           h.seg_begin, h.warp_seg, h.block_seg, h.big_pos, h.big_seg, h.big_chunk, h.pos_x, h.seg_regs, h.seg_pref,
+           h.pmask, h.reg_slot, h.pslot, h.und_list);
+  h.tier_cap = 0;
+}
+
+static void drop_candidates(Handle& h) {
+  drop_all(h, h.cand_idx, h.rk[0], h.rk[1], h.rv[0], h.rv[1], h.rank_cand, h.scan_tmp, h.radix_status, h.acc_flag,
+           h.cand_rec, h.join_rec, h.join_probe, h.join_conf, h.join_list, h.join_tab, h.join_ranks);
+  h.Rcap = h.join_list_cap = h.join_slots = 0;
+}
+
+static int grow_candidates(Handle& h, int64_t R, int c) {
   int st;
   if (R > h.Rcap) {
-    void* old[] = {h.cand_idx, h.rk[0], h.rk[1], h.rv[0], h.rv[1], h.rank_cand, h.scan_tmp,
-                   h.radix_status, h.acc_flag, h.cand_rec, h.join_rec, h.join_probe, h.join_conf, h.join_list};
-    for (void* p : old) device_release(h, p);
+    drop_candidates(h);
     const int64_t tiles = (R + kTile - 1) / kTile;
     const int64_t join_list = std::min<int64_t>(kJoinListPer * R, INT32_MAX);  // runs start at 32-bit offsets
     if ((st = alloc_n(h, &h.cand_idx, R)) || (st = alloc_n(h, &h.rk[0], R)) || (st = alloc_n(h, &h.rk[1], R)) ||
@@ -268,29 +289,36 @@ int ensure_candidates(Handle& h, int64_t R, int c) {
         (st = alloc_n(h, &h.acc_flag, R)) || (st = device_alloc(h, &h.cand_rec, (size_t)32 * R)) ||
         (st = device_alloc(h, &h.join_rec, (size_t)32 * R)) ||
         (st = device_alloc(h, &h.join_probe, (size_t)32 * R)) || (st = alloc_n(h, &h.join_conf, 8 * R)) ||
-        (st = alloc_n(h, &h.join_list, join_list))) {
-      h.Rcap = 0;
+        (st = alloc_n(h, &h.join_list, join_list)))
       return st;
-    }
     h.Rcap = R;
-    h.join_slots = 0;
     h.join_list_cap = join_list;
-    if ((st = grow_join(h))) return st;
   }
+  if (h.join_slots == 0 && (st = grow_join(h))) return st;  // (zero also after a growth that failed)
   if ((st = ensure_scan_status(h, h.Rcap + 1))) return st;
   // the selection's list: a power of two of the scores, usually a few times the candidates
   // (R-MAT graphs: 8 to 40 times, which an eighth of the edges holds; it is 1.5 bytes an edge)
+  const int64_t Rmax = std::max<int64_t>(h.E_off, 1);
   const int64_t list = std::min(Rmax, std::max({4 * h.Rcap, Rmax / 8, (int64_t)1 << 19}));
   if (h.list_cap < list && (st = grow_list(h, list))) return st;
   return h.tiered ? ensure_tiers(h, c) : PDG_OK;
 }
 
+// Buffers for R candidates.  A failure gives back all of them, so that a later call (of a smaller budget, or when
+// there is more memory) starts anew and finds no capacity that stands for a buffer it does not have.
+int ensure_candidates(Handle& h, int64_t R, int c) {
+  R = std::min<int64_t>(std::max<int64_t>(R, 1), std::max<int64_t>(h.E_off, 1));
+  const int st = grow_candidates(h, R, c);
+  if (st) {
+    drop_candidates(h);
+    drop_tiers(h);
+  }
+  return st;
+}
+
 int grow_list(Handle& h, int64_t entries) {
   entries = std::min<int64_t>(entries, std::max<int64_t>(h.E_off, 1));
-  device_release(h, h.list_id);
-  device_release(h, h.list_key);
-  h.list_id = nullptr;
-  h.list_key = nullptr;
+  drop_all(h, h.list_id, h.list_key);
   h.list_cap = 0;
   int st;
   if ((st = alloc_n(h, &h.list_id, entries)) || (st = alloc_n(h, &h.list_key, entries))) return st;
@@ -300,11 +328,8 @@ int grow_list(Handle& h, int64_t entries) {
 
 // the join's cell table: join_factor slots per candidate of the capacity
 int grow_join(Handle& h) {
-  device_release(h, h.join_tab);
-  h.join_tab = nullptr;
+  drop_all(h, h.join_tab, h.join_ranks);
   h.join_slots = 0;
-  device_release(h, h.join_ranks);
-  h.join_ranks = nullptr;
   const int64_t slots = std::min<int64_t>(h.join_factor * h.Rcap + 1024, (1ll << 32) - 16) / 16 * 16;
   int st;
   if ((st = device_alloc(h, &h.join_tab, (size_t)slots * kJoinSlotBytes)) ||
@@ -319,10 +344,7 @@ static int ensure_tiers(Handle& h, int c) {
   const int64_t R = h.Rcap;
   int st;
   if (R > h.tier_cap) {
-    void* old[] = {h.lsort_rank, h.rec_u, h.rec_v, h.rec_anc, h.rec_du, h.rec_dv, h.rec_rank, h.rec_lca, h.rec_b, h.state,
-                   h.seg_begin, h.warp_seg, h.block_seg, h.big_pos, h.big_seg, h.big_chunk, h.pos_x, h.seg_regs,
-                   h.seg_pref, h.pmask, h.reg_slot, h.pslot, h.und_list};
-    for (void* p : old) device_release(h, p);
+    drop_tiers(h);
     if ((st = alloc_n(h, &h.lsort_rank, R)) || (st = alloc_n(h, &h.rec_u, R)) ||
         (st = alloc_n(h, &h.rec_v, R)) || (st = alloc_n(h, &h.rec_anc, 2 * PDG_MAX_C * R)) ||
         (st = alloc_n(h, &h.rec_du, R)) || (st = alloc_n(h, &h.rec_dv, R)) || (st = alloc_n(h, &h.rec_rank, R)) ||
@@ -331,10 +353,8 @@ static int ensure_tiers(Handle& h, int c) {
         (st = alloc_n(h, &h.warp_seg, R)) || (st = alloc_n(h, &h.block_seg, R)) || (st = alloc_n(h, &h.big_pos, R)) || (st = alloc_n(h, &h.big_seg, R)) || (st = alloc_n(h, &h.big_chunk, R)) ||
         (st = alloc_n(h, &h.pos_x, R)) || (st = alloc_n(h, &h.seg_regs, R)) || (st = alloc_n(h, &h.seg_pref, R + 1)) ||
         (st = alloc_n(h, &h.pmask, R)) || (st = alloc_n(h, &h.reg_slot, 16 * R)) || (st = alloc_n(h, &h.und_list, R)) ||
-        (st = alloc_n(h, &h.pslot, 32 * R))) {
-      h.tier_cap = 0;
+        (st = alloc_n(h, &h.pslot, 32 * R)))
       return st;
-    }
     h.tier_cap = R;
   }
   // pair table: twice the registrations plus 16 slots per cooperative subtask (at most R / 33 subtasks)
@@ -346,10 +366,7 @@ int grow_tables(Handle& h, int64_t slots, int64_t xblocks) {
   int st;
   slots = std::min<int64_t>(slots, (1ll << 32) - 1);  // slot indices are 32-bit on the device
   if (slots > h.table_cap) {
-    device_release(h, h.ptab);
-    device_release(h, h.flagbits);
-    h.ptab = nullptr;
-    h.flagbits = nullptr;
+    drop_all(h, h.ptab, h.flagbits);
     if ((st = alloc_n(h, &h.ptab, slots)) || (st = alloc_n(h, &h.flagbits, slots / 32 + 1))) {
       h.table_cap = 0;
       return st;
@@ -358,10 +375,7 @@ int grow_tables(Handle& h, int64_t slots, int64_t xblocks) {
   }
   xblocks = std::max<int64_t>(xblocks, std::max<int64_t>(64, h.table_cap / 16));
   if (xblocks > h.xcap) {
-    device_release(h, h.xtab);
-    device_release(h, h.xund1);
-    h.xtab = nullptr;
-    h.xund1 = nullptr;
+    drop_all(h, h.xtab, h.xund1);
     if ((st = alloc_n(h, &h.xtab, 16 * xblocks)) || (st = alloc_n(h, &h.xund1, 16 * xblocks))) {
       h.xcap = 0;
       return st;
@@ -1029,8 +1043,12 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
       continue;
     }
     if ((err & ERR_TABLE) && !h.tiered) {  // the cells outgrew the table
+      const int64_t factor = h.join_factor;
       h.join_factor *= 4;
-      if ((st = grow_join(h))) return st;
+      if ((st = grow_join(h))) {
+        h.join_factor = factor;
+        return st;
+      }
       first = false;
       continue;
     }

@@ -1,0 +1,164 @@
+// The library's host code (handle life cycle, buffers, recovery driver) on the CUDA runtime of fake_cudart.cc: allocations
+// fail where a check says so, and what the kernels would report is scripted.  Built and run by tests/test_host_driver.py;
+// needs nvcc, no GPU.
+#include "pdg_api.cu"
+
+#include "fake_cudart.h"
+
+namespace {
+
+#define CHECK(x)                                                                   \
+  do {                                                                             \
+    if (!(x)) fake::die("line %d: %s does not hold", __LINE__, #x);                \
+  } while (0)
+
+// what the attempts of the following recoveries report
+void script(const std::function<void(DevScalars&)>& report) {
+  fake::on_copy = [report](void* to, size_t bytes) {
+    if (bytes == sizeof(DevScalars)) report(*static_cast<DevScalars*>(to));
+  };
+}
+
+// what init's kernels would have found in a sound graph
+void sound_graph(const std::string& name, void** a) {
+  if (fake::named(name, "k_val_parent")) (*static_cast<int64_t**>(a[8]))[0] = 1;  // one root
+  if (fake::named(name, "k_gather_rowptr")) {
+    const int64_t* row_ptr = *static_cast<const int64_t**>(a[0]);
+    const int64_t* vtx_ptr = *static_cast<const int64_t**>(a[1]);
+    for (int32_t g = 0; g <= *static_cast<int32_t*>(a[2]); g++) (*static_cast<int64_t**>(a[3]))[g] = row_ptr[vtx_ptr[g]];
+  }
+}
+
+// a handle over n vertices of `degree` entries each, from host memory
+pdg_handle make(int64_t n, int64_t degree, bool use_graph, int* status = nullptr) {
+  fake::on_launch = sound_graph;
+  fake::on_copy = nullptr;
+  std::vector<int64_t> row_ptr(n + 1);
+  for (int64_t v = 0; v <= n; v++) row_ptr[v] = v * degree;
+  std::vector<int32_t> col(n * degree), parent(n);
+  std::vector<double> w(n * degree, 1.0);
+  pdg_options o;
+  pdg_default_options(&o);
+  o.use_graph = use_graph;
+  pdg_handle h = nullptr;
+  const int st = sparsify_init(&h, n, row_ptr.data(), col.data(), w.data(), parent.data(), PDG_MEM_HOST, &o, nullptr);
+  if (status) *status = st;
+  else CHECK(st == PDG_OK);
+  return h;
+}
+
+int recover(pdg_handle h, double alpha, int c = 2) {
+  std::vector<int32_t> ids((size_t)h->h.E_off);
+  int64_t count = 0;
+  return recover_offtree(h, alpha, c, ids.data(), (int64_t)ids.size(), &count, nullptr, PDG_MEM_HOST);
+}
+
+// every buffer that the launches of a recovery read or write
+void check_buffers(const Handle& h, bool tiers) {
+  const size_t R = (size_t)h.Rcap;
+  CHECK(R > 0);
+  fake::need("cand_idx", h.cand_idx, 4 * R);
+  for (int i = 0; i < 2; i++) {
+    fake::need("rk", h.rk[i], 8 * R);
+    fake::need("rv", h.rv[i], 4 * R);
+  }
+  fake::need("rank_cand", h.rank_cand, 4 * R);
+  fake::need("scan_tmp", h.scan_tmp, 8 * (R + 1));
+  fake::need("acc_flag", h.acc_flag, R);
+  fake::need("radix_status", h.radix_status, 4);
+  for (const void* p : {h.cand_rec, h.join_rec, h.join_probe}) fake::need("records", p, 32 * R);
+  fake::need("join_conf", h.join_conf, 32 * R);
+  fake::need("join_list", h.join_list, 4 * (size_t)h.join_list_cap);
+  CHECK(h.join_slots >= 16 && h.join_list_cap > 0);
+  fake::need("join_tab", h.join_tab, (size_t)h.join_slots * kJoinSlotBytes);
+  fake::need("join_ranks", h.join_ranks, (size_t)h.join_slots * kJoinInline * 4);
+  CHECK(h.list_cap > 0);
+  fake::need("list_id", h.list_id, 4 * (size_t)h.list_cap);
+  fake::need("list_key", h.list_key, 8 * (size_t)h.list_cap);
+  fake::need("scan_status", h.scan_status, 8 * (size_t)h.scan_tiles_cap);
+  if (!tiers) return;
+  CHECK(h.tier_cap == h.Rcap && h.table_cap > 0 && h.xcap > 0);
+  for (const void* p : {(void*)h.lsort_rank, (void*)h.rec_u, (void*)h.rec_v, (void*)h.rec_du, (void*)h.rec_dv,
+                        (void*)h.rec_rank, (void*)h.rec_lca, (void*)h.seg_begin, (void*)h.warp_seg, (void*)h.block_seg,
+                        (void*)h.big_pos, (void*)h.big_seg, (void*)h.big_chunk, (void*)h.seg_regs, (void*)h.und_list})
+    fake::need("tiers", p, 4 * R);
+  fake::need("rec_b", h.rec_b, R);
+  fake::need("state", h.state, R);
+  fake::need("pslot", h.pslot, 32 * R);
+  fake::need("reg_slot", h.reg_slot, 16 * R);
+  fake::need("ptab", h.ptab, (size_t)h.table_cap);
+  fake::need("xtab", h.xtab, 16 * (size_t)h.xcap);
+  fake::need("xund1", h.xund1, 16 * (size_t)h.xcap);
+}
+
+// Every allocation of a recovery fails in turn; the call says so, and the next one (the same budget, then a smaller
+// one) has all its buffers.  `report`: what the recovery's attempts report.
+void fail_each(const std::function<void(const Handle&, DevScalars&, int)>& report, bool tiers) {
+  for (double next : {0.5, 0.05})
+    for (int64_t j = 0;; j++) {
+      pdg_handle h = make(2000, 12, false);
+      int attempt = 0;
+      script([&](DevScalars& d) { report(h->h, d, attempt++); });
+      fake::on_launch = [h](const std::string& name, void**) {
+        if (fake::named(name, "k_join_insert") || fake::named(name, "k_build_records"))
+          check_buffers(h->h, fake::named(name, "k_build_records"));
+      };
+      fake::fail_from = fake::allocs + j;
+      fake::fail_count = 1;
+      const int st = recover(h, 0.5);
+      const bool failed = fake::allocs > fake::fail_from;
+      fake::fail_from = -1;
+      CHECK(st == (failed ? PDG_E_OOM : PDG_OK));
+      attempt = 0;
+      CHECK(recover(h, next) == PDG_OK);
+      check_buffers(h->h, tiers);
+      sparsifier_free(h);
+      CHECK(fake::live.empty());
+      if (!failed) break;
+    }
+}
+
+void oom_join() { fail_each([](const Handle&, DevScalars&, int) {}, false); }
+
+void oom_table() {
+  fail_each([](const Handle&, DevScalars& d, int attempt) { d.err = attempt == 0 ? ERR_TABLE : 0; }, false);
+}
+
+void oom_tiers() {
+  fail_each([](const Handle& h, DevScalars& d, int) { d.err = h.tiered ? 0 : ERR_DENSE; }, true);
+}
+
+// a table that could not grow is not asked for at its new size by a call that does without
+void oom_table_keeps_size() {
+  pdg_handle h = make(2000, 12, false);
+  CHECK(recover(h, 0.5) == PDG_OK);
+  const int64_t slots = h->h.join_slots;
+  int attempt = 0;
+  script([&](DevScalars& d) { d.err = attempt++ == 0 ? ERR_TABLE : 0; });
+  fake::fail_from = fake::allocs;
+  fake::fail_count = 1;
+  CHECK(recover(h, 0.5) == PDG_E_OOM);
+  fake::fail_from = -1;
+  CHECK(recover(h, 0.5) == PDG_OK);
+  CHECK(h->h.join_slots == slots);
+  sparsifier_free(h);
+}
+
+const std::map<std::string, void (*)()> kChecks = {
+    {"oom_join", oom_join},
+    {"oom_table", oom_table},
+    {"oom_tiers", oom_tiers},
+    {"oom_table_keeps_size", oom_table_keeps_size},
+};
+
+}  // namespace
+
+int main(int argc, char** argv) {
+  const auto it = argc > 1 ? kChecks.find(argv[1]) : kChecks.end();
+  if (it == kChecks.end()) {
+    for (const auto& c : kChecks) puts(c.first.c_str());
+    return argc > 1 ? 1 : 0;
+  }
+  it->second();
+  return 0;
+}
