@@ -178,6 +178,19 @@ __global__ void k_endpoints(const int32_t* __restrict__ eu, const int32_t* __res
 
 }  // namespace
 
+// releases one of a recovery's growing buffers and forgets it
+template <typename T>
+static void drop(Handle& h, T*& p) {
+  device_release(h, p);
+  p = nullptr;
+  h.buffers++;
+}
+
+template <typename... T>
+static void drop_all(Handle& h, T*&... p) {
+  (drop(h, p), ...);
+}
+
 // status words of the single-pass scan for inputs of up to n_max elements
 int ensure_scan_status(Handle& h, int64_t n_max) {
   const int64_t tiles = (std::max<int64_t>(n_max, 1) + kTile - 1) / kTile;
@@ -187,8 +200,7 @@ int ensure_scan_status(Handle& h, int64_t n_max) {
     PDG_CUDA(cudaMemsetAsync(h.scan_ctr, 0, 2 * sizeof(uint32_t), h.stream));
   }
   if (tiles <= h.scan_tiles_cap) return PDG_OK;
-  device_release(h, h.scan_status);
-  h.scan_status = nullptr;
+  drop(h, h.scan_status);
   h.scan_tiles_cap = 0;
   int st = alloc_n(h, &h.scan_status, tiles);
   if (st) return st;
@@ -249,18 +261,6 @@ static void drop_csr(Handle& h) {
   h.row_ptr = nullptr;
   h.col = nullptr;
   if (!h.w_pending) h.w = nullptr;
-}
-
-// releases a buffer and forgets it
-template <typename T>
-static void drop(Handle& h, T*& p) {
-  device_release(h, p);
-  p = nullptr;
-}
-
-template <typename... T>
-static void drop_all(Handle& h, T*&... p) {
-  (drop(h, p), ...);
 }
 
 static void drop_tiers(Handle& h) {
@@ -1004,8 +1004,8 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
     any_select_cur = any_select;
     if ((st = ensure_candidates(h, std::max<int64_t>(h.Rcap, need + need / 4 + 4096), c))) return st;
     // the launch sequence a CUDA graph bakes in
-    const GraphKey key{c, h.opt.score_mode, any_select ? 1 : 0, h.tiered ? coop_rounds(h, c) : 0, h.Rcap, h.table_cap, h.xcap,
-                       h.join_slots, h.list_cap, h.tiered, (void*)dev_ids, (void*)dev_scores, out_total};
+    const GraphKey key{c, h.opt.score_mode, any_select ? 1 : 0, h.tiered ? coop_rounds(h, c) : 0, h.buffers, h.tiered,
+                       (void*)dev_ids, (void*)dev_scores, out_total};
     bool replayed = false;
     if (first && h.opt.use_graph && h.gexec && key == h.gkey) {
       // replay on the private stream, ordered after the caller's stream

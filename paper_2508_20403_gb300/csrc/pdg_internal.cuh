@@ -163,14 +163,14 @@ struct GraphSel {
 // reads at replay time (budgets, prefix sizes, output offsets).
 struct GraphKey {
   int c = -1, score_mode = -1, any_select = -1, rounds = -1;
-  int64_t Rcap = -1, table_cap = -1, xcap = -1, join_slots = -1, list_cap = -1;
+  int64_t buffers = -1;  // Handle::buffers: the allocations that the launches point into, and their sizes
   bool tiered = false;
   void* out_ids = nullptr;
   void* out_scores = nullptr;
   int64_t out_total = -1;
   bool operator==(const GraphKey& o) const {
-    return c == o.c && score_mode == o.score_mode && any_select == o.any_select && rounds == o.rounds && Rcap == o.Rcap &&
-           table_cap == o.table_cap && xcap == o.xcap && join_slots == o.join_slots && list_cap == o.list_cap && tiered == o.tiered && out_ids == o.out_ids && out_scores == o.out_scores &&
+    return c == o.c && score_mode == o.score_mode && any_select == o.any_select && rounds == o.rounds &&
+           buffers == o.buffers && tiered == o.tiered && out_ids == o.out_ids && out_scores == o.out_scores &&
            out_total == o.out_total;
   }
 };
@@ -260,6 +260,7 @@ struct Handle {
   uint64_t* list_key = nullptr;
   void* list_tile = nullptr;  // int2 per tile of the edge list: its run in the list
   // candidate buffers (grow-only, capacity Rcap)
+  int64_t buffers = 0;  // goes up whenever one of a recovery's growing buffers is given back
   int64_t Rcap = 0;
   // the join: records and probes by rank, cell table, candidates per LCA
   void* cand_rec = nullptr;  // candidates in id order, 32 bytes: u, v, LCA, canonical id, score bits

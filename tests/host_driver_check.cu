@@ -3,6 +3,8 @@
 // needs nvcc, no GPU.
 #include "pdg_api.cu"
 
+#include <set>
+
 #include "fake_cudart.h"
 
 namespace {
@@ -144,7 +146,30 @@ void oom_table_keeps_size() {
   sparsifier_free(h);
 }
 
+// A captured recovery holds addresses: it is not replayed once its buffers were given back, whatever the sizes of the
+// new ones.
+void graph_of_old_buffers() {
+  pdg_handle h = make(2000, 12, true);
+  CHECK(recover(h, 0.1) == PDG_OK && recover(h, 0.1) == PDG_OK);
+  CHECK(fake::graphs == 1 && fake::graph_launches == 1);
+  const int64_t Rcap = h->h.Rcap;
+  fake::fail_from = fake::allocs + 5;  // a larger budget, and memory runs out while its buffers are made
+  fake::fail_count = 1;
+  CHECK(recover(h, 0.9) == PDG_E_OOM);
+  fake::fail_from = -1;
+  std::set<void*> taken;  // (the addresses given back are in use elsewhere now)
+  for (int i = 0; i < 64; i++) taken.insert(malloc(4096));
+  CHECK(recover(h, 0.1) == PDG_OK);
+  CHECK(h->h.Rcap == Rcap);
+  CHECK(fake::graphs == 2 && fake::graph_launches == 1);
+  CHECK(recover(h, 0.1) == PDG_OK);
+  CHECK(fake::graphs == 2 && fake::graph_launches == 2);
+  sparsifier_free(h);
+  for (void* p : taken) free(p);
+}
+
 const std::map<std::string, void (*)()> kChecks = {
+    {"graph_of_old_buffers", graph_of_old_buffers},
     {"oom_join", oom_join},
     {"oom_table", oom_table},
     {"oom_tiers", oom_tiers},

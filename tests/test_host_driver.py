@@ -40,3 +40,9 @@ def test_calls_after_a_failed_allocation(checker, name):
     """Each allocation of a recovery fails once (candidate buffers, the join's table and its growth, the tiers'
     buffers); the call reports it, the next call has every buffer its kernels use, nothing is freed twice."""
     _run(checker, name)
+
+
+def test_a_graph_ends_with_its_buffers(checker):
+    """A budget, captured and replayed; a larger one that runs out of memory; the first again: the buffers are new ones
+    of the old sizes, so the old graph must not run."""
+    _run(checker, "graph_of_old_buffers")
