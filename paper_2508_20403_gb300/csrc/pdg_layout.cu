@@ -61,19 +61,16 @@ __global__ void k_lay_cut(const int32_t* __restrict__ parent, const int64_t* __r
 // parent links away from the root.  Such an arc, or a position outside its
 // graph's tour, marks the tree bad and is not written; so do parent links that
 // hold a 2-cycle, which have fewer distinct edges than a tree.
-__global__ void k_lay_arcs(const int32_t* __restrict__ tadj, const int64_t* __restrict__ tptr,
-                           const int32_t* __restrict__ parent, const uint64_t* __restrict__ own,
-                           const uint64_t* __restrict__ walk, const int64_t* __restrict__ vtx_ptr, int32_t G, int64_t n,
-                           int64_t A, int32_t* __restrict__ tour, int32_t* __restrict__ dflag,
-                           int32_t* __restrict__ bad) {
+__global__ void __launch_bounds__(kBlock) k_lay_arcs(
+    const int32_t* __restrict__ tadj, const int64_t* __restrict__ tptr, const int32_t* __restrict__ parent,
+    const uint64_t* __restrict__ own, const uint64_t* __restrict__ walk, const int64_t* __restrict__ vtx_ptr, int32_t G,
+    int64_t n, int64_t A, int32_t* __restrict__ tour, int32_t* __restrict__ dflag, int32_t* __restrict__ bad) {
   if (blockIdx.x == 0 && threadIdx.x == 0 && tptr[n] != A) *bad = 1;
-  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = tptr[x], e = tptr[x + 1];
-    if (b == e) continue;
+  auto arcs = [&](int64_t x, int64_t b, int64_t e, int step) {
     const int32_t g = (G == 1) ? 0 : part_of(vtx_ptr, G, x);
     const int64_t len = 2 * (vtx_ptr[g + 1] - vtx_ptr[g] - 1);
     const int64_t base = 2 * (vtx_ptr[g] - g);
-    for (int64_t a = b; a < e; a++) {
+    for (int64_t a = b; a < e; a += step) {
       const int32_t y = tadj[a];
       const int32_t rd = arc_rank(own, walk, a);
       if (rd < 0 || rd >= len) {
@@ -85,7 +82,13 @@ __global__ void k_lay_arcs(const int32_t* __restrict__ tadj, const int64_t* __re
       tour[pos] = down ? y : ~(int32_t)x;
       dflag[pos] = down ? 1 : 0;
     }
-  }
+  };
+  for_rows(
+      tptr, n,
+      [&](int64_t x, int64_t b, int64_t e) {
+        if (b < e) arcs(x, b, e, 1);
+      },
+      [&](int64_t x, int64_t b, int64_t e) { arcs(x, b + threadIdx.x, e, kBlock); });
 }
 
 // preorder label of the vertex entered by each down arc: the graph's first
@@ -265,7 +268,7 @@ int build_tree_layout(Handle& h) {
   if ((st = scan_excl_i32(h, tdeg, tptr, n, nullptr, n))) return fail(st);
   if (A > 0) {
     k_st_fill<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, tflag, m, tptr, cur, tadj, rev, arc_uv);
-    k_tour_sort_rows<<<gn, kBlock, 0, s>>>(tptr, n, tadj);
+    k_tour_sort_rows<<<gn, kBlock, 0, s>>>(tptr, n, tadj, succ);  // (succ is written below)
     k_tour_fix_rev<<<gn, kBlock, 0, s>>>(tptr, tadj, n, rev);
     k_st_succ<<<ga, kBlock, 0, s>>>(tadj, rev, tptr, tdeg, n, succ);
     k_lay_cut<<<gn, kBlock, 0, s>>>(h.parent, tptr, tdeg, rev, n, succ, rank);

@@ -664,22 +664,6 @@ __global__ void k_pc_inc_fill(const int32_t* __restrict__ ea, const int32_t* __r
   }
 }
 
-// each incidence list in increasing edge order (a fixed summation order)
-__global__ void k_pc_inc_sort(const int64_t* __restrict__ iptr, int64_t n, int32_t* __restrict__ iedge) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = iptr[v], e = iptr[v + 1];
-    for (int64_t p = b + 1; p < e; p++) {
-      const int32_t x = iedge[p];
-      int64_t q = p - 1;
-      while (q >= b && iedge[q] > x) {
-        iedge[q + 1] = iedge[q];
-        q--;
-      }
-      iedge[q + 1] = x;
-    }
-  }
-}
-
 // --- vectors ---
 __global__ void k_pc_degw(const int64_t* __restrict__ row_ptr, const double* __restrict__ w, int64_t n,
                           double* __restrict__ dw) {
@@ -838,7 +822,7 @@ int pcg_quality(Handle& h, const int32_t* ids, int64_t k, const double* b, doubl
   }
   k_st_fill<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, tflag, m, tptr, cur, tadj, rev, arc_uv);
   // rows in neighbour order: the tour, and so every sum along it, is the same on every run
-  k_tour_sort_rows<<<gn, kBlock, 0, s>>>(tptr, n, tadj);
+  k_tour_sort_rows<<<gn, kBlock, 0, s>>>(tptr, n, tadj, succ);  // (succ is written below)
   k_tour_fix_rev<<<gn, kBlock, 0, s>>>(tptr, tadj, n, rev);
   k_tour_fix_arcs<<<gm, kBlock, 0, s>>>(h.el_u, h.el_v, tflag, m, tptr, tadj, arc_uv);
   const int ga = grid_for(h, std::max<int64_t>(A, 1));
@@ -918,7 +902,8 @@ int pcg_quality(Handle& h, const int32_t* ids, int64_t k, const double* b, doubl
     k_pc_inc_count<<<gk, kBlock, 0, s>>>(ea, eb, k, icnt);
     if ((st = scan_excl_i32(h, icnt, iptr, n, nullptr, n))) return fail(st);
     k_pc_inc_fill<<<gk, kBlock, 0, s>>>(ea, eb, k, iptr, cur, iedge);
-    k_pc_inc_sort<<<gn, kBlock, 0, s>>>(iptr, n, iedge);
+    // each list in increasing edge order (a fixed summation order); the sorted endpoints' keys are not needed any more
+    k_tour_sort_rows<<<gn, kBlock, 0, s>>>(iptr, n, iedge, reinterpret_cast<int32_t*>(ekey));
   }
   // the root's potential (the solves write every other vertex's)
   PC_CK(cudaMemsetAsync(t + root, 0, sizeof(double), s));
