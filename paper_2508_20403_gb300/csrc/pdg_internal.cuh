@@ -370,11 +370,13 @@ __device__ __forceinline__ int64_t row_of(const int64_t* __restrict__ row_ptr, i
 }
 
 // one aligned 32-byte sector in one load (two 16-byte loads of it are two requests, and the second misses L1
-// while the first is in flight)
+// while the first is in flight).  Volatile and clobbering memory: it stays behind dep_sync() and barriers, in order with
+// the kernel's stores, and is never merged with another one.
 __device__ __forceinline__ void load_sector(const void* p, uint4& x, uint4& y) {
-  asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w), "=r"(y.x), "=r"(y.y), "=r"(y.z), "=r"(y.w)
-      : "l"(p));
+  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w), "=r"(y.x), "=r"(y.y), "=r"(y.z), "=r"(y.w)
+               : "l"(p)
+               : "memory");
 }
 
 // index of the first entry >= x in a sorted int32 range, or end
