@@ -477,11 +477,12 @@ void sparsifier_free(pdg_handle hp) {
   delete hp;
 }
 
-int sparsify_batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_ptr, const int64_t* row_ptr,
-                        const int32_t* col, const double* w, const int32_t* parent, int mem_kind,
-                        const pdg_options* opt, void* stream) {
-  if (!out) return PDG_E_INVALID_ARG;
-  *out = nullptr;
+// late: host weights may follow on a second stream (*late: whether they did)
+static int batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_ptr, const int64_t* row_ptr,
+                      const int32_t* col, const double* w, const int32_t* parent, int mem_kind, const pdg_options* opt,
+                      void* stream, bool* late) {
+  const bool may_be_late = *late;
+  *late = false;
   if (num_graphs < 1 || !vtx_ptr || !row_ptr || !parent || (mem_kind != PDG_MEM_HOST && mem_kind != PDG_MEM_DEVICE))
     return PDG_E_INVALID_ARG;
   if (vtx_ptr[0] != 0) return PDG_E_INVALID_ARG;
@@ -547,15 +548,11 @@ int sparsify_batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_
   if (!(h.hsc = static_cast<DevScalars*>(pinned_alloc(sizeof(DevScalars))))) return fail(PDG_E_OOM);
   if ((st = alloc_n(h, &h.dsc, 1))) return fail(st);
   if (cudaMemsetAsync(h.dsc, 0, sizeof(DevScalars), h.stream) != cudaSuccess) return fail(PDG_E_CUDA);
-  if (mem_kind == PDG_MEM_HOST && h.nnz >= kLateWeights && h.sstream) {
+  if (may_be_late && mem_kind == PDG_MEM_HOST && h.nnz >= kLateWeights && h.sstream) {
+    *late = h.w_pending = true;
     const size_t before = h.device_bytes;
-    h.w_pending = alloc_n(h, &h.w_mirror, h.nnz) == PDG_OK && alloc_n(h, &h.w_place, h.m) == PDG_OK;
+    if ((st = alloc_n(h, &h.w_mirror, h.nnz)) || (st = alloc_n(h, &h.w_place, h.m))) return fail(st);
     h.device_bytes = before;  // (given back during init)
-    if (!h.w_pending) {  // no room for the places: the weights come first
-      cudaGetLastError();
-      device_release(h, h.w_mirror);
-      h.w_mirror = nullptr;
-    }
   }
   if ((st = alloc_n(h, &h.parent, n)) || (st = alloc_n(h, &h.d_vtx_ptr, num_graphs + 1)) ||
       (st = alloc_n(h, &h.blk_a, 10240)) || (st = alloc_n(h, &h.blk_b, 2048)) ||
@@ -652,6 +649,19 @@ int sparsify_batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_
   h.k_mem.assign(num_graphs, -1);
   *out = hp;
   return PDG_OK;
+}
+
+int sparsify_batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_ptr, const int64_t* row_ptr,
+                        const int32_t* col, const double* w, const int32_t* parent, int mem_kind,
+                        const pdg_options* opt, void* stream) {
+  if (!out) return PDG_E_INVALID_ARG;
+  *out = nullptr;
+  bool late = true;
+  int st = batch_init(out, num_graphs, vtx_ptr, row_ptr, col, w, parent, mem_kind, opt, stream, &late);
+  // late weights take up to 16 bytes an entry beside the layout's arrays: without that room they come first
+  if (st == PDG_E_OOM && late)
+    st = batch_init(out, num_graphs, vtx_ptr, row_ptr, col, w, parent, mem_kind, opt, stream, &(late = false));
+  return st;
 }
 
 int pdg_spanning_tree(int64_t n, const int64_t* row_ptr, const int32_t* col, const double* w, int mem_kind,

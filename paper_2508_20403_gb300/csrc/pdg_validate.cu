@@ -264,8 +264,10 @@ int build_edge_list(Handle& h) {
   PDG_CUDA(cudaGetLastError());
   device_release(h, h.up_count);
   device_release(h, h.up_off);
+  device_release(h, h.w_mirror);
   h.up_count = nullptr;
   h.up_off = nullptr;
+  h.w_mirror = nullptr;
   return PDG_OK;
 }
 
@@ -277,10 +279,8 @@ int finish_weights(Handle& h) {
   ++h.launches;
   k_edge_weights<<<grid_for(h, h.m), kBlock, 0, h.stream>>>(h.w, h.w_place, h.m, h.el_w, h.dsc);
   PDG_CUDA(cudaGetLastError());
-  device_release(h, h.w_mirror);
   device_release(h, h.w_place);
   device_release(h, h.w);
-  h.w_mirror = nullptr;
   h.w_place = nullptr;
   h.w = nullptr;
   return PDG_OK;

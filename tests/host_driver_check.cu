@@ -168,7 +168,32 @@ void graph_of_old_buffers() {
   for (void* p : taken) free(p);
 }
 
+// Memory that is enough for an init whose weights come first is enough for one that may let them come late.
+void late_weights_memory() {
+  for (int64_t degree : {6, 24, 200}) {
+    const int64_t n = (int64_t(1) << 21) / degree;
+    fake::no_streams = true;  // no second stream: the weights come first
+    fake::peak = 0;
+    sparsifier_free(make(n, degree, false));
+    const size_t enough = fake::peak;
+    fake::no_streams = false;
+    for (size_t capacity : {enough, enough + enough / 8, enough + enough / 4, enough + enough / 2, 2 * enough}) {
+      fake::capacity = capacity;
+      int st = PDG_OK;
+      pdg_handle h = make(n, degree, false, &st);
+      if (st != PDG_OK) fake::die("degree %d, capacity %zu, enough %zu: status %d", (int)degree, capacity, enough, st);
+      sparsifier_free(h);
+      CHECK(fake::live.empty());
+    }
+    fake::capacity = SIZE_MAX;
+    const int late = fake::launches("k_edge_weights");
+    sparsifier_free(make(n, degree, false));
+    CHECK(fake::launches("k_edge_weights") == late + 1);  // with room they do come late
+  }
+}
+
 const std::map<std::string, void (*)()> kChecks = {
+    {"late_weights_memory", late_weights_memory},
     {"graph_of_old_buffers", graph_of_old_buffers},
     {"oom_join", oom_join},
     {"oom_table", oom_table},

@@ -46,3 +46,9 @@ def test_a_graph_ends_with_its_buffers(checker):
     """A budget, captured and replayed; a larger one that runs out of memory; the first again: the buffers are new ones
     of the old sizes, so the old graph must not run."""
     _run(checker, "graph_of_old_buffers")
+
+
+def test_late_weights_need_no_more_memory(checker):
+    """Host weights that follow on a second stream need the places of the mirror images; where memory is short of them
+    but enough for the plain order, init still succeeds."""
+    _run(checker, "late_weights_memory")
