@@ -136,6 +136,7 @@ __global__ void k_reset_attempt(DevScalars* dsc, uint4* __restrict__ tab, int64_
   dsc->err &= ERR_RANGE | ERR_TIMEOUT | ERR_BOUNDS;  // errors of steps A1-A3 end the recovery
   dsc->epoch++;
   dsc->bounds_site = 0;
+  dsc->bounds_pos = -1;
   dsc->rounds_used = 0;
   dsc->n_cand = 0;
   dsc->n_list = 0;
@@ -823,18 +824,27 @@ int sparsify_init(pdg_handle* out, int64_t n, const int64_t* row_ptr, const int3
 
 namespace pdg {
 
-// The recovery driver shared by recover_offtree and recover_offtree_batch.
-// Diagnostics for a failed index check: where position p sits in the
-// segment and tier lists of the attempt that failed.
+// Diagnostics for a failed index check of the tiers: where position p sits in the segment and tier lists of the attempt
+// that failed.  Counts and positions of such an attempt may be anything: nothing beyond the buffers is read.
 static void debug_position(Handle& h, int64_t p) {
   const int64_t N = h.hsc->n_cand, S = h.hsc->n_seg, NB = h.hsc->n_big, NBS = h.hsc->n_big_seg;
-  std::vector<int32_t> seg(S + 1), bpos(NB), bseg(NBS);
-  std::vector<uint8_t> st(N);
-  cudaMemcpy(seg.data(), h.seg_begin, sizeof(int32_t) * (S + 1), cudaMemcpyDeviceToHost);
-  cudaMemcpy(bpos.data(), h.big_pos, sizeof(int32_t) * NB, cudaMemcpyDeviceToHost);
-  cudaMemcpy(bseg.data(), h.big_seg, sizeof(int32_t) * NBS, cudaMemcpyDeviceToHost);
-  cudaMemcpy(st.data(), h.state, N, cudaMemcpyDeviceToHost);
-  int64_t q = std::upper_bound(seg.begin(), seg.end(), (int32_t)p) - seg.begin() - 1;
+  auto in = [&](int64_t count, int64_t lo) { return count >= lo && count <= h.tier_cap; };
+  std::vector<int32_t> seg, bpos, bseg;
+  std::vector<uint8_t> st;
+  auto fetch = [](auto& to, const auto* from, int64_t count) {
+    to.resize((size_t)count);
+    return count == 0 || cudaMemcpy(to.data(), from, sizeof(to[0]) * (size_t)count, cudaMemcpyDeviceToHost) == cudaSuccess;
+  };
+  if (!in(N, 1) || !in(S, 1) || !in(NB, 0) || !in(NBS, 0) || p < 0 || p >= N || !fetch(seg, h.seg_begin, S + 1) ||
+      !fetch(bpos, h.big_pos, NB) || !fetch(bseg, h.big_seg, NBS) || !fetch(st, h.state, N)) {
+    cudaGetLastError();
+    fprintf(stderr, "pdgrass debug: p %lld N %lld n_seg %lld n_big %lld n_big_seg %lld: no position\n", (long long)p,
+            (long long)N, (long long)S, (long long)NB, (long long)NBS);
+    return;
+  }
+  // the last segment that begins at or before p (the first one, should none)
+  const int64_t q = std::min<int64_t>(
+      std::max<int64_t>(std::upper_bound(seg.begin(), seg.end(), (int32_t)p) - seg.begin() - 1, 0), S - 1);
   bool mono = true;
   for (int64_t i = 0; i < S; i++)
     if (seg[i + 1] <= seg[i]) mono = false;
@@ -853,6 +863,7 @@ static void debug_position(Handle& h, int64_t p) {
           (int)seg_big, (int)st[p], (long long)NB, (long long)big_total, (long long)dup, seg[S]);
 }
 
+// The recovery driver shared by recover_offtree and recover_offtree_batch.
 static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, const int64_t* user_out_ptr,
                         int32_t* out_ids, double* out_scores, int out_mem_kind, int64_t* out_count,
                         int32_t* graph_status) {
@@ -1075,7 +1086,9 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
                         "constrained %lld, rounds %d, attempt %d)\n", h.hsc->bounds_site, h.hsc->bounds_where,
                 (long long)h.hsc->bounds_pos, (long long)h.hsc->bounds_val, (long long)h.hsc->n_big,
                 (long long)h.hsc->n_constrained, h.hsc->rounds_used, attempts);
-      if (getenv("PDG_DEBUG_BOUNDS") && h.hsc->bounds_pos >= 0) debug_position(h, h.hsc->bounds_pos / 64);
+      // (a check without a site, the scoring's, records no position; the lists are the tiers')
+      if (getenv("PDG_DEBUG_BOUNDS") && h.tiered && h.hsc->bounds_site != 0 && h.hsc->bounds_pos >= 0)
+        debug_position(h, h.hsc->bounds_pos / 64);
       return PDG_E_CUDA;
     }
     if (err & ERR_CAPACITY) {

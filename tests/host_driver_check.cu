@@ -192,7 +192,37 @@ void late_weights_memory() {
   }
 }
 
+// A failed index check ends the recovery; with PDG_DEBUG_BOUNDS set its report reads nothing that is not there: no
+// buffers of the tiers after a join, no position the check did not record, no segment that was not made.
+void failed_index_check() {
+  for (bool tiers : {false, true})
+    for (int site : {0, 3})
+      for (int64_t pos : {-1ll, 0ll, 64ll * 70, 1ll << 40})
+        for (int64_t n : {0, 1, 50}) {
+          pdg_handle h = make(2000, 12, false);
+          script([&](DevScalars& d) {
+            d = DevScalars{};
+            d.e_max = INT_MIN;
+            if (tiers && !h->h.tiered) {
+              d.err = ERR_DENSE;
+              return;
+            }
+            d.err = ERR_BOUNDS;
+            d.bounds_site = site;
+            d.bounds_pos = pos;
+            d.n_cand = d.n_big = n;
+            d.n_seg = n / 2;
+            d.n_big_seg = n / 3;
+          });
+          CHECK(recover(h, 0.5) == PDG_E_CUDA);
+          CHECK(h->h.stats[11] == site);
+          script([](DevScalars&) {});
+          sparsifier_free(h);
+        }
+}
+
 const std::map<std::string, void (*)()> kChecks = {
+    {"failed_index_check", failed_index_check},
     {"late_weights_memory", late_weights_memory},
     {"graph_of_old_buffers", graph_of_old_buffers},
     {"oom_join", oom_join},

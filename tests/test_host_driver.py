@@ -52,3 +52,7 @@ def test_late_weights_need_no_more_memory(checker):
     """Host weights that follow on a second stream need the places of the mirror images; where memory is short of them
     but enough for the plain order, init still succeeds."""
     _run(checker, "late_weights_memory")
+
+
+def test_report_of_a_failed_index_check(checker):
+    _run(checker, "failed_index_check", PDG_DEBUG_BOUNDS="1")
