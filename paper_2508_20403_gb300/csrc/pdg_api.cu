@@ -940,8 +940,13 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
     dev_ids = h.out_ids;
     dev_scores = out_scores ? h.out_scores : nullptr;
   }
-  // the tiers only where a recovery of the same kind needed them
-  if (!(h.c_mem == c && h.mode_mem == h.opt.score_mode)) h.tiered = false;
+  // the tiers only where a recovery of the same kind and no larger budget needed them
+  if (h.dense_c != c || h.dense_mode != h.opt.score_mode) {
+    h.dense_k = INT64_MAX;
+    h.dense_c = c;
+    h.dense_mode = h.opt.score_mode;
+  }
+  h.tiered = total_k >= h.dense_k;
   h.launches = 0;
   DepScope dep_scope(h);  // kernels of the recovery may launch as programmatic dependents
   const bool prof = h.opt.profile != 0;
@@ -1059,6 +1064,7 @@ static int run_recovery(pdg_sparsifier* hp, const double* alpha, int32_t c, cons
     if (err & ERR_TIMEOUT) return PDG_E_TIMEOUT;
     if ((err & ERR_DENSE) && !h.tiered) {  // the cells are too full for the join: the tiers decide these candidates
       h.tiered = true;
+      h.dense_k = std::min(h.dense_k, total_k);
       if ((st = ensure_candidates(h, h.Rcap, c))) return st;
       first = false;
       continue;

@@ -251,9 +251,12 @@ struct Handle {
   int64_t* d_cand_ptr = nullptr;  // G+1
   int64_t* d_graph_tmp = nullptr;  // G+1 scratch
 
-  // steps A5 + A6: false: the join; true: the tiers (this attempt's candidates fill the join's cells too much;
-  // remembered for later recoveries with (c_mem, mode_mem))
+  // steps A5 + A6: false: the join; true: the tiers (this attempt's candidates fill the join's cells too much).  A
+  // recovery with (dense_c, dense_mode) begins with the tiers from that budget on whose candidates did; those of
+  // smaller budgets are a part of them and keep the join (and the tiers decide the same where this guesses wrong).
   bool tiered = false;
+  int64_t dense_k = INT64_MAX;  // sum over the graphs
+  int dense_c = -1, dense_mode = -1;
   // selection: the edges of the boundary bucket and above (grow-only)
   int64_t list_cap = 0;
   int32_t* list_id = nullptr;

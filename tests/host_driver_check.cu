@@ -221,7 +221,39 @@ void failed_index_check() {
         }
 }
 
+// Budgets from some size on fill the join's cells too much and go to the tiers; the handle remembers that for budgets of
+// that size, not for smaller ones, and for the same c.
+void tiers_by_budget() {
+  pdg_handle h = make(2000, 12, false);
+  int joins = 0, tiers = 0;
+  fake::on_launch = [&](const std::string& name, void**) {
+    joins += fake::named(name, "k_join_insert");
+    tiers += fake::named(name, "k_build_records");
+  };
+  double budget = 0.0;
+  script([&](DevScalars& d) { d.err = !h->h.tiered && budget >= 0.4 ? ERR_DENSE : 0; });
+  auto run = [&](double b, int c, int want_joins, int want_tiers) {
+    budget = b;
+    joins = tiers = 0;
+    CHECK(recover(h, b, c) == PDG_OK);
+    if (joins != want_joins || tiers != want_tiers)
+      fake::die("budget %g, c %d: %d joins, %d tiers", b, c, joins, tiers);
+  };
+  run(0.1, 2, 1, 0);
+  run(0.5, 2, 1, 1);  // the join gives up
+  run(0.5, 2, 0, 1);  // remembered
+  run(0.1, 2, 1, 0);  // a smaller budget never met such cells
+  run(0.5, 2, 0, 1);  // still remembered
+  run(0.9, 2, 0, 1);  // more candidates, fuller cells
+  run(0.4, 2, 1, 1);
+  run(0.4, 2, 0, 1);
+  run(0.5, 1, 1, 1);  // another c has other cells
+  run(0.1, 1, 1, 0);
+  sparsifier_free(h);
+}
+
 const std::map<std::string, void (*)()> kChecks = {
+    {"tiers_by_budget", tiers_by_budget},
     {"failed_index_check", failed_index_check},
     {"late_weights_memory", late_weights_memory},
     {"graph_of_old_buffers", graph_of_old_buffers},

@@ -56,3 +56,9 @@ def test_late_weights_need_no_more_memory(checker):
 
 def test_report_of_a_failed_index_check(checker):
     _run(checker, "failed_index_check", PDG_DEBUG_BOUNDS="1")
+
+
+def test_tiers_are_remembered_by_budget(checker):
+    """A budget whose candidates fill the join's cells is decided by the tiers, and from the start the next time; smaller
+    budgets of the same handle keep the join."""
+    _run(checker, "tiers_by_budget")
