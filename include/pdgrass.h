@@ -211,6 +211,15 @@ int pdg_handle_info(pdg_handle h, int64_t* n, int64_t* m, int64_t* n_offtree, in
 int pdg_last_stats(pdg_handle h, int64_t* stats);
 
 /*
+ * pdg_last_path -- what decided the candidates of the handle's last recovery
+ * (steps A5 + A6): PDG_PATH_JOIN, or PDG_PATH_TIERS where their cells were too
+ * full for the join.  Both decide the same.
+ */
+#define PDG_PATH_JOIN 0
+#define PDG_PATH_TIERS 1
+int pdg_last_path(pdg_handle h, int32_t* path);
+
+/*
  * pdg_last_timings -- device time in milliseconds of each step of the last
  * recovery, measured with CUDA events on the handle's stream when
  * opt.profile = 1 (zeros otherwise): [0] classify (A1), [1] tree (A2),

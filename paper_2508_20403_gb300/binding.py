@@ -32,12 +32,14 @@ MEM_DEVICE = 1
 SCORE_STRETCH = 0
 SCORE_RESISTANCE = 1
 MAX_C = 3
+PATH_JOIN = 0
+PATH_TIERS = 1
 TREE_MAX_WEIGHT = 0
 TREE_FEGRASS = 1
 
 EXPORTS = ("pdg_default_options", "pdg_status_string", "sparsify_init", "recover_offtree", "sparsifier_free",
            "pdg_edge_endpoints", "sparsify_batch_init", "recover_offtree_batch", "pdg_handle_info",
-           "pdg_last_stats", "pdg_last_timings", "pdg_spanning_tree", "pdg_pcg_quality", "pdg_pcg_trace",
+           "pdg_last_stats", "pdg_last_path", "pdg_last_timings", "pdg_spanning_tree", "pdg_pcg_quality", "pdg_pcg_trace",
            "pdg_edge_endpoints_noalloc")
 STEP_NAMES = ("classify", "tree", "score", "select", "sort", "accept", "budget", "total")
 
@@ -88,6 +90,8 @@ def load(path: Optional[str] = None):
     L.pdg_handle_info.restype = c_int
     L.pdg_last_stats.argtypes = [P, P]
     L.pdg_last_stats.restype = c_int
+    L.pdg_last_path.argtypes = [P, ctypes.POINTER(i32)]
+    L.pdg_last_path.restype = c_int
     L.pdg_last_timings.argtypes = [P, P]
     L.pdg_last_timings.restype = c_int
     L.pdg_edge_endpoints_noalloc.argtypes = [i64, P, P, P, i64, P, P, P]
@@ -264,6 +268,14 @@ class Sparsifier:
         keys = ("candidates", "subtasks", "max_subtask", "warp_or_single", "coop_candidates", "coop_rounds",
                 "retries", "attempts", "launches", "coop_constrained", "coop_pairs", "bounds_site")
         return dict(zip(keys, (int(x) for x in a)))
+
+    def last_path(self) -> int:
+        """PATH_JOIN or PATH_TIERS: what decided the last recovery's candidates."""
+        v = ctypes.c_int32(-1)
+        st = self._L.pdg_last_path(self._h, ctypes.byref(v))
+        if st:
+            raise PdgError(st, "pdg_last_path")
+        return int(v.value)
 
     def last_timings(self) -> dict:
         a = np.zeros(8, dtype=np.float32)

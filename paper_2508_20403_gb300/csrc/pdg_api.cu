@@ -1244,6 +1244,12 @@ int pdg_last_stats(pdg_handle hp, int64_t* stats) {
   return PDG_OK;
 }
 
+int pdg_last_path(pdg_handle hp, int32_t* path) {
+  if (!hp || !path) return PDG_E_INVALID_ARG;
+  *path = hp->h.tiered ? PDG_PATH_TIERS : PDG_PATH_JOIN;
+  return PDG_OK;
+}
+
 int pdg_edge_endpoints(pdg_handle hp, const int32_t* ids, int64_t count, int32_t* u, int32_t* v, int mem_kind) {
   if (!hp || count < 0 || (count > 0 && (!ids || !u || !v)) || (mem_kind != PDG_MEM_HOST && mem_kind != PDG_MEM_DEVICE))
     return PDG_E_INVALID_ARG;
