@@ -493,78 +493,75 @@ __global__ void k_pc_capacitance(const uint64_t* __restrict__ table, const doubl
 }
 
 // --- inverse of C in place: the symmetric sweep by blocks of kSw pivots, on the lower triangle (C is symmetric
-// positive definite: no pivoting).  For the pivot block p: B = inv(C_pp), L_i = C_ip, R_i = L_i B; then
-// C_ij -= L_i R_j^T, C_ip = R_i, C_pj = R_j^T, C_pp = -B, and after all blocks C is -inv(C).  Two launches per block.
+// positive definite: no pivoting).  For the pivot block p, C_pp = M D M^T with M unit lower triangular: Y_i = C_ip M^-T,
+// R_i = Y_i D^-1 M^-1 = C_ip inv(C_pp); then C_ij -= (Y_i D^-1) Y_j^T, C_ip = R_i, C_pj = R_j^T, C_pp = -inv(C_pp), and
+// after all blocks C is -inv(C).  Two launches per block.
+// As accurate as pivot by pivot over the whole matrix.  (With R_i = C_ip inv(C_pp) from the block's explicit inverse and
+// C_ij -= C_ip R_j^T, products with inv(C) were 10 to 60 times further off, and the preconditioner's residual, 10^-3
+// where off-tree edges outweigh the tree 10^6 times, was of order 1.)
 // Bound by FP64 (k^3 / 2 multiply-adds at two a clock and SM) and the chain of k pivots (0.7 us each, mostly the
 // reciprocal): k = 500 takes 0.55 ms; pivot by pivot over the whole matrix it was two launches a pivot, 4.4 ms of
 // kernels and as much between them.
 constexpr int kSw = 32;
 
-// B (every block for itself: 32 rows in the registers of eight warps, the pivot row through shared memory), then L and
-// R of this block's eight rows
+// The factors of C_pp (every block for itself: 32 rows in the registers of eight warps, the scaled pivot rows, which are
+// the columns of M, through shared memory), then Y and R of this block's eight rows.  A row of the pivot block takes its
+// row of the identity along instead, and its R is its row of inv(C_pp).
 __global__ void __launch_bounds__(256) k_pc_sweep_panel(const double* __restrict__ C, int k, int p0,
-                                                        double* __restrict__ B, double* __restrict__ R,
-                                                        double* __restrict__ L) {
-  __shared__ double s_row[2][kSw], b[kSw][kSw + 1];
+                                                        double* __restrict__ D, double* __restrict__ R,
+                                                        double* __restrict__ Y) {
+  __shared__ double b[kSw][kSw + 1];  // b[p][j] = M[j][p], j > p
+  __shared__ double s_d[kSw];         // D^-1
   const int nb = min(kSw, k - p0), lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int row = blockIdx.x * 8 + w;  // of L and R
-  double l = 0.0;
-  if (row < k && lane < nb && (row < p0 || row >= p0 + nb))
-    l = row > p0 ? C[(int64_t)row * k + p0 + lane] : C[(int64_t)(p0 + lane) * k + row];
+  const int row = blockIdx.x * 8 + w;  // of Y and R
+  double x = 0.0;
+  if (row >= p0 && row < p0 + nb) x = row - p0 == lane ? 1.0 : 0.0;
+  else if (row < k && lane < nb) x = row > p0 ? C[(int64_t)row * k + p0 + lane] : C[(int64_t)(p0 + lane) * k + row];
   double v[4];  // rows w, w + 8, w + 16, w + 24
 #pragma unroll
   for (int r = 0; r < 4; r++) {
     const int i = w + 8 * r;
     v[r] = i < nb && lane < nb ? C[(int64_t)(p0 + max(i, lane)) * k + p0 + min(i, lane)] : (i == lane ? 1.0 : 0.0);
   }
-  if (w == 0) {
-    const double d = 1.0 / __shfl_sync(0xffffffffu, v[0], 0);
-    v[0] = lane == 0 ? d : v[0] * d;
-    s_row[0][lane] = v[0];
-  }
+  auto pivot_row = [&](double a, int p) {  // row p, up to date: scaled
+    const double d = 1.0 / __shfl_sync(0xffffffffu, a, p);
+    b[p][lane] = a * d;
+    if (lane == p) s_d[p] = d;
+  };
+  if (w == 0) pivot_row(v[0], 0);
   __syncthreads();
 #pragma unroll
   for (int r0 = 0; r0 < 4; r0++)
     for (int q = 0; q < 8; q++) {
-      const int p = 8 * r0 + q;  // the pivot: row r0 of warp q, scaled by the warp already
-      const double piv = s_row[p & 1][lane];
-      auto update = [&](double x) {
-        const double f = __shfl_sync(0xffffffffu, x, p);
-        return (lane == p ? 0.0 : x) - f * piv;
+      const int p = 8 * r0 + q;  // the pivot: row r0 of warp q
+      const double piv = b[p][lane];
+      auto update = [&](double a) {
+        const double f = __shfl_sync(0xffffffffu, a, p);
+        return lane > p ? a - f * piv : a;
       };
       // the next pivot's warp first brings that row up to date and scales it: its division runs beside the others'
       // multiply-adds
       const bool next_here = w == ((q + 1) & 7) && p + 1 < kSw;
-      auto scale = [&](double x) {
-        x = update(x);
-        const double d = 1.0 / __shfl_sync(0xffffffffu, x, p + 1);
-        x = lane == p + 1 ? d : x * d;
-        s_row[(p + 1) & 1][lane] = x;
-        return x;
-      };
       const int rn = q == 7 ? r0 + 1 : r0;
 #pragma unroll
       for (int r = 0; r < 4; r++)
-        if (next_here && r == rn) v[r] = scale(v[r]);
+        if (next_here && r == rn) pivot_row(update(v[r]), p + 1);
 #pragma unroll
-      for (int r = 0; r < 4; r++) {
-        const bool pivot_row = w == q && r == r0;
-        if (!pivot_row && !(next_here && r == rn)) v[r] = update(v[r]);
-      }
+      for (int r = 0; r < 4; r++)  // the rows after it
+        if (w + 8 * r > p + 1) v[r] = update(v[r]);
+      x = update(x);
       __syncthreads();
     }
-#pragma unroll
-  for (int r = 0; r < 4; r++) b[w + 8 * r][lane] = v[r];
-  __syncthreads();
-  if (blockIdx.x == 0)
-#pragma unroll
-    for (int r = 0; r < 4; r++) B[(w + 8 * r) * kSw + lane] = v[r];
+  if (blockIdx.x == 0 && w == 0) D[lane] = s_d[lane];
   if (row >= k) return;  // (warp-uniform)
-  double x = 0.0;
+  Y[(int64_t)row * kSw + lane] = x;
+  double t = x * s_d[lane];
 #pragma unroll
-  for (int t = 0; t < kSw; t++) x += __shfl_sync(0xffffffffu, l, t) * b[t][lane];
-  L[(int64_t)row * kSw + lane] = l;
-  R[(int64_t)row * kSw + lane] = x;
+  for (int p = kSw - 1; p > 0; p--) {
+    const double f = __shfl_sync(0xffffffffu, t, p);
+    if (lane < p) t -= f * b[lane][p];
+  }
+  R[(int64_t)row * kSw + lane] = t;
 }
 
 // the t-th tile of the lower triangle, row by row (y: row); the grid holds no others, so that up to 152 of them lie on
@@ -577,16 +574,16 @@ __device__ __forceinline__ int2 lower_tile(uint32_t t) {
 }
 
 __global__ void __launch_bounds__(256) k_pc_sweep_update(double* __restrict__ C, int k, int p0,
-                                                         const double* __restrict__ B, const double* __restrict__ R,
-                                                         const double* __restrict__ L) {
+                                                         const double* __restrict__ D, const double* __restrict__ R,
+                                                         const double* __restrict__ Y) {
   __shared__ double l[kSw][kSw + 1], r[kSw][kSw + 1];  // by row of C
   const int2 tile = lower_tile(blockIdx.x);
   const int i0 = tile.y * kSw, j0 = tile.x * kSw, tid = threadIdx.x;
   const bool pi = i0 == p0, pj = j0 == p0;
   for (int q = tid; q < kSw * kSw; q += 256) {
     const int i = q / kSw, t = q % kSw;
-    l[i][t] = i0 + i >= k ? 0.0 : pj ? R[(int64_t)(i0 + i) * kSw + t] : L[(int64_t)(i0 + i) * kSw + t];
-    r[i][t] = j0 + i < k ? R[(int64_t)(j0 + i) * kSw + t] : 0.0;
+    l[i][t] = i0 + i >= k ? 0.0 : pj ? R[(int64_t)(i0 + i) * kSw + t] : Y[(int64_t)(i0 + i) * kSw + t] * D[t];
+    r[i][t] = j0 + i >= k ? 0.0 : pi ? R[(int64_t)(j0 + i) * kSw + t] : Y[(int64_t)(j0 + i) * kSw + t];
   }
   __syncthreads();
   const int ti = tid / 16, tj = tid % 16;  // rows ti, ti + 16, columns tj, tj + 16
@@ -608,7 +605,7 @@ __global__ void __launch_bounds__(256) k_pc_sweep_update(double* __restrict__ C,
       const int i = ti + 16 * a, j = tj + 16 * c;
       if (i0 + i >= k || j0 + j >= k) continue;
       double* at = C + (int64_t)(i0 + i) * k + j0 + j;
-      if (pi && pj) *at = -B[i * kSw + j];
+      if (pi && pj) *at = -l[i][j];
       else if (pj) *at = l[i][j];
       else if (pi) *at = r[j][i];
       else *at -= acc[a][c];
@@ -780,7 +777,7 @@ int pcg_quality(Handle& h, const int32_t* ids, int64_t k, const double* b, doubl
   int32_t *ea = nullptr, *eb = nullptr, *seen = nullptr, *flags = nullptr, *icnt = nullptr, *iedge = nullptr;
   int64_t *tptr = nullptr, *iptr = nullptr;
   double *wup = nullptr, *E = nullptr, *D = nullptr, *sums = nullptr, *ewk = nullptr;
-  double *C = nullptr, *swR = nullptr, *swL = nullptr, *swB = nullptr, *dw = nullptr, *bb = nullptr, *x = nullptr;
+  double *C = nullptr, *swR = nullptr, *swY = nullptr, *swD = nullptr, *dw = nullptr, *bb = nullptr, *x = nullptr;
   double *r = nullptr, *z = nullptr, *p = nullptr, *Ap = nullptr, *t = nullptr;
   double *qv = nullptr, *parts = nullptr;
   double2* dist = nullptr;
@@ -794,7 +791,7 @@ int pcg_quality(Handle& h, const int32_t* ids, int64_t k, const double* b, doubl
   place(&arc_uv, m); place(&succ, A); place(&tin, n); place(&tout, n); place(&wup, n); place(&tour, A); place(&E, A);
   place(&sums, T); place(&dist, A); place(&D, A); place(&depth, A); place(&dsums, T); place(&ea, k); place(&eb, k);
   place(&ewk, k); place(&seen, m); place(&flags, 4); place(&icnt, n); place(&iptr, n + 1); place(&iedge, 2 * k);
-  place(&C, k * k); place(&swR, kSw * k); place(&swL, kSw * k); place(&swB, kSw * kSw); place(&ekey, 2 * k);
+  place(&C, k * k); place(&swR, kSw * k); place(&swY, kSw * k); place(&swD, kSw); place(&ekey, 2 * k);
   place(&epos, 2 * k); place(&erank, 2 * k); place(&gaps, 2 * k * gap_rows); place(&dw, n); place(&bb, n);
   place(&x, n); place(&r, n); place(&z, n); place(&p, n); place(&Ap, n); place(&t, n);
   place(&qv, k); place(&parts, 4 * kDotBlocks + std::max<int64_t>(kDotBlocks, T));
@@ -892,8 +889,8 @@ int pcg_quality(Handle& h, const int32_t* ids, int64_t k, const double* b, doubl
     k_pc_capacitance<<<grid_for(h, k * k), kBlock, 0, s>>>(gaps, dist, depth, epos, erank, ewk, (int)k, C);
     const int blocks = (int)((k + kSw - 1) / kSw);
     for (int p0 = 0; p0 < k; p0 += kSw) {
-      k_pc_sweep_panel<<<(int)((k + 7) / 8), 256, 0, s>>>(C, (int)k, p0, swB, swR, swL);
-      k_pc_sweep_update<<<blocks * (blocks + 1) / 2, 256, 0, s>>>(C, (int)k, p0, swB, swR, swL);
+      k_pc_sweep_panel<<<(int)((k + 7) / 8), 256, 0, s>>>(C, (int)k, p0, swD, swR, swY);
+      k_pc_sweep_update<<<blocks * (blocks + 1) / 2, 256, 0, s>>>(C, (int)k, p0, swD, swR, swY);
     }
     k_pc_sweep_end<<<blocks * (blocks + 1) / 2, 256, 0, s>>>(C, (int)k);
     // incidence lists of the recovered edges, in edge order
