@@ -183,7 +183,7 @@ __device__ __forceinline__ double tour_value(const TourArgs& a, int32_t t) {
 // (kFlowEdges and kDrops leave the values in D for the scan)
 template <int MODE, int ITEMS>
 __global__ void __launch_bounds__(kTourThreads) k_pc_tour_sums(TourArgs a) {
-  __shared__ double sh[33];
+  __shared__ double sh[kTourThreads / 32];
   const int64_t base = ((int64_t)blockIdx.x * kTourThreads + threadIdx.x) * ITEMS;
   double s = 0.0;
 #pragma unroll
@@ -193,8 +193,15 @@ __global__ void __launch_bounds__(kTourThreads) k_pc_tour_sums(TourArgs a) {
     if (MODE != kFlow) a.D[base + i] = v;
     s += v;
   }
-  s = block_sum_d(s, sh);
-  if (threadIdx.x == 0) a.sums[blockIdx.x] = s;
+  // added up as k_pc_tour_scan adds it up, so that a tile's prefixes end where the next tile's begin
+  const double incl = warp_incl_scan_d(s);
+  if ((threadIdx.x & 31) == 31) sh[threadIdx.x >> 5] = incl;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double sum = 0.0;
+    for (int i = 0; i < kTourThreads / 32; i++) sum += sh[i];
+    a.sums[blockIdx.x] = sum;
+  }
 }
 
 template <int MODE, int ITEMS>
@@ -217,7 +224,9 @@ __global__ void __launch_bounds__(kTourThreads) k_pc_tour_scan(TourArgs a) {
   const double incl = warp_incl_scan_d(s);
   if (lane == 31) sh2[w] = incl;
   __syncthreads();
-  double run = pre;
+  // what stands before a position in its tile is added up first, and to the tiles before it last: the sum of the tour so
+  // far may be many times larger, and each addition to it rounds at its size
+  double run = 0.0;
   for (int i = 0; i < w; i++) run += sh2[i];
   const double left = __shfl_up_sync(0xffffffffu, incl, 1);
   if (lane) run += left;
@@ -226,9 +235,9 @@ __global__ void __launch_bounds__(kTourThreads) k_pc_tour_scan(TourArgs a) {
   for (int i = 0; i < ITEMS; i++) {
     if (base + i >= a.A) break;
     if (MODE == kFlow || MODE == kFlowEdges) {
-      a.E[base + i] = run;
+      a.E[base + i] = pre + run;
     } else if (t[i] >= 0) {
-      double x = run + v[i];
+      double x = pre + (run + v[i]);
       if (MODE == kDropsZ) {
         if (a.t) x = a.t[t[i]] - x;
         zs += x;
