@@ -149,11 +149,7 @@ __global__ void k_reset_attempt(DevScalars* dsc, uint4* __restrict__ tab, int64_
   dsc->n_big_seg = 0;
   dsc->max_seg = 0;
   dsc->big_regs = 0;
-  dsc->undecided = 0;
   dsc->radix_sel = 0;
-  dsc->radix_skip = 0;
-  dsc->radix_len = 0;
-  dsc->n_warp_cand = 0;
   dsc->n_constrained = 0;
   dsc->n_big_chunk = 0;
   dsc->finish_left = 0;
@@ -556,7 +552,7 @@ static int batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_pt
     h.device_bytes = before;  // (given back during init)
   }
   if ((st = alloc_n(h, &h.parent, n)) || (st = alloc_n(h, &h.d_vtx_ptr, num_graphs + 1)) ||
-      (st = alloc_n(h, &h.blk_a, 10240)) || (st = alloc_n(h, &h.blk_b, 2048)) ||
+      (st = alloc_n(h, &h.blk_a, 10240)) ||
       (st = take_csr(h, row_ptr, col, w, mem_kind)))
     return fail(st);
   if (cudaMemcpyAsync(h.parent, parent, sizeof(int32_t) * n, kind, h.stream) != cudaSuccess ||
@@ -616,7 +612,7 @@ static int batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_pt
       (st = alloc_n(h, &h.lca_count, n)) ||
       (st = device_alloc(h, &h.join_part, (size_t)h.num_sms * 8 * (sizeof(int4) + sizeof(int32_t)))) ||
       (st = alloc_n(h, &h.d_k, num_graphs)) || (st = alloc_n(h, &h.d_out_ptr, num_graphs + 1)) ||
-      (st = alloc_n(h, &h.radix_dtot, 256)) || (st = alloc_n(h, &h.radix_hist, kRadixHistWords)) ||
+      (st = alloc_n(h, &h.radix_hist, kRadixHistWords)) ||
       (st = alloc_n(h, &h.radix_counters, 2 * kRadixPassesMax)) ||
       (st = ensure_scan_status(h, std::max<int64_t>(n, num_graphs) + 1)))
     return fail(st);
@@ -636,7 +632,6 @@ static int batch_init(pdg_handle* out, int32_t num_graphs, const int64_t* vtx_pt
       cudaMemcpyAsync(h.d_off_ptr, h.off_ptr_h.data(), sizeof(int64_t) * (num_graphs + 1), cudaMemcpyHostToDevice,
                       h.stream) != cudaSuccess ||
       cudaMemsetAsync(h.hist, 0, sizeof(uint32_t) * (size_t)num_graphs * kSelBins, h.stream) != cudaSuccess ||
-      cudaMemsetAsync(h.radix_dtot, 0, sizeof(uint32_t) * 256, h.stream) != cudaSuccess ||
       cudaMemsetAsync(h.radix_hist, 0, sizeof(uint32_t) * kRadixHistWords, h.stream) != cudaSuccess ||
       (h.w_late && cudaMemcpyAsync(h.hsc, h.dsc, sizeof(DevScalars), cudaMemcpyDeviceToHost, h.stream) != cudaSuccess) ||
       cudaStreamSynchronize(h.stream) != cudaSuccess)
@@ -706,7 +701,7 @@ int pdg_spanning_tree(int64_t n, const int64_t* row_ptr, const int32_t* col, con
   if (!(h.hsc = static_cast<DevScalars*>(pinned_alloc(sizeof(DevScalars))))) return fail(PDG_E_OOM);
   if ((st = alloc_n(h, &h.dsc, 1)) || (st = take_csr(h, row_ptr, col, w, mem_kind)) ||
       (st = alloc_n(h, &h.parent, n)) || (st = alloc_n(h, &h.d_vtx_ptr, 2)) ||
-      (st = alloc_n(h, &h.blk_a, 10240)) || (st = alloc_n(h, &h.blk_b, 2048)))
+      (st = alloc_n(h, &h.blk_a, 10240)))
     return fail(st);
   if (cudaMemcpyAsync(h.d_vtx_ptr, vp, sizeof(vp), cudaMemcpyHostToDevice, h.stream) != cudaSuccess)
     return fail(PDG_E_CUDA);
@@ -772,7 +767,7 @@ static int pcg_entry(int64_t n, const int64_t* row_ptr, const int32_t* col, cons
       !(h.pcg_host = static_cast<double*>(pinned_alloc(sizeof(double) * kPcgParts))))
     return fail(PDG_E_OOM);
   if ((st = alloc_n(h, &h.dsc, 1)) || (st = take_csr(h, row_ptr, col, w, mem_kind)) || (st = alloc_n(h, &h.parent, n)) || (st = alloc_n(h, &h.d_vtx_ptr, 2)) ||
-      (st = alloc_n(h, &h.blk_a, 10240)) || (st = alloc_n(h, &h.blk_b, 2048)) ||
+      (st = alloc_n(h, &h.blk_a, 10240)) ||
       (st = alloc_n(h, &d_ids, std::max<int64_t>(n_edges, 1))) || (st = alloc_n(h, &d_b, n)))
     return fail(st);
   if (cudaMemcpyAsync(h.parent, parent, sizeof(int32_t) * n, kind, h.stream) != cudaSuccess ||

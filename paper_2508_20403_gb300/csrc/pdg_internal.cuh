@@ -87,13 +87,9 @@ struct DevScalars {
   int64_t n_big_seg;    // subtasks in the cooperative tier
   int64_t max_seg;      // largest subtask
   int64_t big_regs;     // registrations the cooperative tier will make
-  int64_t undecided;    // cooperative tier: still undecided after a round
   int64_t active;       // validation: entries above the diagonal minus entries below
   int64_t max_depth;
   int32_t radix_sel;    // radix sort: which ping-pong buffer holds the keys
-  int32_t radix_skip;   // radix sort: the current digit is uniform
-  int64_t radix_len;    // radix sort: histogram length (256 * tiles)
-  int64_t n_warp_cand;  // candidates in the warp tier
   int64_t n_cand_wanted;  // candidates the selection produced (may exceed capacity)
   int64_t n_list;         // selection: edges of the boundary bucket and above (may exceed the list's capacity)
   int64_t n_constrained;  // cooperative tier: candidates with a possible earlier marker
@@ -210,7 +206,6 @@ struct Handle {
   // step 1 outputs
   double* rtree = nullptr;  // r(v) = fl(1/w(v, parent v))
   int64_t* blk_a = nullptr; // per-block counters (classification, scans)
-  int64_t* blk_b = nullptr;
   bool csr_borrowed = false;  // init: row_ptr, col and w are the caller's device arrays
   // init from host memory: the weights are still on their way (sstream, ev_join) while the structure is worked on
   bool w_pending = false, w_late = false;
@@ -294,7 +289,6 @@ struct Handle {
   uint32_t* scan_ctr = nullptr;        // single-pass scan: tile ticket, blocks finished
   int64_t* scan_sums = nullptr;        // two-launch scan: [kScanSums] tile sums
   int64_t scan_tiles_cap = 0;
-  uint32_t* radix_dtot = nullptr;      // 256
   // records in (lca, rank) order
   int32_t* rec_u = nullptr;
   int32_t* rec_v = nullptr;
@@ -361,16 +355,6 @@ struct Handle {
 };
 
 // ------------------------------------------------------------------ helpers
-
-__device__ __forceinline__ int64_t row_of(const int64_t* __restrict__ row_ptr, int64_t n, int64_t p) {
-  // largest u with row_ptr[u] <= p
-  int64_t lo = 0, hi = n;  // row_ptr[lo] <= p < row_ptr[hi] (row_ptr[n] = nnz > p)
-  while (hi - lo > 1) {
-    int64_t mid = (lo + hi) >> 1;
-    if (__ldg(row_ptr + mid) <= p) lo = mid; else hi = mid;
-  }
-  return lo;
-}
 
 // one aligned 32-byte sector in one load (two 16-byte loads of it are two requests, and the second misses L1
 // while the first is in flight).  Volatile and clobbering memory: it stays behind dep_sync() and barriers, in order with
@@ -573,7 +557,6 @@ constexpr int kScanSums = 4096;
 int ensure_scan_status(Handle& h, int64_t n_max);  // scans of up to n_max elements can run
 int scan_excl_i64(Handle& h, const int64_t* in, int64_t* out, int64_t n_host, const int64_t* n_dev, int64_t n_max);
 int scan_excl_i32(Handle& h, const int32_t* in, int64_t* out, int64_t n_host, const int64_t* n_dev, int64_t n_max);
-int scan_excl_u32(Handle& h, const uint32_t* in, int64_t* out, const int64_t* n_dev, int64_t n_max);
 int scan_excl_u8(Handle& h, const uint8_t* in, int64_t* out, const int64_t* n_dev, int64_t n_max);
 
 // steps

@@ -204,10 +204,6 @@ int scan_excl_i32(Handle& h, const int32_t* in, int64_t* out, int64_t n_host, co
   return scan_impl<int32_t>(h, in, out, n_host, n_dev, n_max);
 }
 
-int scan_excl_u32(Handle& h, const uint32_t* in, int64_t* out, const int64_t* n_dev, int64_t n_max) {
-  return scan_impl<uint32_t>(h, in, out, 0, n_dev, n_max);
-}
-
 int scan_excl_u8(Handle& h, const uint8_t* in, int64_t* out, const int64_t* n_dev, int64_t n_max) {
   return scan_impl<uint8_t>(h, in, out, 0, n_dev, n_max);
 }
