@@ -74,8 +74,9 @@ typedef struct pdg_options {
   int32_t block_tier_max;   /* subtasks with warp_tier_max+1..block_tier_max candidates get one block each
                                (shared-memory marker table); 0 turns the block tier off; at most 896 */
   int32_t sort_tile_keys;   /* keys per tile of the radix-sort scatter: 2048, 3072 or 4096 (0: 3072) */
-  int32_t sort_one_launch;  /* 1 (default): the ordering step runs as one cooperative launch whenever every
-                               tile of the candidates fits in one resident block; 0: one kernel per pass */
+  int32_t sort_one_launch;  /* 1 (default): up to 65,536 candidates of one graph are ordered by tiles ranked against
+                               each other, more by one cooperative launch whenever every tile of them fits in one
+                               resident block; 0: one kernel per radix pass */
 } pdg_options;
 
 typedef struct pdg_sparsifier* pdg_handle; /* opaque, owned by the library */
@@ -103,8 +104,9 @@ const char* pdg_status_string(int status);
  *   stream   cudaStream_t on which all device work of the handle runs
  *            (NULL = the legacy default stream).
  *
- * The library copies the inputs into device memory it owns; the caller may
- * free its buffers when this returns.  On success *out receives a handle to
+ * The library keeps none of the inputs: device arrays are read in place or
+ * copied, host arrays copied, and the caller may free or change its buffers
+ * when this returns (not before: other threads included).  On success *out receives a handle to
  * release with sparsifier_free.  On failure *out is NULL and a negative
  * status is returned (PDG_E_NOT_CSR, PDG_E_NOT_SYMMETRIC, PDG_E_NOT_A_TREE,
  * PDG_E_BAD_WEIGHT, PDG_E_RANGE, PDG_E_OOM, PDG_E_CUDA, PDG_E_INVALID_ARG).

@@ -98,7 +98,7 @@ struct DevScalars {
   int32_t bounds_site;  // first failed bounds check (see ERR_BOUNDS)
   int32_t bounds_where;  // its round (99: serial finisher)
   int64_t bounds_pos, bounds_val;  // its position and offending value
-  unsigned long long join_conf;   // join: (marker, candidate) pairs found
+  unsigned long long join_conf;   // join: (marker, candidate) pairs in the list of the long ones
   int64_t finish_left;  // cooperative tier: candidates the rounds left to the serial finisher
 };
 

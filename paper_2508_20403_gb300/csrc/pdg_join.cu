@@ -44,8 +44,9 @@
 // that all warps add to.
 // Measured on one GB300, mesh 128^3, alpha .10, c = 2 (314,617 candidates):
 // 34 + 42 + 10 us, where the tiers' grouping by LCA, registrations, probes and
-// rounds took 340 us (steps A5 + A6 0.298 ms and three sort passes); a packed
-// batch of 192 graphs (1.43 M candidates) 125 + 325 + 76 us against 1,157 us.
+// rounds took 340 us (steps A5 + A6 0.298 ms and three sort passes).  A packed
+// batch of 192 graphs, 1.43 M candidates: 125 + 325 + 76 us against 1,157; with
+// the 784,789 candidates that its first prefixes hold, 65 + 168 + 41.
 // When the tiers are the better ones: cells of thousands of members, whose
 // pairs grow with the square (kJoinCellMax, kJoinPairsPer).
 #include <algorithm>

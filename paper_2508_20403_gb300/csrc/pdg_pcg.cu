@@ -509,7 +509,7 @@ __global__ void k_pc_capacitance(const uint64_t* __restrict__ table, const doubl
 // C_ij -= C_ip R_j^T, products with inv(C) were 10 to 60 times further off, and the preconditioner's residual, 10^-3
 // where off-tree edges outweigh the tree 10^6 times, was of order 1.)
 // Bound by FP64 (k^3 / 2 multiply-adds at two a clock and SM) and the chain of k pivots (0.7 us each, mostly the
-// reciprocal): k = 500 takes 0.55 ms; pivot by pivot over the whole matrix it was two launches a pivot, 4.4 ms of
+// reciprocal): k = 500 takes 0.56 ms; pivot by pivot over the whole matrix it was two launches a pivot, 4.4 ms of
 // kernels and as much between them.
 constexpr int kSw = 32;
 

@@ -30,14 +30,16 @@ from . import workloads as W
 
 
 def device_bytes_estimate(g) -> int:
-    """Upper estimate of the device memory one graph needs inside a batch
-    handle (resident CSR and tree, per-edge work arrays, candidate buffers).
-    Calibrated from pdg_handle_info on meshes and random geometric graphs."""
+    """Estimate of the device memory one graph needs inside a batch handle
+    (CSR and tree as they come, per-edge work arrays, candidate buffers).
+    pdg_handle_info counts 0.5 to 1.1 times as much after a recovery at
+    alpha .02 and up to 1.5 times at .10 (grids, meshes, triangulations,
+    geometric graphs)."""
     n, m = g.n, g.m
     e_off = max(m - n + 1, 0)
     return int(8 * n + 24 * m + 4 * n  # CSR + parent
-               + 8 * n + 16 * n + 12 * n + 2 * 28 * n  # r, P, Euler tour + labels, range-minimum levels (x2 margin)
-               + 36 * e_off  # off-tree SoA, keys, LCAs
+               + 8 * n + 16 * n + 12 * n + 2 * 28 * n  # r, P, Euler tour + labels, records, range minima
+               + 36 * e_off  # keys, LCAs, the selection's list
                + 400 * max(int(0.2 * n), 1024)  # candidate buffers and tables
                + (1 << 20))
 
