@@ -176,17 +176,17 @@ __device__ __forceinline__ void for_rows(const int64_t* __restrict__ ptr, int64_
   __shared__ int32_t s_long[kBlock];
   __shared__ int s_n;
   for (int64_t v0 = (int64_t)blockIdx.x * kBlock; v0 < n; v0 += (int64_t)gridDim.x * kBlock) {  // block-uniform
+    const int64_t v = v0 + threadIdx.x;
+    const int64_t b = v < n ? ptr[v] : 0, e = v < n ? ptr[v + 1] : 0;
+    const bool is_long = e - b > kRowShort;
+    const bool any = __syncthreads_or(is_long);  // (and the rows listed before are done)
+    if (v < n && !is_long) row(v, b, e);
+    if (!any) continue;
     if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
-    const int64_t v = v0 + threadIdx.x;
-    if (v < n) {
-      const int64_t b = ptr[v], e = ptr[v + 1];
-      if (e - b <= kRowShort) row(v, b, e);
-      else s_long[atomicAdd(&s_n, 1)] = (int32_t)v;
-    }
+    if (is_long) s_long[atomicAdd(&s_n, 1)] = (int32_t)v;
     __syncthreads();
     for (int i = 0; i < s_n; i++) long_row((int64_t)s_long[i], ptr[s_long[i]], ptr[s_long[i] + 1]);
-    __syncthreads();
   }
 }
 
