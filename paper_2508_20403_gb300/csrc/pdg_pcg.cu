@@ -514,15 +514,15 @@ __global__ void k_pc_capacitance(const uint64_t* __restrict__ table, const doubl
 constexpr int kSw = 32;
 
 // The factors of C_pp (every block for itself: 32 rows in the registers of eight warps, the scaled pivot rows, which are
-// the columns of M, through shared memory), then Y and R of this block's eight rows.  A row of the pivot block takes its
+// the columns of M, through shared memory), then Y, S = Y D^-1 and R of this block's eight rows.  A row of the pivot block takes its
 // row of the identity along instead, and its R is its row of inv(C_pp).
 __global__ void __launch_bounds__(256) k_pc_sweep_panel(const double* __restrict__ C, int k, int p0,
-                                                        double* __restrict__ D, double* __restrict__ R,
+                                                        double* __restrict__ S, double* __restrict__ R,
                                                         double* __restrict__ Y) {
   __shared__ double b[kSw][kSw + 1];  // b[p][j] = M[j][p], j > p
   __shared__ double s_d[kSw];         // D^-1
   const int nb = min(kSw, k - p0), lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int row = blockIdx.x * 8 + w;  // of Y and R
+  const int row = blockIdx.x * 8 + w;  // of Y, S and R
   double x = 0.0;
   if (row >= p0 && row < p0 + nb) x = row - p0 == lane ? 1.0 : 0.0;
   else if (row < k && lane < nb) x = row > p0 ? C[(int64_t)row * k + p0 + lane] : C[(int64_t)(p0 + lane) * k + row];
@@ -561,10 +561,10 @@ __global__ void __launch_bounds__(256) k_pc_sweep_panel(const double* __restrict
       x = update(x);
       __syncthreads();
     }
-  if (blockIdx.x == 0 && w == 0) D[lane] = s_d[lane];
   if (row >= k) return;  // (warp-uniform)
   Y[(int64_t)row * kSw + lane] = x;
   double t = x * s_d[lane];
+  S[(int64_t)row * kSw + lane] = t;
 #pragma unroll
   for (int p = kSw - 1; p > 0; p--) {
     const double f = __shfl_sync(0xffffffffu, t, p);
@@ -583,7 +583,7 @@ __device__ __forceinline__ int2 lower_tile(uint32_t t) {
 }
 
 __global__ void __launch_bounds__(256) k_pc_sweep_update(double* __restrict__ C, int k, int p0,
-                                                         const double* __restrict__ D, const double* __restrict__ R,
+                                                         const double* __restrict__ S, const double* __restrict__ R,
                                                          const double* __restrict__ Y) {
   __shared__ double l[kSw][kSw + 1], r[kSw][kSw + 1];  // by row of C
   const int2 tile = lower_tile(blockIdx.x);
@@ -591,8 +591,8 @@ __global__ void __launch_bounds__(256) k_pc_sweep_update(double* __restrict__ C,
   const bool pi = i0 == p0, pj = j0 == p0;
   for (int q = tid; q < kSw * kSw; q += 256) {
     const int i = q / kSw, t = q % kSw;
-    l[i][t] = i0 + i >= k ? 0.0 : pj ? R[(int64_t)(i0 + i) * kSw + t] : Y[(int64_t)(i0 + i) * kSw + t] * D[t];
-    r[i][t] = j0 + i >= k ? 0.0 : pi ? R[(int64_t)(j0 + i) * kSw + t] : Y[(int64_t)(j0 + i) * kSw + t];
+    l[i][t] = i0 + i >= k ? 0.0 : (pj ? R : S)[(int64_t)(i0 + i) * kSw + t];
+    r[i][t] = j0 + i >= k ? 0.0 : (pi ? R : Y)[(int64_t)(j0 + i) * kSw + t];
   }
   __syncthreads();
   const int ti = tid / 16, tj = tid % 16;  // rows ti, ti + 16, columns tj, tj + 16
@@ -786,7 +786,7 @@ int pcg_quality(Handle& h, const int32_t* ids, int64_t k, const double* b, doubl
   int32_t *ea = nullptr, *eb = nullptr, *seen = nullptr, *flags = nullptr, *icnt = nullptr, *iedge = nullptr;
   int64_t *tptr = nullptr, *iptr = nullptr;
   double *wup = nullptr, *E = nullptr, *D = nullptr, *sums = nullptr, *ewk = nullptr;
-  double *C = nullptr, *swR = nullptr, *swY = nullptr, *swD = nullptr, *dw = nullptr, *bb = nullptr, *x = nullptr;
+  double *C = nullptr, *swR = nullptr, *swY = nullptr, *swS = nullptr, *dw = nullptr, *bb = nullptr, *x = nullptr;
   double *r = nullptr, *z = nullptr, *p = nullptr, *Ap = nullptr, *t = nullptr;
   double *qv = nullptr, *parts = nullptr;
   double2* dist = nullptr;
@@ -800,7 +800,7 @@ int pcg_quality(Handle& h, const int32_t* ids, int64_t k, const double* b, doubl
   place(&arc_uv, m); place(&succ, A); place(&tin, n); place(&tout, n); place(&wup, n); place(&tour, A); place(&E, A);
   place(&sums, T); place(&dist, A); place(&D, A); place(&depth, A); place(&dsums, T); place(&ea, k); place(&eb, k);
   place(&ewk, k); place(&seen, m); place(&flags, 4); place(&icnt, n); place(&iptr, n + 1); place(&iedge, 2 * k);
-  place(&C, k * k); place(&swR, kSw * k); place(&swY, kSw * k); place(&swD, kSw); place(&ekey, 2 * k);
+  place(&C, k * k); place(&swR, kSw * k); place(&swY, kSw * k); place(&swS, kSw * k); place(&ekey, 2 * k);
   place(&epos, 2 * k); place(&erank, 2 * k); place(&gaps, 2 * k * gap_rows); place(&dw, n); place(&bb, n);
   place(&x, n); place(&r, n); place(&z, n); place(&p, n); place(&Ap, n); place(&t, n);
   place(&qv, k); place(&parts, 4 * kDotBlocks + std::max<int64_t>(kDotBlocks, T));
@@ -898,8 +898,8 @@ int pcg_quality(Handle& h, const int32_t* ids, int64_t k, const double* b, doubl
     k_pc_capacitance<<<grid_for(h, k * k), kBlock, 0, s>>>(gaps, dist, depth, epos, erank, ewk, (int)k, C);
     const int blocks = (int)((k + kSw - 1) / kSw);
     for (int p0 = 0; p0 < k; p0 += kSw) {
-      k_pc_sweep_panel<<<(int)((k + 7) / 8), 256, 0, s>>>(C, (int)k, p0, swD, swR, swY);
-      k_pc_sweep_update<<<blocks * (blocks + 1) / 2, 256, 0, s>>>(C, (int)k, p0, swD, swR, swY);
+      k_pc_sweep_panel<<<(int)((k + 7) / 8), 256, 0, s>>>(C, (int)k, p0, swS, swR, swY);
+      k_pc_sweep_update<<<blocks * (blocks + 1) / 2, 256, 0, s>>>(C, (int)k, p0, swS, swR, swY);
     }
     k_pc_sweep_end<<<blocks * (blocks + 1) / 2, 256, 0, s>>>(C, (int)k);
     // incidence lists of the recovered edges, in edge order
